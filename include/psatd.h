@@ -216,7 +216,7 @@ psatd_status psatd_coeffs_init(psatd_plan plan);
  *   elements per thread; radix 16 only for the mixed precisions; for 3 * 2^k
  *   lengths only 12 elements per thread: a radix-12 first stage, then radix
  *   2 and 4) with its lines per CTA and component groups (below).
- * Results do not depend on the choice (same arithmetic, same order per line).
+ * Results depend on the radix schedule alone (same arithmetic, same order per line).
  * `report` (may be NULL) receives a one-line summary of the times, the chosen
  * ones marked '*', truncated to report_len - 1 bytes.  Synchronous.
  * Errors: INVALID_ARG (NULL plan, tables not initialised, reps out of range),
@@ -227,8 +227,10 @@ psatd_status psatd_plan_autotune(psatd_plan plan, int32_t reps, char* report, si
  *   cfg[0..3] log2(lines per CTA) of the x forward, y forward (3D), y inverse
  *             (3D) and x inverse passes (-1 / unused: 2D y passes);
  *   cfg[4]    lines per CTA of the fused pass;
- *   cfg[5]    its elements per thread: 8 (radix-8 stages), 16 (radix-16) or,
- *             for a last axis of 3 * 2^k points, 12 (radix 12, then 2/4).
+ *   cfg[5]    its elements per thread: 8 (radix-8 stages), 16 (radix-16; the
+ *             built-in choice of FP32 lines of 1024 points and more and of the mixed
+ *             precisions) or, for a last axis of 3 * 2^k points, 12 (radix 12, then
+ *             2/4), of 5 * 2^k points 20 (radix 10 or 20, then 4).
  * psatd_plan_get_launch reports the shapes the next step will use.
  * psatd_plan_set_launch sets them (-1 entries: the built-in choice) after
  * checking each against the shapes the autotuner would consider
@@ -239,19 +241,18 @@ psatd_status psatd_plan_get_launch(psatd_plan plan, int32_t cfg[6]);
 
 /* Component groups of the fused pass (a launch shape, like cfg[4]): with G > 1
  * each line gets G thread groups that forward- and inverse-transform its
- * components in turn (group j: components j, j + G, ...; their own exchange
- * buffer and barrier each), meeting for the per-mode push; shared memory per
- * line grows from (n_in + 1) to (n_in + G) line buffers.  G = 1 is the plain
+ * components in turn (FP32: pairs of components; group j: units j, j + G, ...),
+ * meeting for the per-mode push.  G = 1 is the plain
  * pass.  Tensor-core plans (PSATD_MIXED_*): 2 only, two 128-row groups that
  * transform component pairs in lockstep and share every tensor-core round
  * (measured slower than one group on GB300; kept as a launch shape).
- * Valid otherwise: 1 always; 2 or 4 for PSATD_FP32 plans whose fused-axis lines
+ * set accepts otherwise: 1 always; 2 or 4 for PSATD_FP32 plans whose fused-axis lines
  * have a multiple of 32 threads (length / elements per thread), at most 512
- * threads and 15 groups per CTA, an even number of modes per thread, and the
- * shared memory within the device's limit.  -1: the built-in choice, 2 where
- * lines have at least 64 threads and the one-group pass keeps fewer than 12
- * warps per SM resident (shared memory: many components on long lines, e.g.
- * 1024-point 3D rho-form lines), else 1.  Results
+ * threads and 15 groups per CTA, an even number of modes per thread, and (n_in + G)
+ * line buffers within the device's shared memory.  -1: the built-in choice, in FP32
+ * the fewest of 1, 2 and 4 groups that fill the SMs' registers with warps (long lines
+ * of many components, launches of few lines; it also takes blocks of several short
+ * lines in groups), else 1.  Results
  * are bitwise the same for every G (each transform and each mode's update
  * runs the same arithmetic).  set: INVALID_ARG when the shape is not valid
  * for the plan's current lines per CTA and elements per thread (a later
@@ -317,7 +318,7 @@ psatd_status fdtd_step(const psatd_desc* desc, int32_t scheme, const psatd_field
  * sum_{j<i} n[2j] n[2j+1]).
  * Patches of equal size form a class (own spectra and tables).  A step runs
  * the persistent passes below where the sizes allow; else one launch per pass
- * and class, forked from the batch's stream into up to four internal streams
+ * and class, forked from the batch's stream into up to four (FP32: two) internal streams
  * that run the classes side by side, and joined back.  A call with nsteps > 1 on a
  * non-default stream records one step of all classes into a CUDA graph
  * (re-recorded when the field/source pointers change) and replays it nsteps

@@ -317,11 +317,40 @@ int pick_log_tb(int L, int64_t nb, bool f32, bool tc = false, bool rows = false)
 // before the cap above (the autotuner measured that faster at 2048^2 x, 1024^2 x,
 // 256^3 x and y: the gathered bin pairs of fewer lines per CTA), keeping the
 // tensor-core minimum
-int pick_log_tb_inv(int L, int64_t nb, bool f32, bool tc = false) {
+int pick_log_tb_inv_raw(int L, int64_t nb, bool f32, bool tc) {
   const int lg = pick_log_tb_raw(L, nb, f32, tc);
   const int T = L / row_ept(L);
   if (lg == 0 || (tc && (T << (lg - 1)) < 128)) return lg;
   return lg - 1;
+}
+constexpr int kSMs = 152;  // GB300
+// Rows per CTA of a row-pair pass (FP32 without tensor cores; pair_rows.cuh) over `nb`
+// rows of each of `planes` planes and components.  Forward: at most 16 rows and 256
+// threads (T rows-pairs' threads), 8 rows where a line is whole warps; inverse: half the
+// threads (2048^2 x inverse: 4 / 8 rows 33.1 / 34.6 us; 256^3 y inverse: 16 / 8 rows
+// 124 / 137 us).  Fewer while the launch has under two CTAs per SM: there a pass lasts as
+// long as one CTA, and rows on idle SMs cost nothing.
+int pick_log_tb_pairs(int L, int64_t nb, int64_t planes, bool fwd, bool rows) {
+  const int T = L / row_ept(L);
+  const int maxthr = fwd ? row_maxthr(L, true) : std::min(row_maxthr(L, true), 256);
+  const int cap = T <= 4 ? 32 : (fwd && rows && T % 32 == 0) ? 8 : 16;
+  int lg = 0;
+  while ((T << (lg + 1)) <= maxthr && (2 << lg) <= cap && nb % (2 << lg) == 0) ++lg;
+  while (lg > 1 && (nb >> lg) * planes < 2 * kSMs) --lg;
+  return lg;
+}
+// lines per CTA of the transposing passes of plan p: 0 x forward, 1 y forward, 2 y
+// inverse, 3 x inverse (the configured value, else the rules above)
+int rows_per_cta(psatd_plan p, int k) {
+  if (p->cfg_log_tb[k] >= 0) return p->cfg_log_tb[k];
+  const bool x = k == 0 || k == 3, fwd = k < 2;
+  const int L = (int)(x ? p->nx / 2 : p->ny);
+  const int64_t nb = x ? p->ny : p->nz;
+  if (p->f32 && !p->tc) {
+    const int64_t planes = (p->ndim == 3 ? (x ? p->nz : p->nxh) : p->npatch) * (fwd ? p->n_in : p->n_out);
+    return pick_log_tb_pairs(L, nb, planes, fwd, x);
+  }
+  return fwd ? pick_log_tb(L, nb, p->f32, p->tc, x) : pick_log_tb_inv_raw(L, nb, p->f32, p->tc);
 }
 
 // shared memory of a transposing pass: one L-element buffer per line, or the
@@ -335,16 +364,17 @@ size_t tpass_smem(int L, int log_tb, size_t nk, size_t csz) {
 // lines per CTA of the fused last-axis pass: as few as make a whole warp (the
 // autotuner found one line per CTA fastest at 256^3, 512^2 and 2048^2: the lines
 // of a CTA only add barriers to each other); the tensor-core variant needs a
-// multiple of 128 threads
-int push_lines_per_cta(int L, int n_in, int64_t nlines, bool tc, bool f32, int ept) {
-  (void)n_in;
-  (void)nlines;
-  (void)f32;
+// multiple of 128 threads.  In FP32, one-warp lines run two to a CTA where the
+// launch then still has four CTAs per SM (256-point lines, eleven components:
+// 0.417 -> 0.390 ms, with two groups 0.382 -> 0.365: the two warps share the
+// instruction stream).
+int push_lines_per_cta(int L, int64_t nlines, bool tc, bool f32, int ept) {
   const int T = L / ept;
   int tb = 1;
   while (tb * T < 32) tb *= 2;
   if (tc)
     while (tb * T < 128) tb *= 2;
+  if (f32 && !tc && T == 32 && nlines >= 8 * kSMs) tb = 2;
   return tb;
 }
 
@@ -370,29 +400,48 @@ bool push_groups_ok(int L, int ept, int tb, int G, bool tc, bool f32) {
 size_t push_smem(int n_in, int L, int tb, int G, size_t csz, bool tc = false) {
   return (size_t)tb * ((size_t)n_in + (size_t)(tc ? 1 : G)) * (size_t)L * csz;
 }
-// The built-in choice (measured on GB300 against the plain pass): two groups
-// where lines have at least 64 threads and the plain pass keeps fewer than 12
-// warps per SM resident for lack of shared memory (3D rho-form and 2D
-// six-component J-form lines of 1024 points: 8 warps, 12 % faster with two
-// groups); one group otherwise (the 2048^2 TE grid, 256^3, the 512-patch
-// batch ran fastest with one).  sm_bytes: shared memory per SM.
-int push_groups_default(int L, int ept, int tb, int n_in, bool tc, bool f32, size_t csz, int maxsm, int sm_bytes) {
+// transform units (pairs and single components) of the FP32 fused pass (pair_push.cuh)
+int push_units_of(int layout, int n_in) {
+  return layout == PSATD_FIELDS_2D_TM ? n_in - 1 : (layout == PSATD_FIELDS_2D_TE ? n_in + 1 : n_in == 6 ? 6 : n_in + 1) / 2;
+}
+// The built-in choice (FP32 without tensor cores; one group elsewhere): the fewest
+// groups (1, 2 or 4, no more than needed for one per unit) that give an SM 14 resident warps (of the 16 that the
+// registers allow) and the launch 256 threads per SM.  Measured with 1 / 2 / 4 groups:
+// 2048-point lines of five components 85.2 / 73.1 / 87.8 us; 1024 points, eleven
+// components 1.350 / 1.026 / 0.884 ms; 512 points, eleven components 0.421 / 0.383 /
+// 0.486 ms; 257 lines of 512 points 12.2 / 11.6 / 11.2 us.  Groups are whole warps.
+int push_groups_default(int layout, int L, int ept, int tb, int n_in, int64_t nlines, bool tc, bool f32, int sm_bytes) {
   if (tc || !f32 || L < ept || sm_bytes <= 0) return 1;
-  const int T = L / ept;
-  if (T < 64) return 1;
-  const size_t smem1 = push_smem(n_in, L, tb, 1, csz) + 1024;  // + the per-CTA reservation
-  int ctas = (int)((size_t)sm_bytes / smem1);
-  ctas = std::min(ctas, std::min(2048 / (T * tb), 32));
-  if (ctas * T * tb / 32 >= 12) return 1;
-  if (push_groups_ok(L, ept, tb, 2, tc, f32) && (maxsm <= 0 || push_smem(n_in, L, tb, 2, csz) <= (size_t)maxsm))
-    return 2;
-  return 1;
+  const int T = L / ept, thr = T * tb;
+  if (thr % 32) return 1;
+  const int ctas = std::max(1, (int)((size_t)sm_bytes / ((size_t)n_in * tb * L * 8 + 1024)));  // + the reservation
+  const int units = push_units_of(layout, n_in);
+  int G = 1;
+  while (G < 4 && G < units && thr * G * 2 <= 512 &&
+         (std::min(ctas * thr * G, 512) < 14 * 32 || nlines * T * G < 256 * kSMs))
+    G *= 2;
+  return G;
 }
 
 // split-BF16 passes: shared memory of the third A piece of `threads` threads
 // (one 128-row piece per 128 threads), after the pass's exchange region
 size_t tc_a3_bytes(psatd_plan p, int threads) {
   return p->tc_bf16 ? (size_t)(threads / 128) * TcGeom<16>::kAPiece : 0;
+}
+
+// lines along the fused axis, and the fused pass's lines per CTA and component groups of
+// the plan's next step (the configured values, else the rules above)
+int64_t push_nlines(psatd_plan p) { return p->ndim == 3 ? p->nxh * p->ny : p->nxh * p->npatch; }
+int push_line_len(psatd_plan p) { return (int)(p->ndim == 3 ? p->nz : p->ny); }
+int push_tb(psatd_plan p) {
+  return p->cfg_push_tb > 0 ? p->cfg_push_tb
+                            : push_lines_per_cta(push_line_len(p), push_nlines(p), p->tc, p->f32, p->push_ept);
+}
+int push_groups(psatd_plan p) {
+  const int L = push_line_len(p), tb = push_tb(p);
+  if (p->cfg_push_groups <= 0)
+    return push_groups_default(p->layout, L, p->push_ept, tb, p->n_in, push_nlines(p), p->tc, p->f32, p->sm_bytes);
+  return push_groups_ok(L, p->push_ept, tb, p->cfg_push_groups, p->tc, p->f32) ? p->cfg_push_groups : 1;
 }
 
 // Event pair around one launch on the plan's stream.  While the stream is being
@@ -502,6 +551,21 @@ PushArgs<R> make_push_args(psatd_plan p, void* sp, int Lline, int64_t nlines) {
   return a;
 }
 
+// Launch of the fused pass by elements per thread; LS: the layout set (launch.h).
+template <typename R, int TC, int LS>
+cudaError_t launch_push(psatd_plan p, int L, dim3 grid, int tb, int G, size_t smem, const PushArgs<R>& a,
+                        const void* tw) {
+  if constexpr (std::is_same<R, float>::value && TC == 0) {
+    if (p->push_ept == 12) return launch_line_push3<R, LS>(L, p->layout, grid, tb, G, smem, p->st, a, tw);
+    if (p->push_ept == 20) return launch_line_push5<R, LS>(L, p->layout, grid, tb, G, smem, p->st, a, tw);
+  }
+  if (p->push_ept == 16) return launch_line_push<R, TC, 16, LS>(L, p->layout, grid, tb, G, smem, p->st, a, tw);
+  if constexpr (TC == 0) {
+    if (p->push_ept == 8) return launch_line_push<R, TC, 8, LS>(L, p->layout, grid, tb, G, smem, p->st, a, tw);
+  }
+  return cudaErrorInvalidValue;
+}
+
 template <typename R, int TC>
 psatd_status run_step(psatd_plan p, const void* in[kMaxComp], void* out[kMaxComp]) {
   typedef typename Types<R>::C C;
@@ -530,7 +594,7 @@ psatd_status run_step(psatd_plan p, const void* in[kMaxComp], void* out[kMaxComp
   // pass 1: x rows (R2C), b = y -> spec1 [c][kx][z][y] (3D) / [c][patch][kx][y] (2D)
   {
     PassGeom g;
-    g.log_tb = p->cfg_log_tb[0] >= 0 ? p->cfg_log_tb[0] : pick_log_tb(Lx, ny, p->f32, TC, true);
+    g.log_tb = rows_per_cta(p, 0);
     g.grid = dim3((unsigned)(ny >> g.log_tb), (unsigned)na0, (unsigned)p->n_in);
     g.smem = tail + tpass_smem(Lx, g.log_tb, 0, csz) + tc_a3_bytes(p, (Lx / row_ept(Lx)) << g.log_tb);
     for (int c = 0; c < p->n_in; ++c) {
@@ -550,7 +614,7 @@ psatd_status run_step(psatd_plan p, const void* in[kMaxComp], void* out[kMaxComp
   if (p->ndim == 3) {
     // pass 2: y lines (C2C), b = z, a0 = kx: spec1 [c][kx][z][y] -> spec2 [c][kx][ky][z]
     PassGeom g;
-    g.log_tb = p->cfg_log_tb[1] >= 0 ? p->cfg_log_tb[1] : pick_log_tb((int)ny, nz, p->f32, TC);
+    g.log_tb = rows_per_cta(p, 1);
     g.grid = dim3((unsigned)(nz >> g.log_tb), (unsigned)nxh, (unsigned)p->n_in);
     g.smem = tail + tpass_smem((int)ny, g.log_tb, (size_t)ny, csz) +
              tc_a3_bytes(p, ((int)ny / row_ept((int)ny)) << g.log_tb);
@@ -572,34 +636,19 @@ psatd_status run_step(psatd_plan p, const void* in[kMaxComp], void* out[kMaxComp
     PushArgs<R> a = make_push_args<R>(p, sp, Lline, nlines);
     const void* twl = p->tw[p->ndim == 3 ? 2 : 1];
     {
-      const int tb = p->cfg_push_tb > 0 ? p->cfg_push_tb
-                                        : push_lines_per_cta(Lline, p->n_in, nlines, TC, p->f32, p->push_ept);
-      int G = p->cfg_push_groups > 0
-                  ? p->cfg_push_groups
-                  : push_groups_default(Lline, p->push_ept, tb, p->n_in, TC, p->f32, csz, p->maxsm, p->sm_bytes);
-      if (!push_groups_ok(Lline, p->push_ept, tb, G, TC, p->f32)) G = 1;
+      const int tb = push_tb(p), G = push_groups(p);
       const size_t smem = tail + push_smem(p->n_in, Lline, tb, G, csz, TC);
       const dim3 grid((unsigned)((nlines + tb - 1) / tb));
       TimedLaunch tl(p, K_PUSH);
-      if (p->push_ept == 12 || p->push_ept == 20) {
-        if constexpr (std::is_same<R, float>::value && TC == 0)
-          e = p->push_ept == 12 ? launch_line_push3<R>(Lline, p->layout, grid, tb, G, smem, p->st, a, twl)
-                                : launch_line_push5<R>(Lline, p->layout, grid, tb, G, smem, p->st, a, twl);
-        else
-          e = cudaErrorInvalidValue;
-      } else if (p->push_ept == 16) {
-        e = launch_line_push<R, TC, 16>(Lline, p->layout, grid, tb, G, smem, p->st, a, twl);
-      } else {
-        if constexpr (TC) e = cudaErrorInvalidValue;
-        else e = launch_line_push<R, false, 8>(Lline, p->layout, grid, tb, G, smem, p->st, a, twl);
-      }
+      e = p->layout < 2 ? launch_push<R, TC, 0>(p, Lline, grid, tb, G, smem, a, twl)
+                        : launch_push<R, TC, 1>(p, Lline, grid, tb, G, smem, a, twl);
       if (e != cudaSuccess) return cuda_fail(p, e, "line_fft_push launch");
     }
   }
   if (p->ndim == 3) {
     // pass 4: inverse y lines: spec2 [c][kx][ky][z] -> spec1 [c][kx][z][y]
     PassGeom g;
-    g.log_tb = p->cfg_log_tb[2] >= 0 ? p->cfg_log_tb[2] : pick_log_tb_inv((int)ny, nz, p->f32, TC);
+    g.log_tb = rows_per_cta(p, 2);
     g.grid = dim3((unsigned)(nz >> g.log_tb), (unsigned)nxh, (unsigned)p->n_out);
     g.smem = tail + tpass_smem((int)ny, g.log_tb, (size_t)ny, csz) +
              tc_a3_bytes(p, ((int)ny / row_ept((int)ny)) << g.log_tb);
@@ -616,7 +665,7 @@ psatd_status run_step(psatd_plan p, const void* in[kMaxComp], void* out[kMaxComp
   // last pass: inverse x rows (C2R): spec1 -> out [z][y][x] (3D) / packed patches (2D)
   {
     PassGeom g;
-    g.log_tb = p->cfg_log_tb[3] >= 0 ? p->cfg_log_tb[3] : pick_log_tb_inv(Lx, ny, p->f32, TC);
+    g.log_tb = rows_per_cta(p, 3);
     g.grid = dim3((unsigned)(ny >> g.log_tb), (unsigned)na0, (unsigned)p->n_out);
     g.smem = tail + tpass_smem(Lx, g.log_tb, 0, csz) + tc_a3_bytes(p, (Lx / row_ept(Lx)) << g.log_tb);
     for (int c = 0; c < p->n_out; ++c) {
@@ -661,7 +710,7 @@ psatd_status check_tc_shape(psatd_plan p, int maxsm) {
                   rows[i].L, (long long)rows[i].nb);
   }
   const int64_t nlines = p->ndim == 3 ? p->nxh * p->ny : p->nxh * p->npatch;
-  const int tb = push_lines_per_cta(Ll, p->n_in, nlines, true, true, 16);
+  const int tb = push_lines_per_cta(Ll, nlines, true, true, 16);
   const size_t smem = (size_t)kTcTail + push_smem(p->n_in, Ll, tb, 1, 8);
   if (maxsm > 0 && smem > (size_t)maxsm)
     return fail(nullptr, PSATD_ERR_UNSUPPORTED, "mixed precision: last-axis length %d needs %zu bytes of shared memory",
@@ -755,7 +804,7 @@ TuneSpace tune_space(psatd_plan p) {
   }
   for (int ept : {8, 16, 12, 20}) {
     // powers of two: radix-8 or radix-16 stages (tensor cores: 16); 3 * 2^k: 12; 5 * 2^k: 20
-    const bool allowed = pow2(ts.Ll) ? (ept == 8 || ept == 16) && (!p->tc || ept == 16) : ept == push_ept(ts.Ll);
+    const bool allowed = pow2(ts.Ll) ? (ept == 8 || ept == 16) && (!p->tc || ept == 16) : ept == push_ept(ts.Ll, p->tc, p->f32);
     if (!allowed || ts.Ll < ept) continue;
     const int T = ts.Ll / ept;
     for (int tb = 1; tb * T <= (T > 256 ? T : 256); tb *= 2) {
@@ -932,7 +981,7 @@ static psatd_status plan_create_n(const psatd_desc* desc, void* cuda_stream, int
   p->f32 = desc->prec != PSATD_FP64;
   p->tc = desc->prec == PSATD_MIXED_FP16 || desc->prec == PSATD_MIXED_BF16;
   p->tc_bf16 = desc->prec == PSATD_MIXED_BF16;
-  p->push_ept = push_ept((int)(desc->ndim == 3 ? desc->n[2] : desc->n[1]), p->tc);
+  p->push_ept = push_ept((int)(desc->ndim == 3 ? desc->n[2] : desc->n[1]), p->tc, p->f32);
   p->order = desc->order;
   p->ndim = desc->ndim;
   p->layout = desc->layout;
@@ -1093,7 +1142,7 @@ psatd_status psatd_plan_set_launch(psatd_plan p, const int32_t cfg[6]) {
   if (!p || !cfg) return fail(p, PSATD_ERR_INVALID_ARG, "plan or cfg is NULL");
   if (!p->coeffs_ready) return fail(p, PSATD_ERR_INVALID_ARG, "psatd_coeffs_init was not called");
   TuneSpace ts = tune_space(p);
-  TuneCfg c{{-1, -1, -1, -1}, -1, push_ept((int)(p->ndim == 3 ? p->nz : p->ny), p->tc)};
+  TuneCfg c{{-1, -1, -1, -1}, -1, push_ept((int)(p->ndim == 3 ? p->nz : p->ny), p->tc, p->f32)};
   for (int k = 0; k < 4; ++k) {
     if (cfg[k] < 0) continue;
     if (cfg[k] > 30 || std::find(ts.rows[k].begin(), ts.rows[k].end(), cfg[k]) == ts.rows[k].end())
@@ -1121,9 +1170,8 @@ psatd_status psatd_plan_set_push_groups(psatd_plan p, int32_t groups) {
     p->cfg_push_groups = -1;
     return PSATD_OK;
   }
-  const int64_t nlines = p->ndim == 3 ? p->nxh * p->ny : p->nxh * p->npatch;
-  const int Ll = (int)(p->ndim == 3 ? p->nz : p->ny);
-  const int tb = p->cfg_push_tb > 0 ? p->cfg_push_tb : push_lines_per_cta(Ll, p->n_in, nlines, p->tc, p->f32, p->push_ept);
+  const int Ll = push_line_len(p);
+  const int tb = push_tb(p);
   int maxsm = 0;
   cudaDeviceGetAttribute(&maxsm, cudaDevAttrMaxSharedMemoryPerBlockOptin, p->device);
   const size_t csz = p->f32 ? 8 : 16;
@@ -1139,29 +1187,14 @@ psatd_status psatd_plan_set_push_groups(psatd_plan p, int32_t groups) {
 
 psatd_status psatd_plan_get_push_groups(psatd_plan p, int32_t* groups) {
   if (!p || !groups) return fail(p, PSATD_ERR_INVALID_ARG, "plan or groups is NULL");
-  const int64_t nlines = p->ndim == 3 ? p->nxh * p->ny : p->nxh * p->npatch;
-  const int Ll = (int)(p->ndim == 3 ? p->nz : p->ny);
-  const int tb = p->cfg_push_tb > 0 ? p->cfg_push_tb : push_lines_per_cta(Ll, p->n_in, nlines, p->tc, p->f32, p->push_ept);
-  int G = p->cfg_push_groups > 0 ? p->cfg_push_groups
-                                 : push_groups_default(Ll, p->push_ept, tb, p->n_in, p->tc, p->f32, p->f32 ? 8 : 16,
-                                                       p->maxsm, p->sm_bytes);
-  if (!push_groups_ok(Ll, p->push_ept, tb, G, p->tc, p->f32)) G = 1;
-  *groups = G;
+  *groups = push_groups(p);
   return PSATD_OK;
 }
 
 psatd_status psatd_plan_get_launch(psatd_plan p, int32_t cfg[6]) {
   if (!p || !cfg) return fail(p, PSATD_ERR_INVALID_ARG, "plan or cfg is NULL");
-  const int Lx = (int)(p->nx / 2);
-  const int64_t nlines = p->ndim == 3 ? p->nxh * p->ny : p->nxh * p->npatch;
-  const int Ll = (int)(p->ndim == 3 ? p->nz : p->ny);
-  const bool tc = p->tc;
-  const int dflt[4] = {pick_log_tb(Lx, p->ny, p->f32, tc, true),
-                       p->ndim == 3 ? pick_log_tb((int)p->ny, p->nz, p->f32, tc) : -1,
-                       p->ndim == 3 ? pick_log_tb_inv((int)p->ny, p->nz, p->f32, tc) : -1,
-                       pick_log_tb_inv(Lx, p->ny, p->f32, tc)};
-  for (int k = 0; k < 4; ++k) cfg[k] = p->cfg_log_tb[k] >= 0 ? p->cfg_log_tb[k] : dflt[k];
-  cfg[4] = p->cfg_push_tb > 0 ? p->cfg_push_tb : push_lines_per_cta(Ll, p->n_in, nlines, p->tc, p->f32, p->push_ept);
+  for (int k = 0; k < 4; ++k) cfg[k] = (p->ndim == 3 || k == 0 || k == 3) ? rows_per_cta(p, k) : p->cfg_log_tb[k];
+  cfg[4] = push_tb(p);
   cfg[5] = p->push_ept;
   return PSATD_OK;
 }
@@ -1428,7 +1461,7 @@ extern "C" psatd_status psatd_step_noalloc(const psatd_desc* desc, const psatd_f
   p.nz = p.ndim == 3 ? desc->n[2] : 1;
   p.nxh = p.nx / 2 + 1;
   p.cs = p.nxh * p.ny * p.nz;
-  p.push_ept = push_ept((int)(p.ndim == 3 ? p.nz : p.ny));
+  p.push_ept = push_ept((int)(p.ndim == 3 ? p.nz : p.ny), false, p.f32);
   const size_t csz = p.f32 ? 8 : 16;
   const int64_t ns[3] = {p.nx, p.ny, p.nz};
   p.tab_e[0] = p.nx / 2 + 1;
@@ -1613,7 +1646,7 @@ bool persist_y_len(int L, bool tc) {
 int fam_of(int L) { return pow2(L) ? 0 : 1; }
 // rows per item of a transposing pass and lines per item of the fused pass
 int persist_x_tb(int L) { return kPersistXThreads / (L / row_ept(L)); }
-int persist_y_tb(int L, bool tc) { return kPersistThreads / (L / (pow2(L) ? (tc ? 16 : 8) : 12)); }
+int persist_y_tb(int L, bool tc) { return kPersistThreads / (L / push_ept(L, tc, true)); }
 
 // X-pass arguments of class plan p for the step's field / source pointers (as
 // run_step's first and last passes in 2D).
@@ -1919,8 +1952,11 @@ extern "C" psatd_status psatd_batch_create(const psatd_desc* base, int32_t npatc
       return s;
     }
   }
-  // branch streams: up to 4, classes assigned largest first to the least loaded branch
-  const int nbr = (int)std::min<size_t>(4, b->cls.size());
+  // branch streams, classes assigned largest first to the least loaded branch: 4, or 2 in FP32, whose
+  // passes fill the SMs' registers by themselves and keep their class's spectra in L2 with fewer classes
+  // in flight (512 patches, four steps with 1 / 2 / 3 / 4 / 8 branches: FP32 10.6 / 9.0 / 9.3 / 9.4 / 10.6
+  // ms, split BF16 23.2 / 22.3 / - / 22.2 / 22.4 ms)
+  const int nbr = (int)std::min<size_t>(b->f32 && !b->cls[0]->tc ? 2 : 4, b->cls.size());
   if (nbr > 1) {
     cudaError_t e = cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming);
     for (int k = 0; k < nbr && e == cudaSuccess; ++k) {

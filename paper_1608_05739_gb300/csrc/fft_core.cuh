@@ -4,9 +4,9 @@
 // elements x[t + T*m], m < EPT, in registers before and after the transform
 // (natural order in both domains).  Lengths: powers of two 8..4096 with 8 or
 // 16 elements per thread (a radix-2/4/8 first stage, then radix-EPT stages),
-// 3 * 2^k, 48..3072, with 24 (radix 3, then 2/4, then 8) or 12 (prime-factor
-// radix 12, then 2, then 4), or 5 * 2^k, 80..1280, with 20 (radix 5, then 2,
-// then 4) -- FFTPlan below.  Between stages the data go
+// 3 * 2^k, 48..3072, with 24 (radix 3, 6 or 12, then 8) or 12 (radix 12, then 2,
+// then 4), or 5 * 2^k, 80..1280, with 20 (radix 10 or 20, then 4) -- FFTPlan
+// below.  Between stages the data go
 // through shared memory in rows of 16 elements whose columns are XOR-swizzled
 // per exchange (free of bank conflicts for each stage's write pattern).
 //
@@ -42,14 +42,47 @@ template <> struct Types<double> {
   static constexpr bool kComp = false;
 };
 
+// Two floats that go through the same arithmetic (the same element of two
+// transforms), computed with the packed FP32 instructions: one instruction for
+// both, each half rounded as the scalar operation, so a transform's bits do not
+// depend on whether it ran in a pair.
+struct alignas(8) F2 {
+  float a, b;
+};
+struct alignas(16) C2 {  // complex pair: (re, re), (im, im)
+  F2 x, y;
+};
+template <> struct Types<F2> {
+  typedef C2 C;
+  typedef float4 W;  // one twiddle serves both halves
+  static constexpr bool kComp = true;
+};
+__device__ __forceinline__ float2 f2v(F2 v) { return make_float2(v.a, v.b); }
+__device__ __forceinline__ F2 f2(float2 v) { return F2{v.x, v.y}; }
+__device__ __forceinline__ F2 operator+(F2 a, F2 b) { return f2(__fadd2_rn(f2v(a), f2v(b))); }
+// a - b as fma(b, -1, a): the product is exact, so this is the one rounding of a - b
+__device__ __forceinline__ F2 operator-(F2 a, F2 b) {
+  return f2(__ffma2_rn(f2v(b), make_float2(-1.f, -1.f), f2v(a)));
+}
+__device__ __forceinline__ F2 operator*(float s, F2 v) { return f2(__fmul2_rn(make_float2(s, s), f2v(v))); }
+__device__ __forceinline__ F2 fma_s(F2 v, float s, F2 c) {
+  return f2(__ffma2_rn(f2v(v), make_float2(s, s), f2v(c)));
+}
+__device__ __forceinline__ float fma_s(float v, float s, float c) { return fmaf(v, s, c); }
+__device__ __forceinline__ double fma_s(double v, float s, double c) { return fma(v, (double)s, c); }
+
 __device__ __forceinline__ float2 mkc(float a, float b) { return make_float2(a, b); }
 __device__ __forceinline__ double2 mkc(double a, double b) { return make_double2(a, b); }
+__device__ __forceinline__ C2 mkc(F2 a, F2 b) { return C2{a, b}; }
 
 template <class C> __device__ __forceinline__ C cadd(C a, C b) { return mkc(a.x + b.x, a.y + b.y); }
 template <class C> __device__ __forceinline__ C csub(C a, C b) { return mkc(a.x - b.x, a.y - b.y); }
 template <class C> __device__ __forceinline__ C cmul_mi(C a) { return mkc(a.y, -a.x); }  // * (-i)
 template <class C> __device__ __forceinline__ C cmul_pi(C a) { return mkc(-a.y, a.x); }  // * (+i)
 template <class C> __device__ __forceinline__ C cconj(C a) { return mkc(a.x, -a.y); }
+// a +- i b (the rotation costs no operation, also in the packed type)
+template <class C> __device__ __forceinline__ C add_i(C a, C b) { return mkc(a.x - b.y, a.y + b.x); }
+template <class C> __device__ __forceinline__ C sub_i(C a, C b) { return mkc(a.x + b.y, a.y - b.x); }
 
 // x * w, compensated: the low parts enter first, the leading product last.
 __device__ __forceinline__ float2 twmul(float2 x, float4 w) {
@@ -71,6 +104,25 @@ __device__ __forceinline__ float2 twmul_conj(float2 x, float4 w) {
   im = fmaf(x.y, w.x, im);
   return make_float2(re, im);
 }
+// the same products in the packed type (term by term as above)
+__device__ __forceinline__ C2 twmul(C2 x, float4 w) {
+  F2 re = fma_s(x.x, w.z, -w.w * x.y);
+  F2 im = fma_s(x.x, w.w, w.z * x.y);
+  re = fma_s(x.y, -w.y, re);
+  im = fma_s(x.y, w.x, im);
+  re = fma_s(x.x, w.x, re);
+  im = fma_s(x.x, w.y, im);
+  return C2{re, im};
+}
+__device__ __forceinline__ C2 twmul_conj(C2 x, float4 w) {
+  F2 re = fma_s(x.x, w.z, w.w * x.y);
+  F2 im = fma_s(x.y, w.z, -w.w * x.x);
+  re = fma_s(x.y, w.y, re);
+  im = fma_s(x.x, -w.y, im);
+  re = fma_s(x.x, w.x, re);
+  im = fma_s(x.y, w.x, im);
+  return C2{re, im};
+}
 __device__ __forceinline__ double2 twmul(double2 x, double2 w) {
   return make_double2(fma(x.x, w.x, -x.y * w.y), fma(x.x, w.y, x.y * w.x));
 }
@@ -81,18 +133,31 @@ __device__ __forceinline__ double2 twmul_conj(double2 x, double2 w) {
 // v * sqrt(1/2); in float as hi + lo (0.70710677f + 1.2101617e-8f).
 __device__ __forceinline__ float rsqrt2_mul(float v) { return fmaf(v, 0.70710677f, v * 1.2101617e-08f); }
 __device__ __forceinline__ double rsqrt2_mul(double v) { return v * 0.70710678118654752440; }
+__device__ __forceinline__ F2 rsqrt2_mul(F2 v) { return fma_s(v, 0.70710677f, 1.2101617e-08f * v); }
+// v * -sqrt(1/2)
+__device__ __forceinline__ float rsqrt2_mul_n(float v) { return fmaf(v, -0.70710677f, v * -1.2101617e-08f); }
+__device__ __forceinline__ double rsqrt2_mul_n(double v) { return v * -0.70710678118654752440; }
+__device__ __forceinline__ F2 rsqrt2_mul_n(F2 v) { return fma_s(v, -0.70710677f, -1.2101617e-08f * v); }
 
 // ---------------------------------------------------------------- butterflies
 // Radix-4 DFT in place (forward: exp(-2 pi i/4) = -i; adjoint: +i).  Exact
 // operations apart from the additions, so the adjoint is exact.
 template <bool ADJ, class C>
-__device__ __forceinline__ void dft4(C& x0, C& x1, C& x2, C& x3) {
-  C s0 = cadd(x0, x2), d0 = csub(x0, x2), s1 = cadd(x1, x3), t = csub(x1, x3);
-  C d1 = ADJ ? cmul_pi(t) : cmul_mi(t);
+__device__ __forceinline__ void dft4_tail(C s0, C d0, C s1, C t, C& x0, C& x1, C& x2, C& x3) {
   x0 = cadd(s0, s1);
-  x1 = cadd(d0, d1);
+  x1 = ADJ ? add_i(d0, t) : sub_i(d0, t);
   x2 = csub(s0, s1);
-  x3 = csub(d0, d1);
+  x3 = ADJ ? sub_i(d0, t) : add_i(d0, t);
+}
+template <bool ADJ, class C>
+__device__ __forceinline__ void dft4(C& x0, C& x1, C& x2, C& x3) {
+  dft4_tail<ADJ>(cadd(x0, x2), csub(x0, x2), cadd(x1, x3), csub(x1, x3), x0, x1, x2, x3);
+}
+// dft4 of (x0, x1, -+ i x2, x3) (forward -i, adjoint +i)
+template <bool ADJ, class C>
+__device__ __forceinline__ void dft4_r2(C& x0, C& x1, C& x2, C& x3) {
+  dft4_tail<ADJ>(ADJ ? add_i(x0, x2) : sub_i(x0, x2), ADJ ? sub_i(x0, x2) : add_i(x0, x2), cadd(x1, x3),
+                 csub(x1, x3), x0, x1, x2, x3);
 }
 
 // Radix-8 forward DFT, natural order in and out: split a_r +- a_(r+4), rotate
@@ -101,12 +166,11 @@ template <class C>
 __device__ __forceinline__ void dft8_fwd(C* a) {
   C b0 = cadd(a[0], a[4]), b1 = cadd(a[1], a[5]), b2 = cadd(a[2], a[6]), b3 = cadd(a[3], a[7]);
   C c0 = csub(a[0], a[4]), c1 = csub(a[1], a[5]), c2 = csub(a[2], a[6]), c3 = csub(a[3], a[7]);
-  // c1 *= s(1 - i); c2 *= -i; c3 *= s(-1 - i)
+  // c1 *= s(1 - i); c2 *= -i; c3 *= s(-1 - i) = (p, -q)
   c1 = mkc(rsqrt2_mul(c1.x + c1.y), rsqrt2_mul(c1.y - c1.x));
-  c2 = cmul_mi(c2);
-  c3 = mkc(rsqrt2_mul(c3.y - c3.x), rsqrt2_mul(-(c3.x + c3.y)));
+  const auto p = rsqrt2_mul(c3.y - c3.x), q = rsqrt2_mul(c3.x + c3.y);
   dft4<false>(b0, b1, b2, b3);
-  dft4<false>(c0, c1, c2, c3);
+  dft4_tail<false>(sub_i(c0, c2), add_i(c0, c2), mkc(c1.x + p, c1.y - q), mkc(c1.x - p, c1.y + q), c0, c1, c2, c3);
   a[0] = b0; a[1] = c0; a[2] = b1; a[3] = c1;
   a[4] = b2; a[5] = c2; a[6] = b3; a[7] = c3;
 }
@@ -118,12 +182,11 @@ __device__ __forceinline__ void dft8_adj(C* a) {
   C c0 = a[1], c1 = a[3], c2 = a[5], c3 = a[7];
   dft4<true>(b0, b1, b2, b3);
   dft4<true>(c0, c1, c2, c3);
-  // c1 *= s(1 + i); c2 *= +i; c3 *= s(-1 + i)
+  // c1 *= s(1 + i); c2 *= +i; c3 *= s(-1 + i) = (-q, p)
   c1 = mkc(rsqrt2_mul(c1.x - c1.y), rsqrt2_mul(c1.x + c1.y));
-  c2 = cmul_pi(c2);
-  c3 = mkc(rsqrt2_mul(-(c3.x + c3.y)), rsqrt2_mul(c3.x - c3.y));
-  a[0] = cadd(b0, c0); a[1] = cadd(b1, c1); a[2] = cadd(b2, c2); a[3] = cadd(b3, c3);
-  a[4] = csub(b0, c0); a[5] = csub(b1, c1); a[6] = csub(b2, c2); a[7] = csub(b3, c3);
+  const auto q = rsqrt2_mul(c3.x + c3.y), p = rsqrt2_mul(c3.x - c3.y);
+  a[0] = cadd(b0, c0); a[1] = cadd(b1, c1); a[2] = add_i(b2, c2); a[3] = mkc(b3.x - q, b3.y + p);
+  a[4] = csub(b0, c0); a[5] = csub(b1, c1); a[6] = sub_i(b2, c2); a[7] = mkc(b3.x + q, b3.y - p);
 }
 
 // Multiplication by constants of the radix-16 DFT: z (p + i q) with p, q the
@@ -144,6 +207,21 @@ template <> struct KMul<float2> {
     return make_float2(re, im);
   }
 };
+template <> struct KMul<C2> {
+  template <int P_NUM>
+  static __device__ __forceinline__ C2 mul(C2 z, double p, double q) {
+    const float ph = (float)p, pl = (float)(p - (double)ph), qh = (float)q, ql = (float)(q - (double)qh);
+    F2 re = pl * z.x;
+    re = fma_s(z.y, -ql, re);
+    re = fma_s(z.y, -qh, re);
+    re = fma_s(z.x, ph, re);
+    F2 im = ql * z.x;
+    im = fma_s(z.y, pl, im);
+    im = fma_s(z.y, ph, im);
+    im = fma_s(z.x, qh, im);
+    return C2{re, im};
+  }
+};
 template <> struct KMul<double2> {
   template <int P_NUM>
   static __device__ __forceinline__ double2 mul(double2 z, double p, double q) {
@@ -153,20 +231,20 @@ template <> struct KMul<double2> {
 constexpr double kCos8 = 0.92387953251128675613;  // cos(pi/8)
 constexpr double kSin8 = 0.38268343236508977173;  // sin(pi/8)
 
-// z * w16^e (forward, w16 = exp(-2 pi i/16)) or z * conj(w16^e) (adjoint), e in {1,2,3,4,6,9}
+// z * w16^e (forward, w16 = exp(-2 pi i/16)) or z * conj(w16^e) (adjoint), e in {1,2,3,6,9}
+// (e = 4, the rotation by -+i, is part of dft4_r2)
 template <int E, bool ADJ, class C>
 __device__ __forceinline__ C w16mul(C z) {
   constexpr double sg = ADJ ? 1.0 : -1.0;  // sign of the imaginary part of the constant
   if constexpr (E == 1) return KMul<C>::template mul<1>(z, kCos8, sg * kSin8);
   else if constexpr (E == 3) return KMul<C>::template mul<3>(z, kSin8, sg * kCos8);
-  else if constexpr (E == 9) { const C u = KMul<C>::template mul<1>(z, kCos8, sg * kSin8); return mkc(-u.x, -u.y); }
-  else if constexpr (E == 4) return ADJ ? cmul_pi(z) : cmul_mi(z);
+  else if constexpr (E == 9) return KMul<C>::template mul<1>(z, -kCos8, -sg * kSin8);
   else if constexpr (E == 2) {
     if constexpr (ADJ) return mkc(rsqrt2_mul(z.x - z.y), rsqrt2_mul(z.x + z.y));
     else return mkc(rsqrt2_mul(z.x + z.y), rsqrt2_mul(z.y - z.x));
   } else {  // E == 6
-    if constexpr (ADJ) return mkc(rsqrt2_mul(-(z.x + z.y)), rsqrt2_mul(z.x - z.y));
-    else return mkc(rsqrt2_mul(z.y - z.x), rsqrt2_mul(-(z.x + z.y)));
+    if constexpr (ADJ) return mkc(rsqrt2_mul_n(z.x + z.y), rsqrt2_mul(z.x - z.y));
+    else return mkc(rsqrt2_mul(z.y - z.x), rsqrt2_mul_n(z.x + z.y));
   }
 }
 
@@ -181,13 +259,15 @@ __device__ __forceinline__ void dft16_fwd(C* a) {
   a[9] = w16mul<2, false>(a[9]);
   a[13] = w16mul<3, false>(a[13]);
   a[6] = w16mul<2, false>(a[6]);
-  a[10] = w16mul<4, false>(a[10]);
   a[14] = w16mul<6, false>(a[14]);
   a[7] = w16mul<3, false>(a[7]);
   a[11] = w16mul<6, false>(a[11]);
   a[15] = w16mul<9, false>(a[15]);
 #pragma unroll
-  for (int k2 = 0; k2 < 4; ++k2) dft4<false>(a[4 * k2], a[4 * k2 + 1], a[4 * k2 + 2], a[4 * k2 + 3]);
+  for (int k2 = 0; k2 < 4; ++k2) {
+    if (k2 == 2) dft4_r2<false>(a[8], a[9], a[10], a[11]);
+    else dft4<false>(a[4 * k2], a[4 * k2 + 1], a[4 * k2 + 2], a[4 * k2 + 3]);
+  }
   C y[16];
 #pragma unroll
   for (int k2 = 0; k2 < 4; ++k2)
@@ -211,13 +291,15 @@ __device__ __forceinline__ void dft16_adj(C* a) {
   x[9] = w16mul<2, true>(x[9]);
   x[13] = w16mul<3, true>(x[13]);
   x[6] = w16mul<2, true>(x[6]);
-  x[10] = w16mul<4, true>(x[10]);
   x[14] = w16mul<6, true>(x[14]);
   x[7] = w16mul<3, true>(x[7]);
   x[11] = w16mul<6, true>(x[11]);
   x[15] = w16mul<9, true>(x[15]);
 #pragma unroll
-  for (int r1 = 0; r1 < 4; ++r1) dft4<true>(x[r1], x[r1 + 4], x[r1 + 8], x[r1 + 12]);
+  for (int r1 = 0; r1 < 4; ++r1) {
+    if (r1 == 2) dft4_r2<true>(x[2], x[6], x[10], x[14]);
+    else dft4<true>(x[r1], x[r1 + 4], x[r1 + 8], x[r1 + 12]);
+  }
 #pragma unroll
   for (int i = 0; i < 16; ++i) a[i] = x[i];
 }
@@ -229,6 +311,10 @@ __device__ __forceinline__ float r3_mul(float v) {
   return fmaf(v, h, v * l);
 }
 __device__ __forceinline__ double r3_mul(double v) { return v * kHalfSqrt3; }
+__device__ __forceinline__ F2 r3_mul(F2 v) {
+  constexpr float h = (float)kHalfSqrt3, l = (float)(kHalfSqrt3 - (double)(float)kHalfSqrt3);
+  return fma_s(v, h, l * v);
+}
 
 // Radix-3 DFT in place (forward: exp(-2 pi i/3) = -1/2 - i sqrt3/2; adjoint:
 // the conjugate constant): X0 = a0 + (a1 + a2), X1,2 = a0 - (a1 + a2)/2 -+ i
@@ -236,12 +322,11 @@ __device__ __forceinline__ double r3_mul(double v) { return v * kHalfSqrt3; }
 template <bool ADJ, class C>
 __device__ __forceinline__ void dft3(C& a0, C& a1, C& a2) {
   const C t = cadd(a1, a2), d = csub(a1, a2);
-  const C m = mkc(a0.x - 0.5f * t.x, a0.y - 0.5f * t.y);
-  const C sd = mkc(r3_mul(d.x), r3_mul(d.y));
-  const C s = ADJ ? cmul_pi(sd) : cmul_mi(sd);
+  const C m = mkc(fma_s(t.x, -0.5f, a0.x), fma_s(t.y, -0.5f, a0.y));
+  const C s = mkc(r3_mul(d.x), r3_mul(d.y));
   a0 = cadd(a0, t);
-  a1 = cadd(m, s);
-  a2 = csub(m, s);
+  a1 = ADJ ? add_i(m, s) : sub_i(m, s);
+  a2 = ADJ ? sub_i(m, s) : add_i(m, s);
 }
 
 // Radix-5 DFT in place.  With t1 = a1 + a4, t2 = a2 + a3, t3 = a1 - a4,
@@ -260,6 +345,11 @@ template <int K> __device__ __forceinline__ float k5_mul(float v) {
   constexpr float h = (float)c, l = (float)(c - (double)(float)c);
   return fmaf(v, h, v * l);
 }
+template <int K> __device__ __forceinline__ F2 k5_mul(F2 v) {
+  constexpr double c = K == 0 ? kC51 : K == 1 ? kC52 : K == 2 ? kS51 : kS52;
+  constexpr float h = (float)c, l = (float)(c - (double)(float)c);
+  return fma_s(v, h, l * v);
+}
 template <int K> __device__ __forceinline__ double k5_mul(double v) {
   return v * (K == 0 ? kC51 : K == 1 ? kC52 : K == 2 ? kS51 : kS52);
 }
@@ -270,57 +360,78 @@ __device__ __forceinline__ void dft5(C* a) {
   const C m2 = mkc(a[0].x + k5_mul<1>(t1.x) + k5_mul<0>(t2.x), a[0].y + k5_mul<1>(t1.y) + k5_mul<0>(t2.y));
   const C n1 = mkc(k5_mul<2>(t3.x) + k5_mul<3>(t4.x), k5_mul<2>(t3.y) + k5_mul<3>(t4.y));
   const C n2 = mkc(k5_mul<3>(t3.x) - k5_mul<2>(t4.x), k5_mul<3>(t3.y) - k5_mul<2>(t4.y));
-  const C in1 = ADJ ? cmul_pi(n1) : cmul_mi(n1), in2 = ADJ ? cmul_pi(n2) : cmul_mi(n2);
   a[0] = cadd(a[0], cadd(t1, t2));
-  a[1] = cadd(m1, in1);
-  a[4] = csub(m1, in1);
-  a[2] = cadd(m2, in2);
-  a[3] = csub(m2, in2);
+  a[1] = ADJ ? add_i(m1, n1) : sub_i(m1, n1);
+  a[4] = ADJ ? sub_i(m1, n1) : add_i(m1, n1);
+  a[2] = ADJ ? add_i(m2, n2) : sub_i(m2, n2);
+  a[3] = ADJ ? sub_i(m2, n2) : add_i(m2, n2);
 }
 
-// Radix-12 DFT in place, natural order in and out, as the prime-factor
-// (Good-Thomas) split 12 = 3 x 4: with n = (4 n1 + 3 n2) mod 12 and
-// k = (4 k1 + 9 k2) mod 12, W12^(n k) = W3^(n1 k1) W4^(n2 k2), so radix-3 DFTs
-// over n1 and radix-4 DFTs over n2 need no twiddles between them.  The adjoint
+// DFT of N1 * N2 points in place, natural order in and out, N1 and N2 coprime, as the
+// prime-factor (Good-Thomas) split: with n = (N2 n1 + N1 n2) mod N and k the residue
+// with k = k1 mod N1, k = k2 mod N2, W_N^(n k) = W_N1^(n1 k1) W_N2^(n2 k2) where N2 k1 =
+// k mod N1 and N1 k2 = k mod N2 fold into the index maps below, so the DFTs over n1 and
+// n2 need no twiddles between them.  k = (K1 k1 + K2 k2) mod N with K1 = 1 mod N1, 0 mod
+// N2 and K2 = 0 mod N1, 1 mod N2, for (N1, N2): (2, 3), (4, 3), (2, 5), (4, 5).  The adjoint
 // runs the same steps in reverse order with the conjugate DFTs.
-template <bool ADJ, class C>
-__device__ __forceinline__ void dft12(C* a) {
-  C y[12];
+template <int N, bool ADJ, class C>
+__device__ __forceinline__ void dft_small(C* a) {
+  if constexpr (N == 2) {
+    const C s = cadd(a[0], a[1]), d = csub(a[0], a[1]);
+    a[0] = s;
+    a[1] = d;
+  } else if constexpr (N == 3) {
+    dft3<ADJ>(a[0], a[1], a[2]);
+  } else if constexpr (N == 4) {
+    dft4<ADJ>(a[0], a[1], a[2], a[3]);
+  } else {
+    dft5<ADJ>(a);
+  }
+}
+template <int N1, int N2, bool ADJ, class C>
+__device__ __forceinline__ void dft_pfa(C* a) {
+  constexpr int N = N1 * N2;
+  constexpr int K1 = N2 == 3 ? (N1 == 2 ? 3 : 9) : 5;             // 1 mod N1, 0 mod N2
+  constexpr int K2 = N2 == 3 ? 4 : (N1 == 2 ? 6 : 16);            // 0 mod N1, 1 mod N2
+  static_assert(K1 % N1 == 1 && K1 % N2 == 0 && K2 % N1 == 0 && K2 % N2 == 1, "index maps");
+  C y[N];  // y[n1 * N2 + k2]
   if constexpr (!ADJ) {
 #pragma unroll
-    for (int n2 = 0; n2 < 4; ++n2) {
-      C c0 = a[(3 * n2) % 12], c1 = a[(4 + 3 * n2) % 12], c2 = a[(8 + 3 * n2) % 12];
-      dft3<false>(c0, c1, c2);
-      y[3 * n2] = c0;
-      y[3 * n2 + 1] = c1;
-      y[3 * n2 + 2] = c2;
+    for (int n1 = 0; n1 < N1; ++n1) {
+      C c[N2];
+#pragma unroll
+      for (int n2 = 0; n2 < N2; ++n2) c[n2] = a[(N2 * n1 + N1 * n2) % N];
+      dft_small<N2, false>(c);
+#pragma unroll
+      for (int k2 = 0; k2 < N2; ++k2) y[n1 * N2 + k2] = c[k2];
     }
 #pragma unroll
-    for (int k1 = 0; k1 < 3; ++k1) {
-      C d0 = y[k1], d1 = y[3 + k1], d2 = y[6 + k1], d3 = y[9 + k1];
-      dft4<false>(d0, d1, d2, d3);
-      a[(4 * k1) % 12] = d0;
-      a[(4 * k1 + 9) % 12] = d1;
-      a[(4 * k1 + 18) % 12] = d2;
-      a[(4 * k1 + 27) % 12] = d3;
+    for (int k2 = 0; k2 < N2; ++k2) {
+      C d[N1];
+#pragma unroll
+      for (int n1 = 0; n1 < N1; ++n1) d[n1] = y[n1 * N2 + k2];
+      dft_small<N1, false>(d);
+#pragma unroll
+      for (int k1 = 0; k1 < N1; ++k1) a[(K1 * k1 + K2 * k2) % N] = d[k1];
     }
   } else {
 #pragma unroll
-    for (int k1 = 0; k1 < 3; ++k1) {
-      C d0 = a[(4 * k1) % 12], d1 = a[(4 * k1 + 9) % 12], d2 = a[(4 * k1 + 18) % 12], d3 = a[(4 * k1 + 27) % 12];
-      dft4<true>(d0, d1, d2, d3);
-      y[k1] = d0;
-      y[3 + k1] = d1;
-      y[6 + k1] = d2;
-      y[9 + k1] = d3;
+    for (int k2 = 0; k2 < N2; ++k2) {
+      C d[N1];
+#pragma unroll
+      for (int k1 = 0; k1 < N1; ++k1) d[k1] = a[(K1 * k1 + K2 * k2) % N];
+      dft_small<N1, true>(d);
+#pragma unroll
+      for (int n1 = 0; n1 < N1; ++n1) y[n1 * N2 + k2] = d[n1];
     }
 #pragma unroll
-    for (int n2 = 0; n2 < 4; ++n2) {
-      C c0 = y[3 * n2], c1 = y[3 * n2 + 1], c2 = y[3 * n2 + 2];
-      dft3<true>(c0, c1, c2);
-      a[(3 * n2) % 12] = c0;
-      a[(4 + 3 * n2) % 12] = c1;
-      a[(8 + 3 * n2) % 12] = c2;
+    for (int n1 = 0; n1 < N1; ++n1) {
+      C c[N2];
+#pragma unroll
+      for (int k2 = 0; k2 < N2; ++k2) c[k2] = y[n1 * N2 + k2];
+      dft_small<N2, true>(c);
+#pragma unroll
+      for (int n2 = 0; n2 < N2; ++n2) a[(N2 * n1 + N1 * n2) % N] = c[n2];
     }
   }
 }
@@ -331,12 +442,16 @@ __device__ __forceinline__ void butterfly(C* a) {
     dft3<ADJ>(a[0], a[1], a[2]);
   } else if constexpr (RS == 5) {
     dft5<ADJ>(a);
+  } else if constexpr (RS == 6) {
+    dft_pfa<2, 3, ADJ>(a);
   } else if constexpr (RS == 12) {
-    dft12<ADJ>(a);
+    dft_pfa<4, 3, ADJ>(a);
+  } else if constexpr (RS == 10) {
+    dft_pfa<2, 5, ADJ>(a);
+  } else if constexpr (RS == 20) {
+    dft_pfa<4, 5, ADJ>(a);
   } else if constexpr (RS == 2) {
-    C s = cadd(a[0], a[1]), d = csub(a[0], a[1]);
-    a[0] = s;
-    a[1] = d;
+    dft_small<2, ADJ>(a);
   } else if constexpr (RS == 4) {
     dft4<ADJ>(a[0], a[1], a[2], a[3]);
   } else if constexpr (RS == 8) {
@@ -349,39 +464,48 @@ __device__ __forceinline__ void butterfly(C* a) {
 // ---------------------------------------------------------------- stage plan
 __host__ __device__ constexpr int ilog2(int v) { return v <= 1 ? 0 : 1 + ilog2(v >> 1); }
 
-// Elements per thread of the transposing row/line passes (16 from L = 16 on)
-// and of the fused last-axis pass (8).
 __host__ __device__ constexpr bool is_pow2(int v) { return v > 0 && (v & (v - 1)) == 0; }
 
-// Lengths 3 * 2^k (k >= 4) are mixed-radix: 24 elements per thread in the
-// transposing passes, 12 in the fused pass (whose shared memory per line is
-// fixed, so that fewer elements per thread keep more threads on an SM).
-// Lengths 5 * 2^k (k >= 4): 20 elements per thread in every pass.
+// Transposing passes: 16 elements per thread; 5 * 2^k lengths 20; 3 * 2^k lengths 12 up
+// to 384 points, where 24 (one exchange fewer, but half the warps: 230 registers a
+// thread) measured slower (192^3 y forward 121 -> 109 us, inverse 72.1 -> 66.1; the FP32
+// batch of 512 patches 10.1 -> 9.4 ms per four steps), and 24 beyond (1536 points: 121
+// us, with 12 131; 768 points: 19.0, with 12 20.6).  The fused pass takes 12 for 3 * 2^k.
 __host__ __device__ constexpr int odd_factor(int v) { return is_pow2(v) ? 1 : (v % 3 == 0 ? 3 : 5); }
+__host__ __device__ constexpr int row_ept(int L) {
+  return odd_factor(L) == 3 ? (L <= 384 ? 12 : 24) : odd_factor(L) == 5 ? 20 : L >= 16 ? 16 : 8;
+}
 template <int L>
-struct RowEPT { static constexpr int value = odd_factor(L) == 3 ? 24 : odd_factor(L) == 5 ? 20 : L >= 16 ? 16 : 8; };
-// The fused pass keeps 8 elements per thread: with 16 a 2048-point line has
-// half the threads and, its shared memory being fixed per line, the SM half
-// the warps (measured slower).  The tensor-core variant (TC) takes 16, so that
-// its stages are radix-16 DFT-matrix contractions.
-template <int L, int TC = 0>
-struct PushEPT { static constexpr int value = odd_factor(L) == 3 ? 12 : odd_factor(L) == 5 ? 20 : TC ? 16 : 8; };
+struct RowEPT { static constexpr int value = row_ept(L); };
+// Elements per thread of the fused pass by default.  8 (radix-8 stages) up to 512
+// points; 16 (radix-16 stages) from 1024 points on in FP32, where they save an
+// exchange and a quarter of the shared-memory traffic and component groups make
+// up for the threads (2048 points TE: 75.7 us with 8, 73.1 us with 16 and two
+// groups; 1024 points, eleven components: 0.968 / 0.884 ms; 512 points: 12.2 /
+// 18.5 us), and in the tensor-core variant (TC), whose stages are radix-16
+// DFT-matrix contractions.
+__host__ __device__ constexpr int push_ept(int L, bool tc, bool f32) {
+  return odd_factor(L) == 3 ? 12 : odd_factor(L) == 5 ? 20 : (tc || (f32 && L >= 1024)) ? 16 : 8;
+}
+template <int L, int TC, bool F32>
+struct PushEPT { static constexpr int value = push_ept(L, TC != 0, F32); };
 
 // Power-of-two L: a radix-2/4/8 first stage when log2 L is not a multiple of
-// log2 EPT, then radix-EPT stages.  Mixed L = 3 * 2^k: with EPT = 24 a radix-3
-// first stage, a radix-2 or radix-4 stage when k is not a multiple of 3, then
-// radix-8 stages; with EPT = 12 a radix-12 first stage (prime-factor 3 x 4),
-// a radix-2 stage when k is odd, then radix-4 stages.  Mixed L = 5 * 2^k
-// (EPT = 20): a radix-5 first stage, a radix-2 stage when k is odd, then
-// radix-4 stages.  Every radix divides EPT.
+// log2 EPT, then radix-EPT stages.  Mixed lengths take the odd factor and a power of
+// two in a prime-factor first stage (no twiddles inside it).  L = 3 * 2^k: with EPT =
+// 24 radix 3, 6 or 12, then radix-8 stages (two exchanges at 384 and 768 points, one
+// at 48 and 96; as radix 3, (2 | 4), 8, .. they had one more); with EPT = 12 radix 12,
+// a radix-2 stage when k is odd, then radix-4 stages.  L = 5 * 2^k (EPT = 20): radix
+// 10 or 20, then radix-4 stages.  Every radix divides EPT.
 template <int L, int EPT = 8>
 struct FFTPlan {
   static constexpr int kEPT = EPT;
   static constexpr int kF = odd_factor(L);  // 1, 3 or 5
   static constexpr bool kMixed = kF > 1;
   static constexpr int kLog = ilog2(L / kF);  // log2 of the power-of-two part
-  static constexpr int kHeadLog = (kF == 3 && EPT == 12) ? 2 : 0;  // power of two taken by the first stage
   static constexpr int kB = kF == 5 ? 2 : kMixed ? (EPT == 12 ? 2 : 3) : ilog2(EPT);
+  // power of two taken by the first stage of a mixed length (prime-factor DFTs: 3 * 2^h, 5 * 2^h)
+  static constexpr int kHeadLog = !kMixed ? 0 : EPT == 12 ? 2 : kF == 5 ? (kLog % 2 ? 1 : 2) : kLog % 3;
   static constexpr int kRem = (kLog - kHeadLog) % kB;
   static constexpr int kR0 = kMixed ? kF << kHeadLog : kRem ? (1 << kRem) : EPT;
   static constexpr int kStages = kMixed ? 1 + (kRem ? 1 : 0) + (kLog - kHeadLog) / kB

@@ -28,8 +28,9 @@ template <typename R, int TC = 0>
 cudaError_t launch_inv_T(int L, bool c2r, const PassGeom& g, cudaStream_t st, const LineIO& io,
                          const void* tw, int64_t in_sa0, int64_t in_sk, int64_t out_sa0,
                          int64_t out_sb, const int64_t* a0_off = nullptr);
-// EPT: 8 or 16 elements per thread (radix-8 / radix-16 stages); TC needs 16.
-template <typename R, int TC, int EPT>
+// EPT: 8 or 16 elements per thread (radix-8 / radix-16 stages); TC needs 16.  LS: the
+// layouts 0, 1 (LS 0) or 2, 3 (LS 1), a translation unit each.
+template <typename R, int TC, int EPT, int LS>
 cudaError_t launch_line_push(int L, int layout, dim3 grid, int tb, int groups, size_t smem, cudaStream_t st,
                              const PushArgs<R>& a, const void* tw);
 
@@ -42,7 +43,7 @@ template <typename R>
 cudaError_t launch_inv_T3(int L, bool c2r, const PassGeom& g, cudaStream_t st, const LineIO& io, const void* tw,
                           int64_t in_sa0, int64_t in_sk, int64_t out_sa0, int64_t out_sb,
                           const int64_t* a0_off = nullptr);
-template <typename R>
+template <typename R, int LS>
 cudaError_t launch_line_push3(int L, int layout, dim3 grid, int tb, int groups, size_t smem, cudaStream_t st,
                               const PushArgs<R>& a, const void* tw);
 
@@ -55,7 +56,7 @@ template <typename R>
 cudaError_t launch_inv_T5(int L, bool c2r, const PassGeom& g, cudaStream_t st, const LineIO& io, const void* tw,
                           int64_t in_sa0, int64_t in_sk, int64_t out_sa0, int64_t out_sb,
                           const int64_t* a0_off = nullptr);
-template <typename R>
+template <typename R, int LS>
 cudaError_t launch_line_push5(int L, int layout, dim3 grid, int tb, int groups, size_t smem, cudaStream_t st,
                               const PushArgs<R>& a, const void* tw);
 

@@ -2,8 +2,13 @@
 // length; included by the per-precision translation units.
 #pragma once
 #include "launch.h"
+#include "pair_push.cuh"
+#include "pair_rows.cuh"
 
 namespace psatd {
+
+// The FP32 passes without tensor cores run in pairs (pair_rows.cuh, pair_push.cuh).
+template <typename R, int TC> constexpr bool kPairs = sizeof(R) == 4 && TC == 0;
 
 // Dynamic shared-memory opt-in (static shared memory adds to the request).  The
 // carveout is left to the driver: a maximal shared carveout shrinks the L1 that
@@ -15,51 +20,69 @@ static cudaError_t set_smem(K kern, size_t smem) {
   return cudaSuccess;
 }
 
+template <typename R, int TC, int L, bool R2C>
+static cudaError_t fwd_T_L_k(const PassGeom& g, cudaStream_t st, const LineIO& io, const void* tw, int64_t a, int64_t b,
+                           int64_t c, int64_t d, const int64_t* off) {
+  typedef typename Types<R>::W W;
+  constexpr int T = FFTPlan<L, RowEPT<L>::value>::kT;
+  cudaError_t e;
+  if constexpr (kPairs<R, TC>) {
+    const unsigned pairs = g.log_tb > 0 ? 1u << (g.log_tb - 1) : 1u;
+    const size_t smem = (size_t)pairs * L * sizeof(C2);
+    auto kern = k_fwd_P<L, R2C>;
+    if ((e = set_smem(kern, smem)) != cudaSuccess) return e;
+    kern<<<g.grid, dim3(T, pairs), smem, st>>>(io, static_cast<const W*>(tw), a, b, c, d, g.log_tb, off);
+  } else {
+    auto kern = k_fwd_T<R, L, R2C, TC>;
+    if ((e = set_smem(kern, g.smem)) != cudaSuccess) return e;
+    kern<<<g.grid, dim3(T, 1u << g.log_tb), g.smem, st>>>(io, static_cast<const W*>(tw), a, b, c, d, g.log_tb, off);
+  }
+  return cudaGetLastError();
+}
 template <typename R, int TC, int L>
 static cudaError_t fwd_T_L(bool r2c, const PassGeom& g, cudaStream_t st, const LineIO& io,
                            const void* tw, int64_t a, int64_t b, int64_t c, int64_t d, const int64_t* off) {
+  if (!r2c) return fwd_T_L_k<R, TC, L, false>(g, st, io, tw, a, b, c, d, off);
+  if constexpr (L <= 2048) return fwd_T_L_k<R, TC, L, true>(g, st, io, tw, a, b, c, d, off);
+  else return cudaErrorInvalidValue;
+}
+
+template <typename R, int TC, int L, bool C2R>
+static cudaError_t inv_T_L_k(const PassGeom& g, cudaStream_t st, const LineIO& io, const void* tw, int64_t a, int64_t b,
+                           int64_t c, int64_t d, const int64_t* off) {
   typedef typename Types<R>::W W;
-  const dim3 block(FFTPlan<L, RowEPT<L>::value>::kT, 1u << g.log_tb);
+  constexpr int T = FFTPlan<L, RowEPT<L>::value>::kT;
   cudaError_t e;
-  if (r2c) {
-    if constexpr (L <= 2048) {
-      auto kern = k_fwd_T<R, L, true, TC>;
-      if ((e = set_smem(kern, g.smem)) != cudaSuccess) return e;
-      kern<<<g.grid, block, g.smem, st>>>(io, static_cast<const W*>(tw), a, b, c, d, g.log_tb, off);
-    } else {
-      return cudaErrorInvalidValue;
-    }
+  if constexpr (kPairs<R, TC>) {
+    const unsigned pairs = g.log_tb > 0 ? 1u << (g.log_tb - 1) : 1u;
+    const size_t smem = (size_t)pairs * L * sizeof(C2);
+    auto kern = k_inv_P<L, C2R>;
+    if ((e = set_smem(kern, smem)) != cudaSuccess) return e;
+    kern<<<g.grid, dim3(T, pairs), smem, st>>>(io, static_cast<const W*>(tw), a, b, c, d, g.log_tb, off);
   } else {
-    auto kern = k_fwd_T<R, L, false, TC>;
+    auto kern = k_inv_T<R, L, C2R, TC>;
     if ((e = set_smem(kern, g.smem)) != cudaSuccess) return e;
-    kern<<<g.grid, block, g.smem, st>>>(io, static_cast<const W*>(tw), a, b, c, d, g.log_tb, off);
+    kern<<<g.grid, dim3(T, 1u << g.log_tb), g.smem, st>>>(io, static_cast<const W*>(tw), a, b, c, d, g.log_tb, off);
   }
   return cudaGetLastError();
 }
-
 template <typename R, int TC, int L>
 static cudaError_t inv_T_L(bool c2r, const PassGeom& g, cudaStream_t st, const LineIO& io,
                            const void* tw, int64_t a, int64_t b, int64_t c, int64_t d, const int64_t* off) {
-  typedef typename Types<R>::W W;
-  const dim3 block(FFTPlan<L, RowEPT<L>::value>::kT, 1u << g.log_tb);
-  cudaError_t e;
-  if (c2r) {
-    if constexpr (L <= 2048) {
-      auto kern = k_inv_T<R, L, true, TC>;
-      if ((e = set_smem(kern, g.smem)) != cudaSuccess) return e;
-      kern<<<g.grid, block, g.smem, st>>>(io, static_cast<const W*>(tw), a, b, c, d, g.log_tb, off);
-    } else {
-      return cudaErrorInvalidValue;
-    }
-  } else {
-    auto kern = k_inv_T<R, L, false, TC>;
-    if ((e = set_smem(kern, g.smem)) != cudaSuccess) return e;
-    kern<<<g.grid, block, g.smem, st>>>(io, static_cast<const W*>(tw), a, b, c, d, g.log_tb, off);
-  }
-  return cudaGetLastError();
+  if (!c2r) return inv_T_L_k<R, TC, L, false>(g, st, io, tw, a, b, c, d, off);
+  if constexpr (L <= 2048) return inv_T_L_k<R, TC, L, true>(g, st, io, tw, a, b, c, d, off);
+  else return cudaErrorInvalidValue;
 }
 
-template <typename R, int TC, int EPT, int L>
+template <typename R, int TC, int EPT, int L, int LAYOUT, bool GRP>
+static auto push_kernel() {
+  // radix-16 lines run in groups by default and share one kernel for any count; the others
+  // keep a plain kernel, 2 to 4 % faster than the group one with a single group
+  if constexpr (kPairs<R, TC>) return k_line_pair<L, LAYOUT, EPT, GRP || EPT == 16>;
+  else return k_line_push<R, L, LAYOUT, TC, EPT, GRP>;
+}
+
+template <typename R, int TC, int EPT, int L, int LS>
 static cudaError_t push_L(int layout, dim3 grid, int tb, int groups, size_t smem, cudaStream_t st,
                           const PushArgs<R>& a, const void* tw) {
   typedef typename Types<R>::W W;
@@ -67,14 +90,15 @@ static cudaError_t push_L(int layout, dim3 grid, int tb, int groups, size_t smem
     return cudaErrorInvalidValue;
   } else {
     const dim3 block(FFTPlan<L, EPT>::kT, tb, groups);
-    // component groups: their own instantiation, for whole-warp lines in FP32 and
-    // for the tensor-core pairs (the host admits groups > 1 nowhere else)
-    constexpr bool kGrpOk = TC ? EPT == 16 : (sizeof(R) == 4 && FFTPlan<L, EPT>::kT % 32 == 0);
-    if (groups > 1 && !kGrpOk) return cudaErrorInvalidValue;
+    // component groups: their own instantiation, in FP32 for blocks of whole-warp groups
+    // and for the tensor-core pairs (the host admits groups > 1 nowhere else)
+    constexpr bool kGrpOk = TC ? EPT == 16 : kPairs<R, TC>;
+    if (groups > 1 && (!kGrpOk || (kPairs<R, TC> && (block.x * block.y) % 32 != 0))) return cudaErrorInvalidValue;
+    if constexpr (kPairs<R, TC>) smem = (size_t)a.n_in * tb * L * sizeof(float2);  // the units alone
     cudaError_t e;
 #define PSATD_PUSH_LAUNCH(LAY, GRP)                                            \
   {                                                                            \
-    auto kern = k_line_push<R, L, LAY, TC, EPT, GRP>;                          \
+    auto kern = push_kernel<R, TC, EPT, L, LAY, GRP>();                        \
     if ((e = set_smem(kern, smem)) != cudaSuccess) return e;                   \
     kern<<<grid, block, smem, st>>>(a, static_cast<const W*>(tw));             \
   }
@@ -88,13 +112,18 @@ static cudaError_t push_L(int layout, dim3 grid, int tb, int groups, size_t smem
     }                                                                          \
     break;                                                                     \
   }
-    switch (layout) {
-      PSATD_PUSH_CASE(0)
-      PSATD_PUSH_CASE(1)
-      PSATD_PUSH_CASE(2)
-      PSATD_PUSH_CASE(3)
-      default:
-        return cudaErrorInvalidValue;
+    if constexpr (LS == 0) {
+      switch (layout) {
+        PSATD_PUSH_CASE(0)
+        PSATD_PUSH_CASE(1)
+        default: return cudaErrorInvalidValue;
+      }
+    } else {
+      switch (layout) {
+        PSATD_PUSH_CASE(2)
+        PSATD_PUSH_CASE(3)
+        default: return cudaErrorInvalidValue;
+      }
     }
 #undef PSATD_PUSH_CASE
 #undef PSATD_PUSH_LAUNCH
@@ -153,15 +182,15 @@ cudaError_t launch_inv_T5(int L, bool c2r, const PassGeom& g, cudaStream_t st, c
                           int64_t in_sa0, int64_t in_sk, int64_t out_sa0, int64_t out_sb, const int64_t* a0_off) {
   PSATD_L5_SWITCH(inv_T_L, c2r, g, st, io, tw, in_sa0, in_sk, out_sa0, out_sb, a0_off)
 }
-template <typename R>
+template <typename R, int LS>
 cudaError_t launch_line_push5(int L, int layout, dim3 grid, int tb, int groups, size_t smem, cudaStream_t st,
                               const PushArgs<R>& a, const void* tw) {
   switch (L) {
-    case 80: return push_L<R, 0, 20, 80>(layout, grid, tb, groups, smem, st, a, tw);
-    case 160: return push_L<R, 0, 20, 160>(layout, grid, tb, groups, smem, st, a, tw);
-    case 320: return push_L<R, 0, 20, 320>(layout, grid, tb, groups, smem, st, a, tw);
-    case 640: return push_L<R, 0, 20, 640>(layout, grid, tb, groups, smem, st, a, tw);
-    case 1280: return push_L<R, 0, 20, 1280>(layout, grid, tb, groups, smem, st, a, tw);
+    case 80: return push_L<R, 0, 20, 80, LS>(layout, grid, tb, groups, smem, st, a, tw);
+    case 160: return push_L<R, 0, 20, 160, LS>(layout, grid, tb, groups, smem, st, a, tw);
+    case 320: return push_L<R, 0, 20, 320, LS>(layout, grid, tb, groups, smem, st, a, tw);
+    case 640: return push_L<R, 0, 20, 640, LS>(layout, grid, tb, groups, smem, st, a, tw);
+    case 1280: return push_L<R, 0, 20, 1280, LS>(layout, grid, tb, groups, smem, st, a, tw);
     default: return cudaErrorInvalidValue;
   }
 }
@@ -176,17 +205,17 @@ cudaError_t launch_inv_T3(int L, bool c2r, const PassGeom& g, cudaStream_t st, c
                           int64_t in_sa0, int64_t in_sk, int64_t out_sa0, int64_t out_sb, const int64_t* a0_off) {
   PSATD_L3_SWITCH(inv_T_L, c2r, g, st, io, tw, in_sa0, in_sk, out_sa0, out_sb, a0_off)
 }
-template <typename R>
+template <typename R, int LS>
 cudaError_t launch_line_push3(int L, int layout, dim3 grid, int tb, int groups, size_t smem, cudaStream_t st,
                               const PushArgs<R>& a, const void* tw) {
   switch (L) {
-    case 48: return push_L<R, 0, 12, 48>(layout, grid, tb, groups, smem, st, a, tw);
-    case 96: return push_L<R, 0, 12, 96>(layout, grid, tb, groups, smem, st, a, tw);
-    case 192: return push_L<R, 0, 12, 192>(layout, grid, tb, groups, smem, st, a, tw);
-    case 384: return push_L<R, 0, 12, 384>(layout, grid, tb, groups, smem, st, a, tw);
-    case 768: return push_L<R, 0, 12, 768>(layout, grid, tb, groups, smem, st, a, tw);
-    case 1536: return push_L<R, 0, 12, 1536>(layout, grid, tb, groups, smem, st, a, tw);
-    case 3072: return push_L<R, 0, 12, 3072>(layout, grid, tb, groups, smem, st, a, tw);
+    case 48: return push_L<R, 0, 12, 48, LS>(layout, grid, tb, groups, smem, st, a, tw);
+    case 96: return push_L<R, 0, 12, 96, LS>(layout, grid, tb, groups, smem, st, a, tw);
+    case 192: return push_L<R, 0, 12, 192, LS>(layout, grid, tb, groups, smem, st, a, tw);
+    case 384: return push_L<R, 0, 12, 384, LS>(layout, grid, tb, groups, smem, st, a, tw);
+    case 768: return push_L<R, 0, 12, 768, LS>(layout, grid, tb, groups, smem, st, a, tw);
+    case 1536: return push_L<R, 0, 12, 1536, LS>(layout, grid, tb, groups, smem, st, a, tw);
+    case 3072: return push_L<R, 0, 12, 3072, LS>(layout, grid, tb, groups, smem, st, a, tw);
     default: return cudaErrorInvalidValue;
   }
 }
@@ -205,10 +234,10 @@ cudaError_t launch_inv_T(int L, bool c2r, const PassGeom& g, cudaStream_t st, co
   PSATD_L_SWITCH(inv_T_L, c2r, g, st, io, tw, in_sa0, in_sk, out_sa0, out_sb, a0_off)
 }
 
-template <typename R, int TC, int EPT>
+template <typename R, int TC, int EPT, int LS>
 static cudaError_t push_L_e(int layout, dim3 grid, int tb, int groups, size_t smem, cudaStream_t st,
                             const PushArgs<R>& a, const void* tw, int L) {
-#define PUSH_E(LL) push_L<R, TC, EPT, LL>
+#define PUSH_E(LL) push_L<R, TC, EPT, LL, LS>
   switch (L) {
     case 8: if constexpr (!TC) return PUSH_E(8)(layout, grid, tb, groups, smem, st, a, tw);
             else return cudaErrorInvalidValue;
@@ -226,10 +255,10 @@ static cudaError_t push_L_e(int layout, dim3 grid, int tb, int groups, size_t sm
 #undef PUSH_E
 }
 
-template <typename R, int TC, int EPT>
+template <typename R, int TC, int EPT, int LS>
 cudaError_t launch_line_push(int L, int layout, dim3 grid, int tb, int groups, size_t smem, cudaStream_t st,
                              const PushArgs<R>& a, const void* tw) {
-  return push_L_e<R, TC, EPT>(layout, grid, tb, groups, smem, st, a, tw, L);
+  return push_L_e<R, TC, EPT, LS>(layout, grid, tb, groups, smem, st, a, tw, L);
 }
 
 }  // namespace psatd

@@ -9,6 +9,7 @@
 // another.  The last CTA to finish zeroes the queue for the next launch.
 #pragma once
 
+#include "pair_push.cuh"
 #include "psatd_kernels.cuh"
 
 namespace psatd {
@@ -145,7 +146,6 @@ __global__ void __launch_bounds__(kPersistThreads, TC ? 2 : 4) k_persist_push(co
   TcCtx tc;
   if constexpr (TC) tc_setup(tc, smem_raw, cls[0].gmat, 0u, cls[0].err, TC == 2, 0u, cls[0].tc_ctl);
   // (the queue's first take has a block barrier before any use of the stage mbarrier)
-  constexpr int EPT = FAM ? 12 : (TC ? 16 : 8);
   for (;;) {
     const int i0 = persist_take(q, &slot);
     if (i0 >= q.n_items) break;
@@ -159,10 +159,17 @@ __global__ void __launch_bounds__(kPersistThreads, TC ? 2 : 4) k_persist_push(co
 #define PSATD_Y_CASE(LL)                                                                                   \
   if (Lc == LL) {                                                                                          \
     matched = true;                                                                                        \
-    constexpr int T = LL / EPT;                                                                            \
-    line_push_body<R, LL, LAYOUT, TC, EPT>(A, static_cast<const W*>(tws[it.cls]), it.blk,                 \
-                                           (int)threadIdx.x % T, (int)threadIdx.x / T, kPersistThreads / T, \
-                                           0, 1, smem_raw, tc, sc);                                        \
+    constexpr int EPT = push_ept(LL, TC != 0, true), T = LL / EPT;                                         \
+    const int t = (int)threadIdx.x % T, g = (int)threadIdx.x / T;                                          \
+    const W* tw = static_cast<const W*>(tws[it.cls]);                                                      \
+    if constexpr (TC) {                                                                                    \
+      line_push_body<R, LL, LAYOUT, TC, EPT>(A, tw, it.blk, t, g, kPersistThreads / T, 0, 1, smem_raw, tc, sc); \
+    } else {                                                                                               \
+      __syncthreads(); /* the previous item's shared memory is free */                                     \
+      if (line_pair_body<LL, LAYOUT, EPT, false>(A, tw, it.blk, t, g, kPersistThreads / T, 0, 1, smem_raw, sc.mbar, \
+                                                 sc.phase))                                                 \
+        sc.phase ^= 1u;                                                                                    \
+    }                                                                                                      \
   }
       PSATD_PERSIST_Y_LENGTHS(FAM, PSATD_Y_CASE)
 #undef PSATD_Y_CASE
@@ -183,8 +190,7 @@ constexpr size_t persist_x_smem() {
 }
 template <typename R, int TC, int FAM>
 constexpr size_t persist_push_smem(int n_in) {
-  return (TC ? kTcTail : 0) +
-         (size_t)(n_in + 1) * kPersistThreads * (FAM ? 12 : (TC ? 16 : 8)) * sizeof(typename Types<R>::C);
+  return (TC ? kTcTail : 0) + (size_t)(n_in + 1) * kPersistThreads * (FAM ? 12 : 16) * sizeof(typename Types<R>::C);
 }
 
 }  // namespace psatd

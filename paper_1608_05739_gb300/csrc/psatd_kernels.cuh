@@ -106,7 +106,7 @@ __global__ void k_nonfinite(NfPtrs ptrs, const int64_t* __restrict__ off, int64_
 }
 
 // Threads per CTA a transposing pass of length L may use (the register budget
-// of 24 elements per thread halves it for the mixed lengths).
+// of 20 or 24 elements per thread halves it).
 template <typename R, int L>
 struct RowThreads { static constexpr int value = RowEPT<L>::value >= 20 ? 256 : sizeof(R) == 4 ? 512 : 256; };
 
@@ -188,48 +188,50 @@ __device__ __forceinline__ void fwd_T_body(const LineIO& io, const typename Type
   block_fft_fwd<R, L, EPT, TC>(v, ex, tw, t, &tc);
 
   if constexpr (R2C) {
-    // X[k] = Fe[k] + W_N^k Fo[k], Fe = (Z[k] + Z*[L-k])/2, Fo = (Z[k] - Z*[L-k])/(2i), k = 0..L,
-    // computed straight into the transposed store: Z of row g goes to this line's buffer
-    // (XOR-ed by a row-dependent mask so that the column-wise reads hit distinct banks),
-    // then each thread produces whole output elements (k, row) and stores them.
+    // X[k] = Fe + W Fo, X[L-k] = conj(Fe - W Fo), Fe = (Z[k] + Z*[L-k])/2, Fo = (Z[k] - Z*[L-k])/(2i),
+    // W = W_2L^k, computed straight into the transposed store: Z of row g goes to this line's
+    // buffer (XOR-ed by a row-dependent mask so that the column-wise reads hit distinct banks),
+    // then each thread produces whole output elements (k, row) and (L - k, row) and stores them.
     C* zb = ex.next();
     const int xg = row_xor(g, log_tb, L);  // stays inside the line for L < 16
 #pragma unroll
     for (int m = 0; m < EPT; ++m) zb[(t + T * m) ^ xg] = v[m];
     __syncthreads();
-    // Thread (k0, gg) produces bins k = k0 + j T, j < EPT (all below L), and thread
-    // k0 = 0 also bin L; twiddles are loaded in groups of four before their use.
-    const typename Types<R>::W* wn = tw + P::kTwEntries;  // W_N^k, N = 2L
+    // Thread (k0, gg) takes the bins k = k0 + j T < L/2 with L - k, and thread k0 = 0 also
+    // L/2; twiddles are loaded in groups of four (or two) before their use.
+    const typename Types<R>::W* wn = tw + P::kTwEntries;  // W_2L^k
     const int tid = g * T + t;
     const int gg = tid & (TB - 1);
     const int k0 = tid >> log_tb;  // in [0, T)
     const int xgg = row_xor(gg, log_tb, L);
     const C* zr = smem + gg * L;
-    C* o = static_cast<C*>(io.out[a1]) + a0 * out_sa0 + b0 + (int64_t)k0 * out_sk + gg;
-    const int64_t ostep = (int64_t)T * out_sk;
+    C* o = static_cast<C*>(io.out[a1]) + a0 * out_sa0 + b0 + gg;
+    auto split = [&](C zk, C zm, typename Types<R>::W w, C& fe, C& wo) {
+      fe = mkc(R(0.5) * (zk.x + zm.x), R(0.5) * (zk.y - zm.y));
+      wo = twmul(mkc(R(0.5) * (zk.y + zm.y), R(0.5) * (zm.x - zk.x)), w);
+    };
+    constexpr int NP = EPT / 2, GP = NP % 4 == 0 ? 4 : 2;
     if (!PART || gg < rows) {
 #pragma unroll
-    for (int j0 = 0; j0 < EPT; j0 += 4) {
-      typename Types<R>::W w[4];
+      for (int j0 = 0; j0 < NP; j0 += GP) {
+        typename Types<R>::W w[GP];
 #pragma unroll
-      for (int j = 0; j < 4; ++j) w[j] = __ldg(&wn[k0 + (j0 + j) * T]);
+        for (int j = 0; j < GP; ++j) w[j] = __ldg(&wn[k0 + (j0 + j) * T]);
 #pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const int k = k0 + (j0 + j) * T;
-        const C zk = zr[k ^ xgg];
-        const C zm = cconj(zr[(is_pow2(L) ? ((L - k) & (L - 1)) : (k == 0 ? 0 : L - k)) ^ xgg]);
-        const C fe = mkc(R(0.5) * (zk.x + zm.x), R(0.5) * (zk.y + zm.y));
-        const C fo = mkc(R(0.5) * (zk.y - zm.y), R(-0.5) * (zk.x - zm.x));
-        o[(j0 + j) * ostep] = cadd(fe, twmul(fo, w[j]));
+        for (int j = 0; j < GP; ++j) {
+          const int k = k0 + (j0 + j) * T;
+          C fe, wo;
+          split(zr[k ^ xgg], zr[(k == 0 ? 0 : L - k) ^ xgg], w[j], fe, wo);
+          o[(int64_t)k * out_sk] = cadd(fe, wo);
+          o[(int64_t)(L - k) * out_sk] = mkc(fe.x - wo.x, wo.y - fe.y);
+        }
       }
-    }
-    if (k0 == 0) {  // k = L: X[L] = Fe[0] - Fo[0]
-      const C z0 = zr[0 ^ xgg];
-      const C zm = cconj(z0);
-      const C fe = mkc(R(0.5) * (z0.x + zm.x), R(0.5) * (z0.y + zm.y));
-      const C fo = mkc(R(0.5) * (z0.y - zm.y), R(-0.5) * (z0.x - zm.x));
-      o[EPT * ostep] = csub(fe, fo);
-    }
+      if (k0 == 0) {
+        const C z = zr[(L / 2) ^ xgg];
+        C fe, wo;
+        split(z, z, __ldg(&wn[L / 2]), fe, wo);
+        o[(int64_t)(L / 2) * out_sk] = cadd(fe, wo);
+      }
     }
   } else {
     C* tile = smem;  // [NK][TB + 1], aliases the exchange buffers
@@ -1024,7 +1026,7 @@ __device__ __forceinline__ void line_push_body(const PushArgs<R>& a_in, const ty
 
 // Block (T, lines per CTA, component groups); the group variant (GRP) takes up
 // to 512 threads (the tensor-core pairs 256), the plain pass 256 (or T).
-template <typename R, int L, int LAYOUT, int TC = 0, int EPT = PushEPT<L, TC>::value, bool GRP = false>
+template <typename R, int L, int LAYOUT, int TC, int EPT, bool GRP>
 __global__ void __launch_bounds__(GRP ? 512 : (FFTPlan<L, EPT>::kT > 256 ? FFTPlan<L, EPT>::kT : 256))
 k_line_push(PushArgs<R> a, const typename Types<R>::W* __restrict__ tw) {
   extern __shared__ __align__(16) unsigned char smem_raw[];

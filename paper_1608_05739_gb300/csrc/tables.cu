@@ -35,11 +35,11 @@ struct Radices {
 static Radices plan_radices(int L, int ept) {
   Radices R{};
   auto lg = [](int v) { int k = 0; while ((1 << k) < v) ++k; return k; };
-  if (L & (L - 1)) {  // 3 * 2^k: radix 3, (2|4), 8, ... (ept 24) or radix 12, (2), 4, ... (ept 12);
-                      // 5 * 2^k: radix 5, (2), 4, ... (ept 20)
-    const int f = L % 3 == 0 ? 3 : 5;
-    const int head = (f == 3 && ept == 12) ? 2 : 0, b = (f == 5 || ept == 12) ? 2 : 3;
-    const int k = lg(L / f) - head, rem = k % b;
+  if (L & (L - 1)) {  // the odd factor times 2^head, (2), then radix 4 or 8
+    const int f = L % 3 == 0 ? 3 : 5, k0 = lg(L / f);
+    const int b = (f == 5 || ept == 12) ? 2 : 3;
+    const int head = ept == 12 ? 2 : f == 5 ? (k0 % 2 ? 1 : 2) : k0 % 3;
+    const int k = k0 - head, rem = k % b;
     R.r[R.n++] = f << head;
     if (rem) R.r[R.n++] = 1 << rem;
     for (int i = 0; i < k / b; ++i) R.r[R.n++] = 1 << b;
