@@ -252,7 +252,7 @@ psatd_status psatd_plan_get_launch(psatd_plan plan, int32_t cfg[6]);
  * line buffers within the device's shared memory.  -1: the built-in choice, in FP32
  * the fewest of 1, 2 and 4 groups that fill the SMs' registers with warps (long lines
  * of many components, launches of few lines; it also takes blocks of several short
- * lines in groups), else 1.  Results
+ * lines in groups), in FP64 2, 3 or 6 for launches of few lines, else 1.  Results
  * are bitwise the same for every G (each transform and each mode's update
  * runs the same arithmetic).  set: INVALID_ARG when the shape is not valid
  * for the plan's current lines per CTA and elements per thread (a later

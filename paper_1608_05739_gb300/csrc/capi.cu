@@ -286,44 +286,31 @@ psatd_status alloc(psatd_plan p, void** ptr, size_t bytes, const char* what) {
 }
 
 // threads per CTA a transposing pass may launch (the kernels' launch bounds)
-int row_maxthr(int L, bool f32) { return row_ept(L) >= 20 || !f32 ? 256 : 512; }
-// lines per CTA for a transposing pass of length L over `nb` lines (a divisor
-// of nb; at most 16 lines: the row-dependent XOR of the transposed store
-// spreads 16 lines over the banks, 32 would read one bank twice; the
-// tensor-core variant goes to 32 where it needs that for 128 threads)
-int pick_log_tb_raw(int L, int64_t nb, bool f32, bool tc) {
-  const int T = L / row_ept(L);
-  const int maxthr = row_maxthr(L, f32);
-  int tb = 1;
-  while (tb * 2 * T <= maxthr && tb * 2 <= 16 && nb % (tb * 2) == 0) tb *= 2;
-  if (tc)
-    while (tb * T < 128 && tb * 2 * T <= maxthr && tb * 2 <= 32 && nb % (tb * 2) == 0) tb *= 2;
+int row_maxthr(int L, bool f32) { return !f32 ? 4096 / row_ept(L, false) : row_ept(L, true) >= 20 ? 256 : 512; }
+// Rows per CTA of a tensor-core transposing pass over `nb` rows: a divisor of nb, at most
+// 16 rows (the row-dependent XOR of the transposed store spreads 16 rows over the banks,
+// 32 would read one bank twice), up to 32 where that is needed for 128 threads.  Inverse:
+// half of that (measured faster: the gathered bin pairs of fewer rows per CTA), keeping
+// the 128 threads.
+int pick_log_tb_tc(int L, int64_t nb, bool fwd) {
+  const int T = L / row_ept(L, true), maxthr = row_maxthr(L, true);
   int lg = 0;
-  while ((1 << lg) < tb) ++lg;
+  while ((T << (lg + 1)) <= maxthr && lg < 4 && nb % (2 << lg) == 0) ++lg;
+  while ((T << lg) < 128 && (T << (lg + 1)) <= maxthr && lg < 5 && nb % (2 << lg) == 0) ++lg;
+  if (!fwd && lg > 0 && (T << (lg - 1)) >= 128) --lg;
   return lg;
 }
-// lines per CTA of a forward transposing pass: as above; for the x rows (R2C,
-// `rows`) at most 8 where a line's threads are whole warps (T a multiple of 32):
-// the lines then synchronise only their own warps between stages (named barriers
-// 1..8), measured faster than 16 lines on one CTA-wide barrier (1024^2 x: 23.0 ->
-// 21.0 us).  The C2C y pass keeps 16 (its tile store writes 128-byte runs of z;
-// 8 lines measured slower at 512 x 512 x 1024: 5.01 -> 5.42 ms).
-int pick_log_tb(int L, int64_t nb, bool f32, bool tc = false, bool rows = false) {
-  const int lg = pick_log_tb_raw(L, nb, f32, tc);
-  const int T = L / row_ept(L);
-  return (rows && !tc && T % 32 == 0 && lg > 3) ? 3 : lg;
-}
-// lines per CTA of an inverse transposing pass: half the forward rule's value
-// before the cap above (the autotuner measured that faster at 2048^2 x, 1024^2 x,
-// 256^3 x and y: the gathered bin pairs of fewer lines per CTA), keeping the
-// tensor-core minimum
-int pick_log_tb_inv_raw(int L, int64_t nb, bool f32, bool tc) {
-  const int lg = pick_log_tb_raw(L, nb, f32, tc);
-  const int T = L / row_ept(L);
-  if (lg == 0 || (tc && (T << (lg - 1)) < 128)) return lg;
-  return lg - 1;
-}
 constexpr int kSMs = 152;  // GB300
+// Rows per CTA of an FP64 transposing pass: up to 512 threads and 16 rows (runs of the
+// transposed store), down to one row while the launch has under two CTAs per SM (the
+// FP64 units of every SM are the bound).
+int pick_log_tb_f64(int L, int64_t nb, int64_t planes) {
+  const int T = L / row_ept(L, false), maxthr = std::min(row_maxthr(L, false), 512);
+  int lg = 0;
+  while ((T << (lg + 1)) <= maxthr && lg < 4 && nb % (2 << lg) == 0) ++lg;
+  while (lg > 0 && (nb >> lg) * planes < 2 * kSMs) --lg;
+  return lg;
+}
 // Rows per CTA of a row-pair pass (FP32 without tensor cores; pair_rows.cuh) over `nb`
 // rows of each of `planes` planes and components.  Forward: at most 16 rows and 256
 // threads (T rows-pairs' threads), 8 rows where a line is whole warps; inverse: half the
@@ -331,7 +318,7 @@ constexpr int kSMs = 152;  // GB300
 // 124 / 137 us).  Fewer while the launch has under two CTAs per SM: there a pass lasts as
 // long as one CTA, and rows on idle SMs cost nothing.
 int pick_log_tb_pairs(int L, int64_t nb, int64_t planes, bool fwd, bool rows) {
-  const int T = L / row_ept(L);
+  const int T = L / row_ept(L, true);
   const int maxthr = fwd ? row_maxthr(L, true) : std::min(row_maxthr(L, true), 256);
   const int cap = T <= 4 ? 32 : (fwd && rows && T % 32 == 0) ? 8 : 16;
   int lg = 0;
@@ -346,11 +333,10 @@ int rows_per_cta(psatd_plan p, int k) {
   const bool x = k == 0 || k == 3, fwd = k < 2;
   const int L = (int)(x ? p->nx / 2 : p->ny);
   const int64_t nb = x ? p->ny : p->nz;
-  if (p->f32 && !p->tc) {
-    const int64_t planes = (p->ndim == 3 ? (x ? p->nz : p->nxh) : p->npatch) * (fwd ? p->n_in : p->n_out);
-    return pick_log_tb_pairs(L, nb, planes, fwd, x);
-  }
-  return fwd ? pick_log_tb(L, nb, p->f32, p->tc, x) : pick_log_tb_inv_raw(L, nb, p->f32, p->tc);
+  const int64_t planes = (p->ndim == 3 ? (x ? p->nz : p->nxh) : p->npatch) * (fwd ? p->n_in : p->n_out);
+  if (!p->f32) return pick_log_tb_f64(L, nb, planes);
+  if (!p->tc) return pick_log_tb_pairs(L, nb, planes, fwd, x);
+  return pick_log_tb_tc(L, nb, fwd);
 }
 
 // shared memory of a transposing pass: one L-element buffer per line, or the
@@ -375,6 +361,8 @@ int push_lines_per_cta(int L, int64_t nlines, bool tc, bool f32, int ept) {
   if (tc)
     while (tb * T < 128) tb *= 2;
   if (f32 && !tc && T == 32 && nlines >= 8 * kSMs) tb = 2;
+  if (!f32)
+    while (tb > 1 && nlines < 2 * kSMs * tb) tb /= 2;  // a line on every SM comes first
   return tb;
 }
 
@@ -404,15 +392,23 @@ size_t push_smem(int n_in, int L, int tb, int G, size_t csz, bool tc = false) {
 int push_units_of(int layout, int n_in) {
   return layout == PSATD_FIELDS_2D_TM ? n_in - 1 : (layout == PSATD_FIELDS_2D_TE ? n_in + 1 : n_in == 6 ? 6 : n_in + 1) / 2;
 }
-// The built-in choice (FP32 without tensor cores; one group elsewhere): the fewest
+// The built-in choice (one group with tensor cores).  FP32: the fewest
 // groups (1, 2 or 4, no more than needed for one per unit) that give an SM 14 resident warps (of the 16 that the
 // registers allow) and the launch 256 threads per SM.  Measured with 1 / 2 / 4 groups:
 // 2048-point lines of five components 85.2 / 73.1 / 87.8 us; 1024 points, eleven
 // components 1.350 / 1.026 / 0.884 ms; 512 points, eleven components 0.421 / 0.383 /
 // 0.486 ms; 257 lines of 512 points 12.2 / 11.6 / 11.2 us.  Groups are whole warps.
+// FP64: 2, 3 or 6 groups while the launch has under 256 threads per SM (a warp's FP64
+// instruction takes 64 cycles: a small launch's time is the instructions of a thread).
 int push_groups_default(int layout, int L, int ept, int tb, int n_in, int64_t nlines, bool tc, bool f32, int sm_bytes) {
-  if (tc || !f32 || L < ept || sm_bytes <= 0) return 1;
+  if (tc || L < ept || sm_bytes <= 0) return 1;
   const int T = L / ept, thr = T * tb;
+  if (!f32) {
+    int G = 1;
+    for (int c : {2, 3, 6})
+      if (c <= n_in && thr * c <= 512 && nlines * T * G < 256 * kSMs) G = c;
+    return G;
+  }
   if (thr % 32) return 1;
   const int ctas = std::max(1, (int)((size_t)sm_bytes / ((size_t)n_in * tb * L * 8 + 1024)));  // + the reservation
   const int units = push_units_of(layout, n_in);
@@ -596,7 +592,7 @@ psatd_status run_step(psatd_plan p, const void* in[kMaxComp], void* out[kMaxComp
     PassGeom g;
     g.log_tb = rows_per_cta(p, 0);
     g.grid = dim3((unsigned)(ny >> g.log_tb), (unsigned)na0, (unsigned)p->n_in);
-    g.smem = tail + tpass_smem(Lx, g.log_tb, 0, csz) + tc_a3_bytes(p, (Lx / row_ept(Lx)) << g.log_tb);
+    g.smem = tail + tpass_smem(Lx, g.log_tb, 0, csz) + tc_a3_bytes(p, (Lx / row_ept(Lx, p->f32)) << g.log_tb);
     for (int c = 0; c < p->n_in; ++c) {
       io.in[c] = in[c];
       io.out[c] = s1 + c * cs;
@@ -617,7 +613,7 @@ psatd_status run_step(psatd_plan p, const void* in[kMaxComp], void* out[kMaxComp
     g.log_tb = rows_per_cta(p, 1);
     g.grid = dim3((unsigned)(nz >> g.log_tb), (unsigned)nxh, (unsigned)p->n_in);
     g.smem = tail + tpass_smem((int)ny, g.log_tb, (size_t)ny, csz) +
-             tc_a3_bytes(p, ((int)ny / row_ept((int)ny)) << g.log_tb);
+             tc_a3_bytes(p, ((int)ny / row_ept((int)ny, p->f32)) << g.log_tb);
     for (int c = 0; c < p->n_in; ++c) {
       io.in[c] = s1 + c * cs;
       io.out[c] = s2 + c * cs;
@@ -651,7 +647,7 @@ psatd_status run_step(psatd_plan p, const void* in[kMaxComp], void* out[kMaxComp
     g.log_tb = rows_per_cta(p, 2);
     g.grid = dim3((unsigned)(nz >> g.log_tb), (unsigned)nxh, (unsigned)p->n_out);
     g.smem = tail + tpass_smem((int)ny, g.log_tb, (size_t)ny, csz) +
-             tc_a3_bytes(p, ((int)ny / row_ept((int)ny)) << g.log_tb);
+             tc_a3_bytes(p, ((int)ny / row_ept((int)ny, p->f32)) << g.log_tb);
     for (int c = 0; c < p->n_out; ++c) {
       io.in[c] = s2 + c * cs;
       io.out[c] = s1 + c * cs;
@@ -667,7 +663,7 @@ psatd_status run_step(psatd_plan p, const void* in[kMaxComp], void* out[kMaxComp
     PassGeom g;
     g.log_tb = rows_per_cta(p, 3);
     g.grid = dim3((unsigned)(ny >> g.log_tb), (unsigned)na0, (unsigned)p->n_out);
-    g.smem = tail + tpass_smem(Lx, g.log_tb, 0, csz) + tc_a3_bytes(p, (Lx / row_ept(Lx)) << g.log_tb);
+    g.smem = tail + tpass_smem(Lx, g.log_tb, 0, csz) + tc_a3_bytes(p, (Lx / row_ept(Lx, p->f32)) << g.log_tb);
     for (int c = 0; c < p->n_out; ++c) {
       io.in[c] = s1 + c * cs;
       io.out[c] = out[c];
@@ -703,8 +699,8 @@ psatd_status check_tc_shape(psatd_plan p, int maxsm) {
     return fail(nullptr, PSATD_ERR_UNSUPPORTED, "mixed precision needs nx >= 32 and ny, nz >= 16");
   struct { int L; int64_t nb; } rows[2] = {{Lx, p->ny}, {(int)p->ny, p->nz}};
   for (int i = 0; i < (p->ndim == 3 ? 2 : 1); ++i) {
-    const int T = rows[i].L / row_ept(rows[i].L);
-    if ((T << pick_log_tb(rows[i].L, rows[i].nb, true, true)) < 128)
+    const int T = rows[i].L / row_ept(rows[i].L, true);
+    if ((T << pick_log_tb_tc(rows[i].L, rows[i].nb, true)) < 128)
       return fail(nullptr, PSATD_ERR_UNSUPPORTED,
                   "mixed precision: a line pass of length %d over %lld lines has fewer than 128 threads per CTA",
                   rows[i].L, (long long)rows[i].nb);
@@ -793,7 +789,7 @@ TuneSpace tune_space(psatd_plan p) {
   for (int k = 0; k < 4; ++k) {
     ts.rowL[k] = rowL[k];
     if (!rowOn[k]) continue;
-    const int T = rowL[k] / row_ept(rowL[k]);
+    const int T = rowL[k] / row_ept(rowL[k], p->f32);
     const int maxthr = row_maxthr(rowL[k], p->f32);
     for (int lg = 0; (1 << lg) <= 32 && rowNb[k] % (1 << lg) == 0 && (T << lg) <= maxthr; ++lg) {
       if (p->tc && (T << lg) < 128) continue;
@@ -1080,7 +1076,7 @@ psatd_status psatd_coeffs_init(psatd_plan p) {
     for (int i = 0; i < p->ndim; ++i) {
       const int L = i == 0 ? (int)(ns[0] / 2) : (int)ns[i];
       const bool push_axis = (i == p->ndim - 1) && i > 0;
-      e = launch_twiddles(p->tw[i], L, push_axis ? p->push_ept : row_ept(L), i == 0, p->f32, p->st);
+      e = launch_twiddles(p->tw[i], L, push_axis ? p->push_ept : row_ept(L, p->f32), i == 0, p->f32, p->st);
       if (e != cudaSuccess) return cuda_fail(p, e, "twiddle table launch");
     }
     if (p->tc) {
@@ -1545,7 +1541,7 @@ extern "C" psatd_status psatd_step_noalloc(const psatd_desc* desc, const psatd_f
   for (int i = 0; i < p.ndim; ++i) {
     const int L = i == 0 ? (int)(ns[0] / 2) : (int)ns[i];
     const bool push_axis = (i == p.ndim - 1) && i > 0;
-    e = launch_twiddles(p.tw[i], L, push_axis ? p.push_ept : row_ept(L), i == 0, p.f32, p.st);
+    e = launch_twiddles(p.tw[i], L, push_axis ? p.push_ept : row_ept(L, p.f32), i == 0, p.f32, p.st);
     if (e != cudaSuccess) return cuda_fail(nullptr, e, "twiddle table launch");
   }
   const double N = (double)p.nx * (double)p.ny * (double)p.nz;
@@ -1645,7 +1641,7 @@ bool persist_y_len(int L, bool tc) {
 }
 int fam_of(int L) { return pow2(L) ? 0 : 1; }
 // rows per item of a transposing pass and lines per item of the fused pass
-int persist_x_tb(int L) { return kPersistXThreads / (L / row_ept(L)); }
+int persist_x_tb(int L) { return kPersistXThreads / (L / row_ept(L, true)); }
 int persist_y_tb(int L, bool tc) { return kPersistThreads / (L / push_ept(L, tc, true)); }
 
 // X-pass arguments of class plan p for the step's field / source pointers (as

@@ -13,15 +13,27 @@
 // lie in one warp (T <= 32, a power of two), else the named barrier `bar`.
 #pragma once
 
+#include <type_traits>
+
 #include "fft_core.cuh"
 
 namespace psatd {
 
-template <int T>
+// SUB: several lines of a warp may run apart (FP64, whose groups need not be whole
+// warps): only the line's own lanes meet.  The block's x dimension is T, so that a line's
+// lanes are an aligned run of T.
+template <int T, bool SUB = false>
 __device__ __forceinline__ void line_sync(int bar) {
   static_assert((T & (T - 1)) == 0, "a line's threads must not straddle warps");
-  if constexpr (T <= 32) __syncwarp();
-  else asm volatile("bar.sync %0, %1;" ::"r"(bar), "n"(T) : "memory");
+  if constexpr (T > 32) {
+    asm volatile("bar.sync %0, %1;" ::"r"(bar), "n"(T) : "memory");
+  } else if constexpr (SUB && T < 32) {
+    unsigned lane;
+    asm volatile("mov.u32 %0, %%laneid;" : "=r"(lane));
+    __syncwarp(((1u << T) - 1u) << (lane & ~(unsigned)(T - 1)));
+  } else {
+    __syncwarp();
+  }
 }
 
 // Position of element i in the exchange buffer that stage S writes.  8-byte
@@ -82,14 +94,14 @@ __device__ __forceinline__ void line_load_tw(W (&w)[PFCount<L, EPT>::value], con
 // exchange barrier (in registers to spare); else each stage loads its own.
 template <class V, int L, int EPT, bool PF, int S>
 __device__ __forceinline__ void line_fwd_stage(typename Types<V>::C (&v)[EPT], typename Types<V>::C* buf,
-                                               const float4* __restrict__ tw, int t, int gx, int bar,
-                                               float4 (&w)[PFCount<L, EPT>::value]) {
+                                               const typename Types<V>::W* __restrict__ tw, int t, int gx, int bar,
+                                               typename Types<V>::W (&w)[PFCount<L, EPT>::value]) {
   typedef typename Types<V>::C C;
   typedef FFTPlan<L, EPT> P;
   typedef ExPos<P, S, (int)sizeof(C)> X;
   constexpr int RS = P::radix(S), NS = P::span(S), Q = EPT / RS, T = P::kT;
   constexpr bool LAST = (S == P::kStages - 1);
-  if constexpr (!LAST) line_sync<T>(bar);  // the buffer's earlier reads are done
+  if constexpr (!LAST) line_sync<T, std::is_same<V, double>::value>(bar);  // the buffer's earlier reads are done
   if constexpr (!PF) line_load_tw<L, EPT, S>(w, tw, t);
 #pragma unroll
   for (int q = 0; q < Q; ++q) {
@@ -115,7 +127,7 @@ __device__ __forceinline__ void line_fwd_stage(typename Types<V>::C (&v)[EPT], t
   }
   if constexpr (!LAST) {
     if constexpr (PF) line_load_tw<L, EPT, S + 1>(w, tw, t);
-    line_sync<T>(bar);
+    line_sync<T, std::is_same<V, double>::value>(bar);
     const int pt = X::at(t, gx);
 #pragma unroll
     for (int m = 0; m < EPT; ++m) v[m] = buf[X::add(pt, t, T * m, gx)];
@@ -127,21 +139,21 @@ __device__ __forceinline__ void line_fwd_stage(typename Types<V>::C (&v)[EPT], t
 // thread touched since (the first exchange of an inverse).
 template <class V, int L, int EPT, bool PF, int S>
 __device__ __forceinline__ void line_inv_stage(typename Types<V>::C (&v)[EPT], typename Types<V>::C* buf,
-                                               const float4* __restrict__ tw, int t, int gx, int bar,
-                                               float4 (&w)[PFCount<L, EPT>::value]) {
+                                               const typename Types<V>::W* __restrict__ tw, int t, int gx, int bar,
+                                               typename Types<V>::W (&w)[PFCount<L, EPT>::value]) {
   typedef typename Types<V>::C C;
   typedef FFTPlan<L, EPT> P;
   typedef ExPos<P, S, (int)sizeof(C)> X;
   constexpr int RS = P::radix(S), NS = P::span(S), Q = EPT / RS, T = P::kT;
   constexpr bool FIRST = (S == P::kStages - 1);
   if constexpr (!FIRST) {
-    if constexpr (S < P::kStages - 2) line_sync<T>(bar);  // the previous exchange's reads are done
+    if constexpr (S < P::kStages - 2) line_sync<T, std::is_same<V, double>::value>(bar);  // the previous exchange's reads are done
     const int pt = X::at(t, gx);
 #pragma unroll
     for (int m = 0; m < EPT; ++m) buf[X::add(pt, t, T * m, gx)] = v[m];
   }
   if constexpr (PF) line_load_tw<L, EPT, S>(w, tw, t);
-  if constexpr (!FIRST) line_sync<T>(bar);
+  if constexpr (!FIRST) line_sync<T, std::is_same<V, double>::value>(bar);
 #pragma unroll
   for (int q = 0; q < Q; ++q) {
     const int j = t + q * T;
@@ -171,17 +183,17 @@ __device__ __forceinline__ void line_inv_stage(typename Types<V>::C (&v)[EPT], t
 
 template <class V, int L, int EPT, bool PF, int... S>
 __device__ __forceinline__ void line_fwd_seq(typename Types<V>::C (&v)[EPT], typename Types<V>::C* buf,
-                                             const float4* __restrict__ tw, int t, int gx, int bar,
+                                             const typename Types<V>::W* __restrict__ tw, int t, int gx, int bar,
                                              std::integer_sequence<int, S...>) {
-  float4 w[PFCount<L, EPT>::value];
+  typename Types<V>::W w[PFCount<L, EPT>::value];
   if constexpr (PF) line_load_tw<L, EPT, 1>(w, tw, t);
   (line_fwd_stage<V, L, EPT, PF, S>(v, buf, tw, t, gx, bar, w), ...);
 }
 template <class V, int L, int EPT, bool PF, int... S>
 __device__ __forceinline__ void line_inv_seq(typename Types<V>::C (&v)[EPT], typename Types<V>::C* buf,
-                                             const float4* __restrict__ tw, int t, int gx, int bar,
+                                             const typename Types<V>::W* __restrict__ tw, int t, int gx, int bar,
                                              std::integer_sequence<int, S...>) {
-  float4 w[PFCount<L, EPT>::value];
+  typename Types<V>::W w[PFCount<L, EPT>::value];
   (line_inv_stage<V, L, EPT, PF, FFTPlan<L, EPT>::kStages - 1 - S>(v, buf, tw, t, gx, bar, w), ...);
 }
 
@@ -189,14 +201,14 @@ __device__ __forceinline__ void line_inv_seq(typename Types<V>::C (&v)[EPT], typ
 // be read by other threads of the line on entry, and is on exit.
 template <class V, int L, int EPT, bool PF>
 __device__ __forceinline__ void line_fft_fwd(typename Types<V>::C (&v)[EPT], typename Types<V>::C* buf,
-                                             const float4* __restrict__ tw, int t, int gx, int bar) {
+                                             const typename Types<V>::W* __restrict__ tw, int t, int gx, int bar) {
   line_fwd_seq<V, L, EPT, PF>(v, buf, tw, t, gx, bar, std::make_integer_sequence<int, FFTPlan<L, EPT>::kStages>{});
 }
 // Unnormalised inverse (adjoint).  On entry no other thread may still touch this
 // thread's own positions ExPos<P, kStages - 2>::at(t + T m).
 template <class V, int L, int EPT, bool PF>
 __device__ __forceinline__ void line_fft_inv(typename Types<V>::C (&v)[EPT], typename Types<V>::C* buf,
-                                             const float4* __restrict__ tw, int t, int gx, int bar) {
+                                             const typename Types<V>::W* __restrict__ tw, int t, int gx, int bar) {
   line_inv_seq<V, L, EPT, PF>(v, buf, tw, t, gx, bar, std::make_integer_sequence<int, FFTPlan<L, EPT>::kStages>{});
 }
 

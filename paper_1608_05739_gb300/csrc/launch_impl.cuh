@@ -24,7 +24,7 @@ template <typename R, int TC, int L, bool R2C>
 static cudaError_t fwd_T_L_k(const PassGeom& g, cudaStream_t st, const LineIO& io, const void* tw, int64_t a, int64_t b,
                            int64_t c, int64_t d, const int64_t* off) {
   typedef typename Types<R>::W W;
-  constexpr int T = FFTPlan<L, RowEPT<L>::value>::kT;
+  constexpr int T = FFTPlan<L, RowEPT<L, R>::value>::kT;
   cudaError_t e;
   if constexpr (kPairs<R, TC>) {
     const unsigned pairs = g.log_tb > 0 ? 1u << (g.log_tb - 1) : 1u;
@@ -51,7 +51,7 @@ template <typename R, int TC, int L, bool C2R>
 static cudaError_t inv_T_L_k(const PassGeom& g, cudaStream_t st, const LineIO& io, const void* tw, int64_t a, int64_t b,
                            int64_t c, int64_t d, const int64_t* off) {
   typedef typename Types<R>::W W;
-  constexpr int T = FFTPlan<L, RowEPT<L>::value>::kT;
+  constexpr int T = FFTPlan<L, RowEPT<L, R>::value>::kT;
   cudaError_t e;
   if constexpr (kPairs<R, TC>) {
     const unsigned pairs = g.log_tb > 0 ? 1u << (g.log_tb - 1) : 1u;
@@ -78,7 +78,7 @@ template <typename R, int TC, int EPT, int L, int LAYOUT, bool GRP>
 static auto push_kernel() {
   // radix-16 lines run in groups by default and share one kernel for any count; the others
   // keep a plain kernel, 2 to 4 % faster than the group one with a single group
-  if constexpr (kPairs<R, TC>) return k_line_pair<L, LAYOUT, EPT, GRP || EPT == 16>;
+  if constexpr (TC == 0) return k_line_pair<R, L, LAYOUT, EPT, GRP || (EPT == 16 && sizeof(R) == 4)>;
   else return k_line_push<R, L, LAYOUT, TC, EPT, GRP>;
 }
 
@@ -90,11 +90,10 @@ static cudaError_t push_L(int layout, dim3 grid, int tb, int groups, size_t smem
     return cudaErrorInvalidValue;
   } else {
     const dim3 block(FFTPlan<L, EPT>::kT, tb, groups);
-    // component groups: their own instantiation, in FP32 for blocks of whole-warp groups
-    // and for the tensor-core pairs (the host admits groups > 1 nowhere else)
-    constexpr bool kGrpOk = TC ? EPT == 16 : kPairs<R, TC>;
+    // component groups: their own instantiation; FP32 groups are whole warps
+    constexpr bool kGrpOk = TC ? EPT == 16 : true;
     if (groups > 1 && (!kGrpOk || (kPairs<R, TC> && (block.x * block.y) % 32 != 0))) return cudaErrorInvalidValue;
-    if constexpr (kPairs<R, TC>) smem = (size_t)a.n_in * tb * L * sizeof(float2);  // the units alone
+    if constexpr (TC == 0) smem = (size_t)a.n_in * tb * L * 2 * sizeof(R);  // the units alone
     cudaError_t e;
 #define PSATD_PUSH_LAUNCH(LAY, GRP)                                            \
   {                                                                            \

@@ -1,6 +1,7 @@
-// pair_push.cuh -- the FP32 fused last-axis pass (no tensor cores): as k_line_push
-// (psatd_kernels.cuh), with the components of a line transformed two at a time in
-// packed arithmetic (fft_line.cuh).
+// pair_push.cuh -- the fused last-axis pass without tensor cores: as k_line_push
+// (psatd_kernels.cuh), in FP32 with the components of a line transformed two at a time
+// in packed arithmetic (fft_line.cuh).  FP64 transforms them one at a time (every unit
+// below is a single).
 //
 // Components in slot order form units: pairs (c, c + 1) and, where a group has an
 // odd count, singles (pair_width).  A unit of a line owns one contiguous region of
@@ -16,7 +17,9 @@
 // two CTAs of 2048-point lines), then the L1 / shared-memory data pipe (49 % busy).
 // One component per thread -> pairs: 2048^2 TE 84.6 -> 73.7 us (113.5k -> 73.6k
 // wavefronts per SM, 46.9 M -> 35.0 M instructions), 256^3 with eleven components 439 ->
-// 371 us, 512 x 512 x 1024 9.47 -> 6.83 ms.
+// 371 us, 512 x 512 x 1024 9.47 -> 6.83 ms.  FP64 is bound by its units (half an operation
+// per cycle and scheduler): 128^2, six components, 97 us with two lines to a one-warp
+// CTA, 36 us with a line's components over six groups on an SM of its own.
 //
 // Component groups (GRP, G = blockDim.z): group j takes the units j, j + G, ...
 // (inverse: from G - 1 - j); the block meets before and after the push, whose
@@ -29,30 +32,32 @@
 namespace psatd {
 
 // Components of the unit that starts at slot c (slot order: psatd_kernels.cuh).
-template <int LAYOUT>
+template <typename R, int LAYOUT>
 __device__ __forceinline__ int pair_width(int c) {
-  if constexpr (LAYOUT == 2) return c == 2 ? 1 : 2;               // (E0 E1) B2 (J0 J1) (rho rho')
+  if constexpr (sizeof(R) == 8) return 1;
+  else if constexpr (LAYOUT == 2) return c == 2 ? 1 : 2;               // (E0 E1) B2 (J0 J1) (rho rho')
   else if constexpr (LAYOUT == 3) return c == 0 ? 2 : 1;          // (E2 B0) B1 J2
   else return c == 8 ? 1 : 2;                                     // (E0 E1) (E2 B0) (B1 B2) (J0 J1) J2 (rho rho')
 }
-template <int LAYOUT>
+template <typename R, int LAYOUT>
 __host__ __device__ constexpr bool pair_start(int c) {
-  return LAYOUT == 2 ? (c == 0 || c == 3 || c == 5) : LAYOUT == 3 ? c == 0 : (c == 0 || c == 2 || c == 4 || c == 6 || c == 9);
+  return sizeof(R) == 8 ? false : LAYOUT == 2 ? (c == 0 || c == 3 || c == 5) : LAYOUT == 3 ? c == 0 : (c == 0 || c == 2 || c == 4 || c == 6 || c == 9);
 }
 
 // The update of one mode whose slot values sit at p2 (pairs) and p1 (singles)
 // within the units of this line; us: stride of one component over the block's
 // lines, g1 / g2: this line's offset in a single's / pair's unit (bytes).
-template <int LAYOUT, bool PSTD>
+template <typename R, int LAYOUT, bool PSTD>
 __device__ __forceinline__ void push_units(unsigned char* base, int us, int g1, int g2, int p1, int p2,
-                                           const CoefReg<float>& f, float mx, float my, float mz,
-                                           const PushArgs<float>& a, const float4* P) {
-  const float2 Z = make_float2(0.f, 0.f);
+                                           const CoefReg<R>& f, R mx, R my, R mz,
+                                           const PushArgs<R>& a, const typename Types<R>::W* P) {
+  typedef typename Types<R>::C C;
+  const C Z = mkc(R(0), R(0));
   const int form = a.form;
   const int zmask = a.ndim == 3 ? 7 : 3;
   constexpr int NF = LAYOUT >= 2 ? 3 : 6, NJ = LAYOUT == 2 ? 2 : LAYOUT == 3 ? 1 : 3;
-  float2 s[kMaxComp];
-  auto turn = [&](int c, float2 v, bool back) {  // staggered plans: to the true position and back
+  C s[kMaxComp];
+  auto turn = [&](int c, C v, bool back) {  // staggered plans: to the true position and back
     if (P) {
       const int m = slot_stagger<LAYOUT>(c) & zmask;
 #pragma unroll
@@ -65,20 +70,20 @@ __device__ __forceinline__ void push_units(unsigned char* base, int us, int g1, 
   for (int c = 0; c < kMaxComp; ++c) {
     if (c >= NF + NJ + (LAYOUT == 3 ? 0 : 2)) break;
     const bool on = c < NF || (c < NF + NJ ? form >= 1 : form == 2);
-    if (pair_start<LAYOUT>(c)) {
+    if (pair_start<R, LAYOUT>(c)) {
       float4 q = make_float4(0.f, 0.f, 0.f, 0.f);
       if (on) q = *reinterpret_cast<const float4*>(base + c * us + g2 + p2 * 16);
-      s[c] = on ? turn(c, make_float2(q.x, q.z), false) : Z;
-      s[c + 1] = on ? turn(c + 1, make_float2(q.y, q.w), false) : Z;
-    } else if (c == 0 || !pair_start<LAYOUT>(c - 1)) {
-      s[c] = on ? turn(c, *reinterpret_cast<const float2*>(base + c * us + g1 + p1 * 8), false) : Z;
+      s[c] = on ? turn(c, mkc(R(q.x), R(q.z)), false) : Z;
+      s[c + 1] = on ? turn(c + 1, mkc(R(q.y), R(q.w)), false) : Z;
+    } else if (c == 0 || !pair_start<R, LAYOUT>(c - 1)) {
+      s[c] = on ? turn(c, *reinterpret_cast<const C*>(base + c * us + g1 + p1 * (int)sizeof(C)), false) : Z;
     }
   }
-  float cS_h, cS_l, Sc_h, Sc_l;
+  R cS_h, cS_l, Sc_h, Sc_l;
   prod2(a.c_h, a.c_l, f.S_h, f.S_l, cS_h, cS_l);
   prod2(a.ic_h, a.ic_l, f.S_h, f.S_l, Sc_h, Sc_l);
   if constexpr (PSTD) {  // J-form or vacuum
-    float2 E[3] = {Z, Z, Z}, B[3] = {Z, Z, Z}, J[3] = {Z, Z, Z};
+    C E[3] = {Z, Z, Z}, B[3] = {Z, Z, Z}, J[3] = {Z, Z, Z};
     if constexpr (LAYOUT == 2) {
       E[0] = s[0]; E[1] = s[1]; B[2] = s[2]; J[0] = s[3]; J[1] = s[4];
     } else if constexpr (LAYOUT == 3) {
@@ -87,7 +92,7 @@ __device__ __forceinline__ void push_units(unsigned char* base, int us, int g1, 
 #pragma unroll
       for (int i = 0; i < 3; ++i) { E[i] = s[i]; B[i] = s[3 + i]; J[i] = s[6 + i]; }
     }
-    pstd_modes<float>(E, B, J, mx, my, mz, a);
+    pstd_modes<R>(E, B, J, mx, my, mz, a);
     if constexpr (LAYOUT == 2) {
       s[0] = E[0]; s[1] = E[1]; s[2] = B[2];
     } else if constexpr (LAYOUT == 3) {
@@ -97,46 +102,47 @@ __device__ __forceinline__ void push_units(unsigned char* base, int us, int g1, 
       for (int i = 0; i < 3; ++i) { s[i] = E[i]; s[3 + i] = B[i]; }
     }
   } else if constexpr (LAYOUT == 2) {
-    push_te<float>(s[0], s[1], s[2], s[3], s[4], s[5], s[6], mx, my, f, cS_h, cS_l, Sc_h, Sc_l, a, form);
+    push_te<R>(s[0], s[1], s[2], s[3], s[4], s[5], s[6], mx, my, f, cS_h, cS_l, Sc_h, Sc_l, a, form);
   } else if constexpr (LAYOUT == 3) {
-    push_tm<float>(s[0], s[1], s[2], s[3], mx, my, f, cS_h, cS_l, Sc_h, Sc_l, a, form);
+    push_tm<R>(s[0], s[1], s[2], s[3], mx, my, f, cS_h, cS_l, Sc_h, Sc_l, a, form);
   } else if constexpr (LAYOUT == 1) {
-    push_te<float>(s[0], s[1], s[5], s[6], s[7], s[9], s[10], mx, my, f, cS_h, cS_l, Sc_h, Sc_l, a, form);
-    push_tm<float>(s[2], s[3], s[4], s[8], mx, my, f, cS_h, cS_l, Sc_h, Sc_l, a, form);
+    push_te<R>(s[0], s[1], s[5], s[6], s[7], s[9], s[10], mx, my, f, cS_h, cS_l, Sc_h, Sc_l, a, form);
+    push_tm<R>(s[2], s[3], s[4], s[8], mx, my, f, cS_h, cS_l, Sc_h, Sc_l, a, form);
   } else {
-    float2 E[3] = {s[0], s[1], s[2]}, B[3] = {s[3], s[4], s[5]};
-    const float2 J[3] = {s[6], s[7], s[8]};
-    push_3d<float>(E, B, J, s[9], s[10], mx, my, mz, f, cS_h, cS_l, Sc_h, Sc_l, a, form);
+    C E[3] = {s[0], s[1], s[2]}, B[3] = {s[3], s[4], s[5]};
+    const C J[3] = {s[6], s[7], s[8]};
+    push_3d<R>(E, B, J, s[9], s[10], mx, my, mz, f, cS_h, cS_l, Sc_h, Sc_l, a, form);
 #pragma unroll
     for (int i = 0; i < 3; ++i) { s[i] = E[i]; s[3 + i] = B[i]; }
   }
 #pragma unroll
   for (int c = 0; c < NF; ++c) {
-    if (pair_start<LAYOUT>(c)) {
-      const float2 u = turn(c, s[c], true), w = turn(c + 1, s[c + 1], true);
-      *reinterpret_cast<float4*>(base + c * us + g2 + p2 * 16) = make_float4(u.x, w.x, u.y, w.y);
-    } else if (c == 0 || !pair_start<LAYOUT>(c - 1)) {
-      *reinterpret_cast<float2*>(base + c * us + g1 + p1 * 8) = turn(c, s[c], true);
+    if (pair_start<R, LAYOUT>(c)) {
+      const C u = turn(c, s[c], true), w = turn(c + 1, s[c + 1], true);
+      *reinterpret_cast<float4*>(base + c * us + g2 + p2 * 16) = make_float4((float)u.x, (float)w.x, (float)u.y, (float)w.y);
+    } else if (c == 0 || !pair_start<R, LAYOUT>(c - 1)) {
+      *reinterpret_cast<C*>(base + c * us + g1 + p1 * (int)sizeof(C)) = turn(c, s[c], true);
     }
   }
 }
 
 // The push of this thread's modes l = t + T (grp + G i) (as push_line_modes).
-template <int L, int LAYOUT, int EPT, bool STAG, bool PSTD>
+template <typename R, int L, int LAYOUT, int EPT, bool STAG, bool PSTD>
 __device__ __forceinline__ void push_line_units(unsigned char* base, int us, int g1, int g2, int gx,
-                                                const PushArgs<float>& a, const Coef<float>* trow, int t, int grp,
-                                                int G, int mxi, int myi, float kpx, float kpy, float4 phx, float4 phy) {
+                                                const PushArgs<R>& a, const Coef<R>* trow, int t, int grp,
+                                                int G, int mxi, int myi, R kpx, R kpy, typename Types<R>::W phx,
+                                                typename Types<R>::W phy) {
   typedef FFTPlan<L, EPT> P;
   constexpr int T = P::kT;
-  auto coef = [&](int l) -> Coef<float> {
+  auto coef = [&](int l) -> Coef<R> {
     if constexpr (!PSTD) return trow[(l <= L / 2) ? l : L - l];  // |m| along the line axis
-    else return Coef<float>{};
+    else return Coef<R>{};
   };
   // two modes per iteration: both loads issued together, the next two before this update
-  Coef<float> qn[2] = {coef(t + T * grp), coef(t + T * (grp + G < EPT ? grp + G : grp))};
+  Coef<R> qn[2] = {coef(t + T * grp), coef(t + T * (grp + G < EPT ? grp + G : grp))};
 #pragma unroll 1
   for (int m0 = grp; m0 < EPT; m0 += 2 * G) {
-    const Coef<float> q[2] = {qn[0], qn[1]};
+    const Coef<R> q[2] = {qn[0], qn[1]};
     const int mn = m0 + 2 * G;
     if (mn < EPT) {
       qn[0] = coef(t + T * mn);
@@ -147,20 +153,21 @@ __device__ __forceinline__ void push_line_units(unsigned char* base, int us, int
       const int m = m0 + G * h;
       if (m >= EPT) break;
       const int l = t + T * m;
-      CoefReg<float> f;
+      CoefReg<R> f;
       f.C_h = q[h].C_h; f.C_l = q[h].C_l; f.S_h = q[h].S_h; f.S_l = q[h].S_l;
       f.A1 = q[h].A1; f.A4 = q[h].A4; f.B1 = q[h].B1; f.B2 = q[h].B2;
-      const int p1 = own_pos<L, EPT, 8>(t, m, 0), p2 = own_pos<L, EPT, 16>(t, m, gx);
-      float mx, my, mz;
+      const int p1 = own_pos<L, EPT, 2 * (int)sizeof(R)>(t, m, sizeof(R) == 8 ? gx : 0);
+      const int p2 = sizeof(R) == 8 ? 0 : own_pos<L, EPT, 16>(t, m, gx);
+      R mx, my, mz;
       if constexpr (STAG) {
         const int ml = l < L / 2 ? l : l - L;
-        float kl;
-        float4 pl;
+        R kl;
+        typename Types<R>::W pl;
         stag_axis(a, a.ndim == 2 ? 1 : 2, ml, kl, pl);
-        float4 Ph[3];
+        typename Types<R>::W Ph[3];
         Ph[0] = phx;
         if (a.ndim == 2) {
-          mx = kpx; my = kl; mz = 0.f;
+          mx = kpx; my = kl; mz = R(0);
           Ph[1] = pl;
           Ph[2] = phy;
         } else {
@@ -168,15 +175,15 @@ __device__ __forceinline__ void push_line_units(unsigned char* base, int us, int
           Ph[1] = phy;
           Ph[2] = pl;
         }
-        push_units<LAYOUT, PSTD>(base, us, g1, g2, p1, p2, f, mx, my, mz, a, Ph);
+        push_units<R, LAYOUT, PSTD>(base, us, g1, g2, p1, p2, f, mx, my, mz, a, Ph);
       } else {
         const int ml = (l == L / 2) ? 0 : (l < L / 2 ? l : l - L);
         if (a.ndim == 2) {
-          mx = a.rx * float(mxi); my = a.ry * float(ml); mz = 0.f;
+          mx = a.rx * R(mxi); my = a.ry * R(ml); mz = R(0);
         } else {
-          mx = a.rx * float(mxi); my = a.ry * float(myi); mz = a.rz * float(ml);
+          mx = a.rx * R(mxi); my = a.ry * R(myi); mz = a.rz * R(ml);
         }
-        push_units<LAYOUT, PSTD>(base, us, g1, g2, p1, p2, f, mx, my, mz, a, nullptr);
+        push_units<R, LAYOUT, PSTD>(base, us, g1, g2, p1, p2, f, mx, my, mz, a, nullptr);
       }
     }
   }
@@ -185,12 +192,15 @@ __device__ __forceinline__ void push_line_units(unsigned char* base, int us, int
 // Body of one CTA: line block bx (tb lines; line g of the block handled by the
 // threads (t, g, grp)); mbar / phase: the stage mbarrier and the parity of its
 // next phase.  Returns false when a failed index check left the phase unused.
-template <int L, int LAYOUT, int EPT, bool GRP>
-__device__ __forceinline__ bool line_pair_body(const PushArgs<float>& a_in, const float4* __restrict__ tw, int bx,
+template <typename R, int L, int LAYOUT, int EPT, bool GRP>
+__device__ __forceinline__ bool line_pair_body(const PushArgs<R>& a_in, const typename Types<R>::W* __restrict__ tw, int bx,
                                                int t, int g, int tb, int grp, int G, unsigned char* smem_raw,
                                                uint32_t mbar, uint32_t phase) {
-  const PushArgs<float> a = a_in;  // a private copy: its scalars stay in registers
+  const PushArgs<R> a = a_in;  // a private copy: its scalars stay in registers
+  typedef typename Types<R>::C C;
+  typedef typename Types<R>::W W;
   typedef FFTPlan<L, EPT> P;
+  constexpr int CS = (int)sizeof(C);
   constexpr int T = P::kT;
   // twiddles one stage ahead where a stage's fit beside two transforms' elements
   constexpr bool PF = EPT == 8 || EPT == 12;
@@ -208,24 +218,24 @@ __device__ __forceinline__ bool line_pair_body(const PushArgs<float>& a_in, cons
                      (int64_t)(row_c + 1) * a.tab_row > a.tab_ext || row_c < 0;
     if (cta_out_of_bounds(bad, a.chk_err)) return false;
   }
-  const int us = tb * L * 8;  // stride of one component over the block's lines
-  const int g1 = g * L * 8, g2 = 2 * g1;
-  const int gx = line_gx<P>(g);
+  const int us = tb * L * CS;  // stride of one component over the block's lines
+  const int g1 = g * L * CS, g2 = 2 * g1;
+  const int gx = line_gx<P>(g), gx1 = CS == 16 ? gx : 0;  // pairs', singles'
   const int bar = 1 + g * G + grp;
-  float2* spec = static_cast<float2*>(a.spec);
+  C* spec = static_cast<C*>(a.spec);
   // stage every input slot of the block's lines: one bulk copy per line and slot,
   // issued by the first warp, completing on the stage mbarrier; lines past the
   // last are zero-filled
   const int nv = a.nlines - line0 < tb ? a.nlines - line0 : tb;  // valid lines of the block
   if (!valid)
     for (int c = 0, w; c < a.n_in; c += w) {
-      w = pair_width<LAYOUT>(c);
+      w = pair_width<R, LAYOUT>(c);
       float4* dst = reinterpret_cast<float4*>(smem_raw + c * us + w * g1);
-      for (int i = t + grp * T; i < w * L / 2; i += G * T) dst[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+      for (int i = t + grp * T; i < w * L * CS / 16; i += G * T) dst[i] = make_float4(0.f, 0.f, 0.f, 0.f);
     }
   __syncthreads();  // the mbarrier is initialised; the zeros are visible
   if (tid < 32) {
-    constexpr uint32_t bytes = (uint32_t)(L * 8);
+    constexpr uint32_t bytes = (uint32_t)(L * CS);
     if (tid == 0) {
       fence_async_smem();
       mbar_arrive_expect_tx(mbar, (uint32_t)(nv * a.n_in) * bytes);
@@ -234,22 +244,22 @@ __device__ __forceinline__ bool line_pair_body(const PushArgs<float>& a_in, cons
     const int step = nthr < 32 ? nthr : 32;
     for (int i = tid; i < nv * a.n_in; i += step) {
       const int gl = i / a.n_in, c = i - gl * a.n_in;
-      const bool second = c > 0 && pair_start<LAYOUT>(c - 1);
+      const bool second = c > 0 && pair_start<R, LAYOUT>(c - 1);
       const int c0 = second ? c - 1 : c;
-      const int w = pair_width<LAYOUT>(c0);
-      bulk_copy_g2s(smem_u32(smem_raw + c0 * us + (gl * w + (second ? 1 : 0)) * (L * 8)),
+      const int w = pair_width<R, LAYOUT>(c0);
+      bulk_copy_g2s(smem_u32(smem_raw + c0 * us + (gl * w + (second ? 1 : 0)) * (L * CS)),
                     spec + c * a.cs + (int64_t)(line0 + gl) * L, bytes, mbar);
     }
   }
   int mxi, myi, rowi;
   line_modes(a, valid ? line : 0, mxi, myi, rowi);
-  float kpx = 0.f, kpy = 0.f;
-  float4 phx{}, phy{};
+  R kpx = R(0), kpy = R(0);
+  W phx{}, phy{};
   if (a.stag) {
     stag_axis(a, 0, mxi, kpx, phx);
     if (a.ndim == 3) stag_axis(a, 1, myi, kpy, phy);
   }
-  const Coef<float>* trow = a.tab + (int64_t)rowi * a.tab_row;
+  const Coef<R>* trow = a.tab + (int64_t)rowi * a.tab_row;
   // the push's coefficient entries: start bringing them into L2 now
 #pragma unroll
   for (int m = grp; m < EPT; m += G) {
@@ -266,73 +276,77 @@ __device__ __forceinline__ bool line_pair_body(const PushArgs<float>& a_in, cons
 
 #pragma unroll 1
   for (int c = 0, u = 0, w; c < a.n_in; c += w, ++u) {
-    w = pair_width<LAYOUT>(c);
+    w = pair_width<R, LAYOUT>(c);
     if (GRP && u % G != grp) continue;
-    if (w == 2) {
-      const float2* s0 = reinterpret_cast<const float2*>(smem_raw + c * us + g2);
-      C2* buf = reinterpret_cast<C2*>(smem_raw + c * us + g2);
-      C2 v[EPT];
+    if constexpr (sizeof(R) == 4) {
+      if (w == 2) {
+        const float2* s0 = reinterpret_cast<const float2*>(smem_raw + c * us + g2);
+        C2* buf = reinterpret_cast<C2*>(smem_raw + c * us + g2);
+        C2 v[EPT];
 #pragma unroll
-      for (int m = 0; m < EPT; ++m) {
-        const float2 x = s0[t + T * m], y = s0[L + t + T * m];
-        v[m] = C2{F2{x.x, y.x}, F2{x.y, y.y}};
+        for (int m = 0; m < EPT; ++m) {
+          const float2 x = s0[t + T * m], y = s0[L + t + T * m];
+          v[m] = C2{F2{x.x, y.x}, F2{x.y, y.y}};
+        }
+        line_fft_fwd<F2, L, EPT, PF>(v, buf, tw, t, gx, bar);
+#pragma unroll
+        for (int m = 0; m < EPT; ++m) buf[own_pos<L, EPT, 16>(t, m, gx)] = v[m];
+        continue;
       }
-      line_fft_fwd<F2, L, EPT, PF>(v, buf, tw, t, gx, bar);
-#pragma unroll
-      for (int m = 0; m < EPT; ++m) buf[own_pos<L, EPT, 16>(t, m, gx)] = v[m];
-    } else {
-      float2* buf = reinterpret_cast<float2*>(smem_raw + c * us + g1);
-      float2 v[EPT];
-#pragma unroll
-      for (int m = 0; m < EPT; ++m) v[m] = buf[t + T * m];
-      line_fft_fwd<float, L, EPT, PF>(v, buf, tw, t, 0, bar);
-#pragma unroll
-      for (int m = 0; m < EPT; ++m) buf[own_pos<L, EPT, 8>(t, m, 0)] = v[m];
     }
+    C* buf = reinterpret_cast<C*>(smem_raw + c * us + g1);
+    C v[EPT];
+#pragma unroll
+    for (int m = 0; m < EPT; ++m) v[m] = buf[t + T * m];
+    line_fft_fwd<R, L, EPT, PF>(v, buf, tw, t, gx1, bar);
+#pragma unroll
+    for (int m = 0; m < EPT; ++m) buf[own_pos<L, EPT, CS>(t, m, gx1)] = v[m];
   }
   if (G > 1) __syncthreads();  // every group's spectra are in their units
 
   if (a.scheme == 0) {
     if (a.stag)
-      push_line_units<L, LAYOUT, EPT, true, false>(smem_raw, us, g1, g2, gx, a, trow, t, grp, G, mxi, myi, kpx, kpy, phx, phy);
+      push_line_units<R, L, LAYOUT, EPT, true, false>(smem_raw, us, g1, g2, gx, a, trow, t, grp, G, mxi, myi, kpx, kpy, phx, phy);
     else
-      push_line_units<L, LAYOUT, EPT, false, false>(smem_raw, us, g1, g2, gx, a, trow, t, grp, G, mxi, myi, kpx, kpy, phx, phy);
+      push_line_units<R, L, LAYOUT, EPT, false, false>(smem_raw, us, g1, g2, gx, a, trow, t, grp, G, mxi, myi, kpx, kpy, phx, phy);
   } else {
     if (a.stag)
-      push_line_units<L, LAYOUT, EPT, true, true>(smem_raw, us, g1, g2, gx, a, trow, t, grp, G, mxi, myi, kpx, kpy, phx, phy);
+      push_line_units<R, L, LAYOUT, EPT, true, true>(smem_raw, us, g1, g2, gx, a, trow, t, grp, G, mxi, myi, kpx, kpy, phx, phy);
     else
-      push_line_units<L, LAYOUT, EPT, false, true>(smem_raw, us, g1, g2, gx, a, trow, t, grp, G, mxi, myi, kpx, kpy, phx, phy);
+      push_line_units<R, L, LAYOUT, EPT, false, true>(smem_raw, us, g1, g2, gx, a, trow, t, grp, G, mxi, myi, kpx, kpy, phx, phy);
   }
   if (G > 1) __syncthreads();  // every mode is pushed
 
 #pragma unroll 1
   for (int c = 0, u = 0, w; c < a.n_out; c += w, ++u) {
-    w = pair_width<LAYOUT>(c);
+    w = pair_width<R, LAYOUT>(c);
     if (GRP && u % G != G - 1 - grp) continue;
-    float2* dst = spec + c * a.cs + (int64_t)line * L;
-    if (w == 2) {
-      C2* buf = reinterpret_cast<C2*>(smem_raw + c * us + g2);
-      C2 v[EPT];
+    C* dst = spec + c * a.cs + (int64_t)line * L;
+    if constexpr (sizeof(R) == 4) {
+      if (w == 2) {
+        C2* buf = reinterpret_cast<C2*>(smem_raw + c * us + g2);
+        C2 v[EPT];
 #pragma unroll
-      for (int m = 0; m < EPT; ++m) v[m] = buf[own_pos<L, EPT, 16>(t, m, gx)];
-      line_fft_inv<F2, L, EPT, PF>(v, buf, tw, t, gx, bar);
-      if (valid) {
+        for (int m = 0; m < EPT; ++m) v[m] = buf[own_pos<L, EPT, 16>(t, m, gx)];
+        line_fft_inv<F2, L, EPT, PF>(v, buf, tw, t, gx, bar);
+        if (valid) {
 #pragma unroll
-        for (int m = 0; m < EPT; ++m) {
-          dst[t + T * m] = make_float2(v[m].x.a, v[m].y.a);
-          dst[a.cs + t + T * m] = make_float2(v[m].x.b, v[m].y.b);
+          for (int m = 0; m < EPT; ++m) {
+            dst[t + T * m] = make_float2(v[m].x.a, v[m].y.a);
+            dst[a.cs + t + T * m] = make_float2(v[m].x.b, v[m].y.b);
+          }
         }
+        continue;
       }
-    } else {
-      float2* buf = reinterpret_cast<float2*>(smem_raw + c * us + g1);
-      float2 v[EPT];
+    }
+    C* buf = reinterpret_cast<C*>(smem_raw + c * us + g1);
+    C v[EPT];
 #pragma unroll
-      for (int m = 0; m < EPT; ++m) v[m] = buf[own_pos<L, EPT, 8>(t, m, 0)];
-      line_fft_inv<float, L, EPT, PF>(v, buf, tw, t, 0, bar);
-      if (valid) {
+    for (int m = 0; m < EPT; ++m) v[m] = buf[own_pos<L, EPT, CS>(t, m, gx1)];
+    line_fft_inv<R, L, EPT, PF>(v, buf, tw, t, gx1, bar);
+    if (valid) {
 #pragma unroll
-        for (int m = 0; m < EPT; ++m) dst[t + T * m] = make_float2(v[m].x, v[m].y);
-      }
+      for (int m = 0; m < EPT; ++m) dst[t + T * m] = v[m];
     }
   }
   return true;
@@ -341,14 +355,14 @@ __device__ __forceinline__ bool line_pair_body(const PushArgs<float>& a_in, cons
 // Block (T, lines per CTA, component groups); up to 512 threads (128 registers), or 256
 // without groups (GRP false).  Groups are whole warps: with several, T times the lines
 // per CTA is a multiple of 32.
-template <int L, int LAYOUT, int EPT, bool GRP>
+template <typename R, int L, int LAYOUT, int EPT, bool GRP>
 __global__ void __launch_bounds__(GRP ? 512 : 256)
-k_line_pair(PushArgs<float> a, const float4* __restrict__ tw) {
+k_line_pair(PushArgs<R> a, const typename Types<R>::W* __restrict__ tw) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ __align__(8) uint64_t stage_mbar;
   const uint32_t mbar = smem_u32(&stage_mbar);
   if (threadIdx.x == 0 && threadIdx.y == 0 && threadIdx.z == 0) mbar_init(mbar, 1);
-  line_pair_body<L, LAYOUT, EPT, GRP>(a, tw, (int)blockIdx.x, (int)threadIdx.x, (int)threadIdx.y, (int)blockDim.y,
+  line_pair_body<R, L, LAYOUT, EPT, GRP>(a, tw, (int)blockIdx.x, (int)threadIdx.x, (int)threadIdx.y, (int)blockDim.y,
                                       (int)threadIdx.z, (int)blockDim.z, smem_raw, mbar, 0u);
 }
 

@@ -166,7 +166,7 @@ __global__ void __launch_bounds__(kPersistThreads, TC ? 2 : 4) k_persist_push(co
       line_push_body<R, LL, LAYOUT, TC, EPT>(A, tw, it.blk, t, g, kPersistThreads / T, 0, 1, smem_raw, tc, sc); \
     } else {                                                                                               \
       __syncthreads(); /* the previous item's shared memory is free */                                     \
-      if (line_pair_body<LL, LAYOUT, EPT, false>(A, tw, it.blk, t, g, kPersistThreads / T, 0, 1, smem_raw, sc.mbar, \
+      if (line_pair_body<R, LL, LAYOUT, EPT, false>(A, tw, it.blk, t, g, kPersistThreads / T, 0, 1, smem_raw, sc.mbar, \
                                                  sc.phase))                                                 \
         sc.phase ^= 1u;                                                                                    \
     }                                                                                                      \

@@ -106,9 +106,11 @@ __global__ void k_nonfinite(NfPtrs ptrs, const int64_t* __restrict__ off, int64_
 }
 
 // Threads per CTA a transposing pass of length L may use (the register budget
-// of 20 or 24 elements per thread halves it).
+// of 20 or 24 elements per thread halves it; FP64: 4096 elements).
 template <typename R, int L>
-struct RowThreads { static constexpr int value = RowEPT<L>::value >= 20 ? 256 : sizeof(R) == 4 ? 512 : 256; };
+struct RowThreads {
+  static constexpr int value = sizeof(R) == 8 ? 4096 / RowEPT<L, R>::value : RowEPT<L, R>::value >= 20 ? 256 : 512;
+};
 
 // XOR mask of row r's buffer in the transposed stores and reads (TB = 1 << log_tb
 // rows): rows spread over the 16 eight-byte bank pairs (at most 16 rows: one row
@@ -139,7 +141,7 @@ __device__ __forceinline__ void fwd_T_body(const LineIO& io, const typename Type
                                            const int64_t* __restrict__ in_off, const RowCta& cta,
                                            unsigned char* smem_raw, TcCtx& tc) {
   typedef typename Types<R>::C C;
-  constexpr int EPT = RowEPT<L>::value;
+  constexpr int EPT = RowEPT<L, R>::value;
   typedef FFTPlan<L, EPT> P;
   constexpr int T = P::kT;
   constexpr int NK = R2C ? L + 1 : L;
@@ -253,7 +255,7 @@ __device__ __forceinline__ void fwd_T_body(const LineIO& io, const typename Type
 // thread).  The tensor-core variants then keep part of each row on the stack,
 // but measured faster so than with 128 registers and half the resident warps.
 template <typename R, int L, bool R2C, int TC = 0>
-__global__ void __launch_bounds__(RowThreads<R, L>::value, 2) k_fwd_T(LineIO io, const typename Types<R>::W* __restrict__ tw,
+__global__ void __launch_bounds__(RowThreads<R, L>::value, sizeof(R) == 8 ? 1 : 2) k_fwd_T(LineIO io, const typename Types<R>::W* __restrict__ tw,
                                                int64_t in_sa0, int64_t in_sb, int64_t out_sa0,
                                                int64_t out_sk, int log_tb, const int64_t* __restrict__ in_off) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -276,7 +278,7 @@ __device__ __forceinline__ void inv_T_body(const LineIO& io, const typename Type
                                            const int64_t* __restrict__ out_off, const RowCta& cta,
                                            unsigned char* smem_raw, TcCtx& tc) {
   typedef typename Types<R>::C C;
-  constexpr int EPT = RowEPT<L>::value;
+  constexpr int EPT = RowEPT<L, R>::value;
   typedef FFTPlan<L, EPT> P;
   constexpr int T = P::kT;
   constexpr int NK = C2R ? L + 1 : L;
@@ -398,7 +400,7 @@ __device__ __forceinline__ void inv_T_body(const LineIO& io, const typename Type
 }
 
 template <typename R, int L, bool C2R, int TC = 0>
-__global__ void __launch_bounds__(RowThreads<R, L>::value, 2) k_inv_T(LineIO io, const typename Types<R>::W* __restrict__ tw,
+__global__ void __launch_bounds__(RowThreads<R, L>::value, sizeof(R) == 8 ? 1 : 2) k_inv_T(LineIO io, const typename Types<R>::W* __restrict__ tw,
                                                int64_t in_sa0, int64_t in_sk, int64_t out_sa0,
                                                int64_t out_sb, int log_tb, const int64_t* __restrict__ out_off) {
   extern __shared__ __align__(16) unsigned char smem_raw[];

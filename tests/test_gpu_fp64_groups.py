@@ -1,0 +1,39 @@
+"""FP64 passes at the edges of their split: lines of one thread to many, single lines per
+block in component groups that are not whole warps (2, 3 or 6 groups by component count),
+blocks of several lines, the longest lines.  One step against the FP64 oracle at the FP64
+bound (1e-12), and the built-in shape against one group and one line per CTA, bitwise (the
+split changes no operation)."""
+import numpy as np
+import pytest
+
+from gpu_helpers import ensure_lib, mask_layout, psatd_gpu, rel_l2_fields
+from oracle import psatd as orc
+from paper_1608_05739_gb300 import capi, synth
+
+pytestmark = pytest.mark.gpu
+
+CASES = [
+    ((8, 16), "te", "J"), ((16, 32), "2d6", "rho"), ((32, 64), "tm", "none"), ((128, 128), "2d6", "none"),
+    ((64, 256), "te", "rho"), ((128, 1024), "te", "J"), ((8, 8, 16), "3d6", "J"), ((16, 64, 32), "3d6", "rho"),
+    ((16, 4096), "tm", "J"), ((2048, 32), "te", "none"),
+]
+
+
+@pytest.mark.parametrize("shape,layout,src", CASES)
+def test_fp64_split(shape, layout, src):
+    ensure_lib()
+    d, dt = (1.0, 0.9, 1.1)[:len(shape)], 0.4
+    E = mask_layout(synth.random_fields(shape, 3, 81), layout, "E")
+    B = mask_layout(synth.random_fields(shape, 3, 82), layout, "B")
+    J = mask_layout(synth.random_fields(shape, 3, 83), layout, "J")
+    r0, r1 = (synth.random_fields(shape, 1, s)[0] for s in (84, 85))
+    Eo, Bo = orc.psatd_step(E, B, J if src != "none" else None, r0 if src == "rho" else None,
+                            r1 if src == "rho" else None, d=d, dt=dt, form=src)
+    plan = capi.Plan(tuple(reversed(shape)), d, dt, layout=layout, prec="fp64", src=src)
+    Eg, Bg = psatd_gpu(shape, d, dt, E, B, J, r0, r1, layout=layout, prec="fp64", src=src, plan=plan)
+    assert rel_l2_fields(Eg, Bg, mask_layout(Eo, layout, "E"), mask_layout(Bo, layout, "B")) < 1e-12
+    plan.set_launch([0, -1 if len(shape) == 2 else 0, -1 if len(shape) == 2 else 0, 0, 1, -1])
+    plan.set_push_groups(1)
+    E1, B1 = psatd_gpu(shape, d, dt, E, B, J, r0, r1, layout=layout, prec="fp64", src=src, plan=plan)
+    assert np.array_equal(E1, Eg) and np.array_equal(B1, Bg)
+    plan.destroy()
