@@ -404,8 +404,8 @@ psatd_status psatd_batch_destroy(psatd_batch batch);
  * global: layout 2D6, TE or TM; precision, source form, cell sizes, dt, c and
  * eps0 as in psatd_plan_create; n[0], n[1] need not be powers of two, but the
  * extended sizes ix + 2 guard and iy + 2 guard must satisfy psatd_plan_create's
- * limits.  Owns a plan of the extended size (px*py patches) and the packed
- * patch arrays (n_in * px*py * (ix+2g) * (iy+2g) values).
+ * limits.  Owns a plan of the extended size (px*py patches); the patches' cells
+ * are read from and written to the global arrays, never stored.
  * Errors: INVALID_ARG (NULL, px/py not dividing the grid, guard < 0),
  * UNSUPPORTED (3D, extended sizes out of range), OOM, CUDA.                 */
 typedef struct psatd_local_s* psatd_local;
@@ -413,9 +413,10 @@ psatd_status psatd_local_create(const psatd_desc* global, int32_t px, int32_t py
                                 void* cuda_stream, psatd_local* out);
 
 /* Advance the global fields by nsteps local-FFT steps (sources held constant;
- * arrays as for psatd_step, of the global size).  Per step: guard refresh of
- * the fields (sources once per call), the batched patch step, write-back of the
- * interiors.  Asynchronous.  Errors as psatd_step.                           */
+ * arrays as for psatd_step, of the global size).  Per step: the batched patch
+ * step, whose first pass reads every extended patch's rows from the global
+ * arrays (the guard refresh) and whose last writes the interiors back.
+ * Asynchronous.  Errors as psatd_step.                                      */
 psatd_status psatd_local_step(psatd_local local, const psatd_fields* fields,
                               const psatd_sources* sources, int32_t nsteps);
 

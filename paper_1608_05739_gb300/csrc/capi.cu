@@ -19,7 +19,6 @@
 
 #include "farfield.h"
 #include "launch.h"
-#include "local.h"
 #include "tables.h"
 
 using namespace psatd;
@@ -86,6 +85,7 @@ struct psatd_plan_s {
   void* gmat = nullptr;       // their split DFT matrices (kTcTail image, device)
   int* d_err = nullptr;       // device error word of the tensor-core passes
   int64_t caller_elems = 0;   // elements of each caller array (checked mode's extents)
+  LocalMap loc = {};          // psatd_local_step: the caller's arrays are the global grid's (px = 0: off)
 };
 
 namespace {
@@ -580,7 +580,8 @@ psatd_status run_step(psatd_plan p, const void* in[kMaxComp], void* out[kMaxComp
   // test hook reports each array one element shorter than it is)
   const bool chk = (p->d.flags & PSATD_FLAG_CHECKED) != 0;
   const int64_t shrink = (p->d.flags & PSATD_FLAG_TEST_SHORT_EXTENT) ? 1 : 0;
-  const int64_t ext_user = chk ? p->caller_elems - shrink : 0, ext_spec = chk ? cs - shrink : 0;
+  const int64_t user_elems = p->loc.px ? (int64_t)p->loc.nx * p->loc.ny : p->caller_elems;
+  const int64_t ext_user = chk ? user_elems - shrink : 0, ext_spec = chk ? cs - shrink : 0;
   io.chk_err = p->d_err;
   const size_t tail = TC ? (size_t)kTcTail : 0;  // tensor-core passes: matrices + mbarrier first
 
@@ -599,6 +600,7 @@ psatd_status run_step(psatd_plan p, const void* in[kMaxComp], void* out[kMaxComp
     }
     io.in_ext = ext_user;
     io.out_ext = ext_spec;
+    io.loc = p->loc;
     TimedLaunch tl(p, K_FWD_X);
     e = fwd_T_any<R, TC>(Lx, true, g, p->st, io, p->tw[0], d3 ? ny * nx : 0, nx, d3 ? ny : nxh * ny, nz * ny,
                         d3 ? nullptr : p->d_off);
@@ -683,8 +685,9 @@ psatd_status step_once(psatd_plan p, const void* in[kMaxComp], void* out[kMaxCom
   if (p->tc) s = p->tc_bf16 ? run_step<float, 2>(p, in, out) : run_step<float, 1>(p, in, out);
   else s = p->f32 ? run_step<float, 0>(p, in, out) : run_step<double, 0>(p, in, out);
   if (s == PSATD_OK && (p->d.flags & PSATD_FLAG_CHECKED)) {
-    cudaError_t e = launch_nonfinite(p->f32, out, p->n_out, p->d_off, p->npatch, p->nx * p->ny * p->nz, p->d_err,
-                                     p->st);
+    const bool loc = p->loc.px != 0;
+    cudaError_t e = launch_nonfinite(p->f32, out, p->n_out, loc ? nullptr : p->d_off, loc ? 1 : p->npatch,
+                                     loc ? (int64_t)p->loc.nx * p->loc.ny : p->nx * p->ny * p->nz, p->d_err, p->st);
     if (e != cudaSuccess) return cuda_fail(p, e, "non-finite scan launch");
   }
   return s;
@@ -2170,8 +2173,6 @@ struct psatd_local_s {
   cudaStream_t st = nullptr;
   int px = 1, py = 1, g = 0;
   int64_t nx = 0, ny = 0;
-  void* fbuf = nullptr;       // packed extended patches, one array per input slot
-  size_t comp_bytes = 0;
 };
 
 extern "C" psatd_status psatd_local_create(const psatd_desc* global, int32_t px, int32_t py, int32_t guard,
@@ -2214,13 +2215,10 @@ extern "C" psatd_status psatd_local_create(const psatd_desc* global, int32_t px,
       cudaError_t e = cudaMemcpy(p->d_off, offs.data(), offs.size() * sizeof(int64_t), cudaMemcpyHostToDevice);
       if (e != cudaSuccess) s = cuda_fail(p, e, "patch offset upload");
     }
-    L->comp_bytes = (size_t)npatch * pd.n[0] * pd.n[1] * (p->f32 ? 4 : 8);
-    if (s == PSATD_OK) s = alloc(p, &L->fbuf, (size_t)p->n_in * L->comp_bytes, "patch fields");
     if (s == PSATD_OK) s = psatd_coeffs_init(p);
     if (s != PSATD_OK) g_err = p->err;
   }
   if (s != PSATD_OK) {
-    if (L->fbuf) cudaFree(L->fbuf);
     if (p) {
       release(p);
       delete p;
@@ -2242,35 +2240,11 @@ extern "C" psatd_status psatd_local_step(psatd_local L, const psatd_fields* fiel
   void* out[kMaxComp] = {};
   psatd_status s = gather_slots(p, fields, sources, in, out);
   if (s != PSATD_OK) return s;
-  const void* pin[kMaxComp] = {};
-  void* pout[kMaxComp] = {};
-  for (int c = 0; c < p->n_in; ++c) {
-    pin[c] = static_cast<char*>(L->fbuf) + c * L->comp_bytes;
-    if (c < p->n_out) pout[c] = const_cast<void*>(pin[c]);
-  }
-  LocalComps fc{}, sc{};
-  for (int c = 0; c < p->n_out; ++c) {
-    fc.global[c] = in[c];
-    fc.global_out[c] = out[c];
-    fc.patch[c] = pout[c];
-  }
-  for (int c = p->n_out; c < p->n_in; ++c) {
-    sc.global[c - p->n_out] = in[c];
-    sc.patch[c - p->n_out] = const_cast<void*>(pin[c]);
-  }
-  cudaError_t e;
-  if (p->n_in > p->n_out) {  // sources: held constant over the call, refreshed once
-    e = launch_guard_gather(p->f32, sc, p->n_in - p->n_out, L->nx, L->ny, L->px, L->py, L->g, p->st);
-    if (e != cudaSuccess) return cuda_fail(p, e, "guard gather (sources)");
-  }
-  for (int i = 0; i < nsteps; ++i) {
-    e = launch_guard_gather(p->f32, fc, p->n_out, L->nx, L->ny, L->px, L->py, L->g, p->st);
-    if (e != cudaSuccess) return cuda_fail(p, e, "guard gather");
-    if ((s = step_once(p, pin, pout)) != PSATD_OK) return s;
-    e = launch_guard_scatter(p->f32, fc, p->n_out, L->nx, L->ny, L->px, L->py, L->g, p->st);
-    if (e != cudaSuccess) return cuda_fail(p, e, "guard scatter");
-  }
-  return PSATD_OK;
+  // the x passes read the guard cells from, and write the interiors to, the global arrays
+  p->loc = LocalMap{L->px, L->g, (int)(L->nx / L->px), (int)(L->ny / L->py), (int)L->nx, (int)L->ny};
+  for (int i = 0; i < nsteps && s == PSATD_OK; ++i) s = step_once(p, in, out);
+  p->loc = LocalMap{};
+  return s;
 }
 
 extern "C" psatd_plan psatd_local_plan(psatd_local L) { return L ? L->plan : nullptr; }
@@ -2278,7 +2252,6 @@ extern "C" psatd_plan psatd_local_plan(psatd_local L) { return L ? L->plan : nul
 extern "C" psatd_status psatd_local_destroy(psatd_local L) {
   if (!L) return PSATD_OK;
   cudaStreamSynchronize(L->st);
-  if (L->fbuf) cudaFree(L->fbuf);
   if (L->plan) {
     release(L->plan);
     delete L->plan;

@@ -20,7 +20,7 @@ static cudaError_t set_smem(K kern, size_t smem) {
   return cudaSuccess;
 }
 
-template <typename R, int TC, int L, bool R2C>
+template <typename R, int TC, int L, bool R2C, bool LOC>
 static cudaError_t fwd_T_L_k(const PassGeom& g, cudaStream_t st, const LineIO& io, const void* tw, int64_t a, int64_t b,
                            int64_t c, int64_t d, const int64_t* off) {
   typedef typename Types<R>::W W;
@@ -29,11 +29,11 @@ static cudaError_t fwd_T_L_k(const PassGeom& g, cudaStream_t st, const LineIO& i
   if constexpr (kPairs<R, TC>) {
     const unsigned pairs = g.log_tb > 0 ? 1u << (g.log_tb - 1) : 1u;
     const size_t smem = (size_t)pairs * L * sizeof(C2);
-    auto kern = k_fwd_P<L, R2C>;
+    auto kern = k_fwd_P<L, R2C, LOC>;
     if ((e = set_smem(kern, smem)) != cudaSuccess) return e;
     kern<<<g.grid, dim3(T, pairs), smem, st>>>(io, static_cast<const W*>(tw), a, b, c, d, g.log_tb, off);
   } else {
-    auto kern = k_fwd_T<R, L, R2C, TC>;
+    auto kern = k_fwd_T<R, L, R2C, TC, LOC>;
     if ((e = set_smem(kern, g.smem)) != cudaSuccess) return e;
     kern<<<g.grid, dim3(T, 1u << g.log_tb), g.smem, st>>>(io, static_cast<const W*>(tw), a, b, c, d, g.log_tb, off);
   }
@@ -42,12 +42,14 @@ static cudaError_t fwd_T_L_k(const PassGeom& g, cudaStream_t st, const LineIO& i
 template <typename R, int TC, int L>
 static cudaError_t fwd_T_L(bool r2c, const PassGeom& g, cudaStream_t st, const LineIO& io,
                            const void* tw, int64_t a, int64_t b, int64_t c, int64_t d, const int64_t* off) {
-  if (!r2c) return fwd_T_L_k<R, TC, L, false>(g, st, io, tw, a, b, c, d, off);
-  if constexpr (L <= 2048) return fwd_T_L_k<R, TC, L, true>(g, st, io, tw, a, b, c, d, off);
+  if (!r2c) return fwd_T_L_k<R, TC, L, false, false>(g, st, io, tw, a, b, c, d, off);
+  if constexpr (L <= 2048)
+    return io.loc.px ? fwd_T_L_k<R, TC, L, true, true>(g, st, io, tw, a, b, c, d, off)
+                     : fwd_T_L_k<R, TC, L, true, false>(g, st, io, tw, a, b, c, d, off);
   else return cudaErrorInvalidValue;
 }
 
-template <typename R, int TC, int L, bool C2R>
+template <typename R, int TC, int L, bool C2R, bool LOC>
 static cudaError_t inv_T_L_k(const PassGeom& g, cudaStream_t st, const LineIO& io, const void* tw, int64_t a, int64_t b,
                            int64_t c, int64_t d, const int64_t* off) {
   typedef typename Types<R>::W W;
@@ -56,11 +58,11 @@ static cudaError_t inv_T_L_k(const PassGeom& g, cudaStream_t st, const LineIO& i
   if constexpr (kPairs<R, TC>) {
     const unsigned pairs = g.log_tb > 0 ? 1u << (g.log_tb - 1) : 1u;
     const size_t smem = (size_t)pairs * L * sizeof(C2);
-    auto kern = k_inv_P<L, C2R>;
+    auto kern = k_inv_P<L, C2R, LOC>;
     if ((e = set_smem(kern, smem)) != cudaSuccess) return e;
     kern<<<g.grid, dim3(T, pairs), smem, st>>>(io, static_cast<const W*>(tw), a, b, c, d, g.log_tb, off);
   } else {
-    auto kern = k_inv_T<R, L, C2R, TC>;
+    auto kern = k_inv_T<R, L, C2R, TC, LOC>;
     if ((e = set_smem(kern, g.smem)) != cudaSuccess) return e;
     kern<<<g.grid, dim3(T, 1u << g.log_tb), g.smem, st>>>(io, static_cast<const W*>(tw), a, b, c, d, g.log_tb, off);
   }
@@ -69,8 +71,10 @@ static cudaError_t inv_T_L_k(const PassGeom& g, cudaStream_t st, const LineIO& i
 template <typename R, int TC, int L>
 static cudaError_t inv_T_L(bool c2r, const PassGeom& g, cudaStream_t st, const LineIO& io,
                            const void* tw, int64_t a, int64_t b, int64_t c, int64_t d, const int64_t* off) {
-  if (!c2r) return inv_T_L_k<R, TC, L, false>(g, st, io, tw, a, b, c, d, off);
-  if constexpr (L <= 2048) return inv_T_L_k<R, TC, L, true>(g, st, io, tw, a, b, c, d, off);
+  if (!c2r) return inv_T_L_k<R, TC, L, false, false>(g, st, io, tw, a, b, c, d, off);
+  if constexpr (L <= 2048)
+    return io.loc.px ? inv_T_L_k<R, TC, L, true, true>(g, st, io, tw, a, b, c, d, off)
+                     : inv_T_L_k<R, TC, L, true, false>(g, st, io, tw, a, b, c, d, off);
   else return cudaErrorInvalidValue;
 }
 

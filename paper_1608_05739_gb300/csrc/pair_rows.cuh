@@ -50,7 +50,7 @@ __device__ __forceinline__ C2 get_rows(const float2* p, bool two) {
   return mkpair(v, v);
 }
 
-template <int L, bool R2C>
+template <int L, bool R2C, bool LOC = false>
 __global__ void __launch_bounds__(RowPairThreads<L>::value, RowEPT<L>::value >= 20 ? 3 : 2)
 k_fwd_P(LineIO io, const float4* __restrict__ tw, int64_t in_sa0, int64_t in_sb, int64_t out_sa0, int64_t out_sk,
         int log_tb, const int64_t* __restrict__ in_off) {
@@ -66,14 +66,23 @@ k_fwd_P(LineIO io, const float4* __restrict__ tw, int64_t in_sa0, int64_t in_sb,
   const int a0 = blockIdx.y, a1 = blockIdx.z;
   const int64_t b0 = (int64_t)blockIdx.x << log_tb;
   const int64_t b = b0 + 2 * g;  // the pair's rows b, b + 1
-  const int64_t o0 = in_off ? in_off[a0] : a0 * in_sa0;  // per-patch offsets of a batch
+  const int64_t o0 = LOC ? 0 : in_off ? in_off[a0] : a0 * in_sa0;  // per-patch offsets of a batch
   if (io.in_ext) {  // checked mode: the rows read and the transposed block written
-    const int64_t in_end = o0 + (b + (two ? 1 : 0)) * in_sb + (R2C ? 2 * L : L);
+    int64_t in_end = o0 + (b + (two ? 1 : 0)) * in_sb + (R2C ? 2 * L : L);
+    if constexpr (LOC)
+      in_end = (int64_t)(max(LocalRow(io.loc, a0, (int)b).y, LocalRow(io.loc, a0, (int)b + (two ? 1 : 0)).y) + 1) * io.loc.nx;
     const int64_t out_end = a0 * out_sa0 + b0 + (1 << log_tb) + (int64_t)(NK - 1) * out_sk;
     if (cta_out_of_bounds(in_end > io.in_ext || out_end > io.out_ext || o0 < 0, io.chk_err)) return;
   }
   C2 v[EPT];
-  {
+  if constexpr (LOC) {
+    const LocalRow l0(io.loc, a0, (int)b), l1(io.loc, a0, (int)b + (two ? 1 : 0));
+    const float* p = static_cast<const float*>(io.in[a1]);
+    const float *r0 = p + (int64_t)l0.y * io.loc.nx, *r1 = p + (int64_t)l1.y * io.loc.nx;
+#pragma unroll
+    for (int m = 0; m < EPT; ++m)
+      v[m] = mkpair(local_load(r0, io.loc, l0.x0, 2 * (t + T * m)), local_load(r1, io.loc, l0.x0, 2 * (t + T * m)));
+  } else {
     const float2 *r0, *r1;
     if constexpr (R2C) {
       const float* p = static_cast<const float*>(io.in[a1]) + o0 + b * in_sb;
@@ -145,7 +154,7 @@ k_fwd_P(LineIO io, const float4* __restrict__ tw, int64_t in_sa0, int64_t in_sb,
   }
 }
 
-template <int L, bool C2R>
+template <int L, bool C2R, bool LOC = false>
 __global__ void __launch_bounds__(RowPairThreads<L>::value, RowEPT<L>::value >= 20 ? 3 : 2)
 k_inv_P(LineIO io, const float4* __restrict__ tw, int64_t in_sa0, int64_t in_sk, int64_t out_sa0, int64_t out_sb,
         int log_tb, const int64_t* __restrict__ out_off) {
@@ -161,10 +170,15 @@ k_inv_P(LineIO io, const float4* __restrict__ tw, int64_t in_sa0, int64_t in_sk,
   const int a0 = blockIdx.y, a1 = blockIdx.z;
   const int64_t b0 = (int64_t)blockIdx.x << log_tb;
   const int64_t b = b0 + 2 * g;
-  const int64_t o0 = out_off ? out_off[a0] : a0 * out_sa0;
+  const int64_t o0 = LOC ? 0 : out_off ? out_off[a0] : a0 * out_sa0;
   if (io.in_ext) {  // checked mode: the transposed block read and the rows written
     const int64_t in_end = a0 * in_sa0 + b0 + (1 << log_tb) + (int64_t)(NK - 1) * in_sk;
-    const int64_t out_end = o0 + (b + (two ? 1 : 0)) * out_sb + (C2R ? 2 * L : L);
+    int64_t out_end = o0 + (b + (two ? 1 : 0)) * out_sb + (C2R ? 2 * L : L);
+    if constexpr (LOC) {
+      const int64_t e0 = local_out(io.loc, a0, (int)b), e1 = local_out(io.loc, a0, (int)b + (two ? 1 : 0));
+      out_end = e0 > e1 ? e0 : e1;
+      out_end = out_end < 0 ? 0 : out_end + io.loc.ix;
+    }
     if (cta_out_of_bounds(in_end > io.in_ext || out_end > io.out_ext || o0 < 0, io.chk_err)) return;
   }
   const int tid = g * T + t;
@@ -222,6 +236,19 @@ k_inv_P(LineIO io, const float4* __restrict__ tw, int64_t in_sa0, int64_t in_sk,
   for (int m = 0; m < EPT; ++m) v[m] = line[(t + T * m) ^ xg];
   if constexpr (P::kStages > 1) line_sync<T>(bar);  // read by the whole line before the exchanges overwrite it
   line_fft_inv<F2, L, EPT, false>(v, line, tw, t, line_gx<P>(g), bar);
+  if constexpr (LOC) {
+    const int64_t e0 = local_out(io.loc, a0, (int)b), e1 = two ? local_out(io.loc, a0, (int)b + 1) : -1;
+    float* p = static_cast<float*>(io.out[a1]) - io.loc.g;
+    if (e0 >= 0) {
+#pragma unroll
+      for (int m = 0; m < EPT; ++m) local_store(p + e0, io.loc, 2 * (t + T * m), make_float2(v[m].x.a, v[m].y.a));
+    }
+    if (e1 >= 0) {
+#pragma unroll
+      for (int m = 0; m < EPT; ++m) local_store(p + e1, io.loc, 2 * (t + T * m), make_float2(v[m].x.b, v[m].y.b));
+    }
+    return;
+  }
   float2 *r0, *r1;
   if constexpr (C2R) {
     float* p = static_cast<float*>(io.out[a1]) + o0 + b * out_sb;

@@ -21,6 +21,15 @@ namespace psatd {
 
 constexpr int kMaxComp = 11;
 
+// Patch map of a local-FFT decomposition (px = 0: off): patch (p, q) = (a0 % px, a0 / px)
+// holds at (i, j) the global cell ((p ix - g + i) mod nx, (q iy - g + j) mod ny).  The x
+// passes read the guard cells' global cells themselves and write the interiors, so the
+// patches are never stored (with copies of the patches around the step, 3840 x 1920 cells
+// in 16 x 8 patches of 240^2 + 8 took 713 us a step, without 223).
+struct LocalMap {
+  int px, g, ix, iy, nx, ny;
+};
+
 // Per-component base pointers of a pass (index = grid z = component slot).
 struct LineIO {
   const void* in[kMaxComp];
@@ -32,6 +41,7 @@ struct LineIO {
   // (0: unchecked) and the error word that a failed index check sets
   int64_t in_ext, out_ext;
   int* chk_err;
+  LocalMap loc;      // x passes of a local decomposition
 };
 
 // k-space coefficient table entry (one per |m|-octant point), see tables.cu.
@@ -119,6 +129,46 @@ __device__ __forceinline__ int row_xor(int r, int log_tb, int L) {
   return (log_tb <= 4 ? r * (16 >> log_tb) : r) & 15 & (L - 1);
 }
 
+// Row b of patch a0 in the global grid: its cell 0 is column x0 of row y (guard rows
+// and columns wrap).
+struct LocalRow {
+  int x0, y;
+  __device__ __forceinline__ LocalRow(const LocalMap& m, int a0, int b) {
+    const int p = a0 % m.px, q = a0 / m.px;
+    y = (q * m.iy - m.g + b) % m.ny;
+    y += y < 0 ? m.ny : 0;
+    x0 = (p * m.ix - m.g) % m.nx;
+    x0 += x0 < 0 ? m.nx : 0;
+  }
+};
+// Cells e, e + 1 (e even) of a guarded row; global rows have an even length, so the pair
+// is one aligned access where the guard is even.
+template <typename R>
+__device__ __forceinline__ typename Types<R>::C local_load(const R* row, const LocalMap& m, int x0, int e) {
+  typedef typename Types<R>::C C;
+  int x = x0 + e;
+  while (x >= m.nx) x -= m.nx;
+  if (!(m.g & 1)) return *reinterpret_cast<const C*>(row + x);
+  return mkc(row[x], row[x + 1 == m.nx ? 0 : x + 1]);
+}
+// Cells e, e + 1 of interior row b (`row`: the global row's cell of the patch's column 0,
+// which lies g before the interior) back to the global grid.
+template <typename R>
+__device__ __forceinline__ void local_store(R* row, const LocalMap& m, int e, typename Types<R>::C v) {
+  typedef typename Types<R>::C C;
+  if (!(m.g & 1)) {
+    if (e >= m.g && e < m.g + m.ix) *reinterpret_cast<C*>(row + e) = v;
+  } else {
+    if (e >= m.g && e < m.g + m.ix) row[e] = v.x;
+    if (e + 1 >= m.g && e + 1 < m.g + m.ix) row[e + 1] = v.y;
+  }
+}
+// Offset of that cell, or -1 for a guard row
+__device__ __forceinline__ int64_t local_out(const LocalMap& m, int a0, int b) {
+  if (b < m.g || b >= m.g + m.iy) return -1;
+  return (int64_t)((a0 / m.px) * m.iy + b - m.g) * m.nx + (a0 % m.px) * m.ix;
+}
+
 // ---------------------------------------------------------------- pass 1 / 2
 // Forward FFT along the contiguous axis of TB consecutive lines b, written out
 // with b contiguous: out[a1] + a0*out_sa0 + k*out_sk + b.  R2C: the input rows
@@ -135,7 +185,7 @@ struct RowCta {
   int64_t nb;
 };
 
-template <typename R, int L, bool R2C, int TC, bool PART>
+template <typename R, int L, bool R2C, int TC, bool PART, bool LOC = false>
 __device__ __forceinline__ void fwd_T_body(const LineIO& io, const typename Types<R>::W* __restrict__ tw,
                                            int64_t in_sa0, int64_t in_sb, int64_t out_sa0, int64_t out_sk,
                                            const int64_t* __restrict__ in_off, const RowCta& cta,
@@ -156,8 +206,9 @@ __device__ __forceinline__ void fwd_T_body(const LineIO& io, const typename Type
   const int rows = PART ? (int)(cta.nb - b0 < TB ? cta.nb - b0 : TB) : TB;  // valid rows of the block
   const int a0 = cta.a0, a1 = cta.a1;
   if (io.in_ext) {  // checked mode: the rows read and the transposed block written
-    const int64_t o0c = in_off ? in_off[a0] : a0 * in_sa0;
-    const int64_t in_end = valid ? o0c + b * in_sb + (R2C ? 2 * L : L) : 0;
+    const int64_t o0c = LOC ? 0 : in_off ? in_off[a0] : a0 * in_sa0;
+    int64_t in_end = valid ? o0c + b * in_sb + (R2C ? 2 * L : L) : 0;
+    if constexpr (LOC) in_end = (int64_t)(LocalRow(io.loc, a0, (int)b).y + 1) * io.loc.nx;
     const int64_t out_end = a0 * out_sa0 + b0 + rows + (int64_t)(NK - 1) * out_sk;
     if (cta_out_of_bounds(in_end > io.in_ext || out_end > io.out_ext || o0c < 0, io.chk_err)) return;
   }
@@ -175,7 +226,12 @@ __device__ __forceinline__ void fwd_T_body(const LineIO& io, const typename Type
     }
 
   C v[EPT];
-  {
+  if constexpr (LOC) {
+    const LocalRow lr(io.loc, a0, (int)b);
+    const R* row = static_cast<const R*>(io.in[a1]) + (int64_t)lr.y * io.loc.nx;
+#pragma unroll
+    for (int m = 0; m < EPT; ++m) v[m] = local_load(row, io.loc, lr.x0, 2 * (t + T * m));
+  } else {
     const C* row;
     const int64_t o0 = in_off ? in_off[a0] : a0 * in_sa0;  // per-patch offsets of a batch
     if constexpr (R2C)
@@ -254,7 +310,7 @@ __device__ __forceinline__ void fwd_T_body(const LineIO& io, const typename Type
 // Launch bounds: two CTAs of the largest block per SM (at most 64 registers a
 // thread).  The tensor-core variants then keep part of each row on the stack,
 // but measured faster so than with 128 registers and half the resident warps.
-template <typename R, int L, bool R2C, int TC = 0>
+template <typename R, int L, bool R2C, int TC = 0, bool LOC = false>
 __global__ void __launch_bounds__(RowThreads<R, L>::value, sizeof(R) == 8 ? 1 : 2) k_fwd_T(LineIO io, const typename Types<R>::W* __restrict__ tw,
                                                int64_t in_sa0, int64_t in_sb, int64_t out_sa0,
                                                int64_t out_sk, int log_tb, const int64_t* __restrict__ in_off) {
@@ -263,7 +319,7 @@ __global__ void __launch_bounds__(RowThreads<R, L>::value, sizeof(R) == 8 ? 1 : 
   if constexpr (TC) tc_setup(tc, smem_raw, io.gmat, 0u, io.err, TC == 2, 0u, io.tc_ctl);
   const RowCta cta{(int)blockIdx.x, (int)blockIdx.y, (int)blockIdx.z, (int)threadIdx.x, (int)threadIdx.y, log_tb,
                    (int64_t)gridDim.x << log_tb};
-  fwd_T_body<R, L, R2C, TC, false>(io, tw, in_sa0, in_sb, out_sa0, out_sk, in_off, cta, smem_raw, tc);
+  fwd_T_body<R, L, R2C, TC, false, LOC>(io, tw, in_sa0, in_sb, out_sa0, out_sk, in_off, cta, smem_raw, tc);
   if constexpr (TC) tc_teardown(tc);
 }
 
@@ -272,7 +328,7 @@ __global__ void __launch_bounds__(RowThreads<R, L>::value, sizeof(R) == 8 ? 1 : 
 // in[a1] + a0*in_sa0 + k*in_sk + b, inverse FFT along k, write the lines
 // contiguously to out[a1] + a0*out_sa0 + b*out_sb.  C2R: L+1 Hermitian bins
 // in, real rows of length 2L out (unnormalised).
-template <typename R, int L, bool C2R, int TC, bool PART>
+template <typename R, int L, bool C2R, int TC, bool PART, bool LOC = false>
 __device__ __forceinline__ void inv_T_body(const LineIO& io, const typename Types<R>::W* __restrict__ tw,
                                            int64_t in_sa0, int64_t in_sk, int64_t out_sa0, int64_t out_sb,
                                            const int64_t* __restrict__ out_off, const RowCta& cta,
@@ -293,9 +349,13 @@ __device__ __forceinline__ void inv_T_body(const LineIO& io, const typename Type
   const int rows = PART ? (int)(cta.nb - b0 < TB ? cta.nb - b0 : TB) : TB;  // valid rows of the block
   const int a0 = cta.a0, a1 = cta.a1;
   if (io.in_ext) {  // checked mode: the transposed block read and the rows written
-    const int64_t o0c = out_off ? out_off[a0] : a0 * out_sa0;
+    const int64_t o0c = LOC ? 0 : out_off ? out_off[a0] : a0 * out_sa0;
     const int64_t in_end = a0 * in_sa0 + b0 + rows + (int64_t)(NK - 1) * in_sk;
-    const int64_t out_end = valid ? o0c + b * out_sb + (C2R ? 2 * L : L) : 0;
+    int64_t out_end = valid ? o0c + b * out_sb + (C2R ? 2 * L : L) : 0;
+    if constexpr (LOC) {
+      out_end = local_out(io.loc, a0, (int)b);
+      out_end = out_end < 0 ? 0 : out_end + io.loc.ix;
+    }
     if (cta_out_of_bounds(in_end > io.in_ext || out_end > io.out_ext || o0c < 0, io.chk_err)) return;
   }
   __shared__ const void* twslot;
@@ -389,6 +449,14 @@ __device__ __forceinline__ void inv_T_body(const LineIO& io, const typename Type
     }
   block_fft_inv<R, L, EPT, TC>(v, ex, tw, t, &tc);
   if (PART && !valid) return;
+  if constexpr (LOC) {
+    const int64_t o = local_out(io.loc, a0, (int)b);
+    if (o < 0) return;
+    R* row = static_cast<R*>(io.out[a1]) + o - io.loc.g;
+#pragma unroll
+    for (int m = 0; m < EPT; ++m) local_store(row, io.loc, 2 * (t + T * m), v[m]);
+    return;
+  }
   C* row;
   const int64_t o0 = out_off ? out_off[a0] : a0 * out_sa0;  // per-patch offsets of a batch
   if constexpr (C2R)
@@ -399,7 +467,7 @@ __device__ __forceinline__ void inv_T_body(const LineIO& io, const typename Type
   for (int m = 0; m < EPT; ++m) row[t + T * m] = v[m];
 }
 
-template <typename R, int L, bool C2R, int TC = 0>
+template <typename R, int L, bool C2R, int TC = 0, bool LOC = false>
 __global__ void __launch_bounds__(RowThreads<R, L>::value, sizeof(R) == 8 ? 1 : 2) k_inv_T(LineIO io, const typename Types<R>::W* __restrict__ tw,
                                                int64_t in_sa0, int64_t in_sk, int64_t out_sa0,
                                                int64_t out_sb, int log_tb, const int64_t* __restrict__ out_off) {
@@ -408,7 +476,7 @@ __global__ void __launch_bounds__(RowThreads<R, L>::value, sizeof(R) == 8 ? 1 : 
   if constexpr (TC) tc_setup(tc, smem_raw, io.gmat, 0u, io.err, TC == 2, 0u, io.tc_ctl);
   const RowCta cta{(int)blockIdx.x, (int)blockIdx.y, (int)blockIdx.z, (int)threadIdx.x, (int)threadIdx.y, log_tb,
                    (int64_t)gridDim.x << log_tb};
-  inv_T_body<R, L, C2R, TC, false>(io, tw, in_sa0, in_sk, out_sa0, out_sb, out_off, cta, smem_raw, tc);
+  inv_T_body<R, L, C2R, TC, false, LOC>(io, tw, in_sa0, in_sk, out_sa0, out_sb, out_off, cta, smem_raw, tc);
   if constexpr (TC) tc_teardown(tc);
 }
 
