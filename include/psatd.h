@@ -244,8 +244,8 @@ psatd_status psatd_plan_get_launch(psatd_plan plan, int32_t cfg[6]);
  * components in turn (FP32: pairs of components; group j: units j, j + G, ...),
  * meeting for the per-mode push.  G = 1 is the plain
  * pass.  Tensor-core plans (PSATD_MIXED_*): 2 only, two 128-row groups that
- * transform component pairs in lockstep and share every tensor-core round
- * (measured slower than one group on GB300; kept as a launch shape).
+ * transform the components in turn, each with its own tensor-core rounds (the
+ * built-in choice where the lines of a CTA are 128 threads).
  * set accepts otherwise: 1 always; 2 or 4 for PSATD_FP32 plans whose fused-axis lines
  * have a multiple of 32 threads (length / elements per thread), at most 512
  * threads and 15 groups per CTA, an even number of modes per thread, and (n_in + G)

@@ -287,20 +287,18 @@ psatd_status alloc(psatd_plan p, void** ptr, size_t bytes, const char* what) {
 
 // threads per CTA a transposing pass may launch (the kernels' launch bounds)
 int row_maxthr(int L, bool f32) { return !f32 ? 4096 / row_ept(L, false) : row_ept(L, true) >= 20 ? 256 : 512; }
-// Rows per CTA of a tensor-core transposing pass over `nb` rows: a divisor of nb, at most
-// 16 rows (the row-dependent XOR of the transposed store spreads 16 rows over the banks,
-// 32 would read one bank twice), up to 32 where that is needed for 128 threads.  Inverse:
-// half of that (measured faster: the gathered bin pairs of fewer rows per CTA), keeping
-// the 128 threads.
-int pick_log_tb_tc(int L, int64_t nb, bool fwd) {
-  const int T = L / row_ept(L, true), maxthr = row_maxthr(L, true);
+constexpr int kSMs = 152;  // GB300
+// Rows per CTA of a tensor-core transposing pass over `nb` rows of each of `planes` planes
+// and components: a divisor of nb, at most 32, giving 256 threads (256^3 split FP16, x forward
+// 16 / 32 rows 394 / 349 us, y inverse 8 / 16 rows 287 / 232 us), or 128, the least a unit
+// takes, while the launch has under two CTAs per SM (512^2: 8 / 16 rows 13.1 / 14.6 us).
+int pick_log_tb_tc(int L, int64_t nb, int64_t planes) {
+  const int T = L / row_ept(L, true);
   int lg = 0;
-  while ((T << (lg + 1)) <= maxthr && lg < 4 && nb % (2 << lg) == 0) ++lg;
-  while ((T << lg) < 128 && (T << (lg + 1)) <= maxthr && lg < 5 && nb % (2 << lg) == 0) ++lg;
-  if (!fwd && lg > 0 && (T << (lg - 1)) >= 128) --lg;
+  while ((T << (lg + 1)) <= 256 && lg < 5 && nb % (2 << lg) == 0) ++lg;
+  while ((T << lg) > 128 && lg > 0 && (nb >> lg) * planes < 2 * kSMs) --lg;
   return lg;
 }
-constexpr int kSMs = 152;  // GB300
 // Rows per CTA of an FP64 transposing pass: up to 512 threads and 16 rows (runs of the
 // transposed store), down to one row while the launch has under two CTAs per SM (the
 // FP64 units of every SM are the bound).
@@ -336,7 +334,7 @@ int rows_per_cta(psatd_plan p, int k) {
   const int64_t planes = (p->ndim == 3 ? (x ? p->nz : p->nxh) : p->npatch) * (fwd ? p->n_in : p->n_out);
   if (!p->f32) return pick_log_tb_f64(L, nb, planes);
   if (!p->tc) return pick_log_tb_pairs(L, nb, planes, fwd, x);
-  return pick_log_tb_tc(L, nb, fwd);
+  return pick_log_tb_tc(L, nb, planes);
 }
 
 // shared memory of a transposing pass: one L-element buffer per line, or the
@@ -392,7 +390,9 @@ size_t push_smem(int n_in, int L, int tb, int G, size_t csz, bool tc = false) {
 int push_units_of(int layout, int n_in) {
   return layout == PSATD_FIELDS_2D_TM ? n_in - 1 : (layout == PSATD_FIELDS_2D_TE ? n_in + 1 : n_in == 6 ? 6 : n_in + 1) / 2;
 }
-// The built-in choice (one group with tensor cores).  FP32: the fewest
+// The built-in choice.  Tensor cores: two groups where they fit, each a unit of its own
+// (2048^2 TE split BF16 / FP16 166 -> 142 / 155 -> 128 us, 128-point lines of eleven
+// components 630 -> 541 us; the same shared memory with twice the warps).  FP32: the fewest
 // groups (1, 2 or 4, no more than needed for one per unit) that give an SM 14 resident warps (of the 16 that the
 // registers allow) and the launch 256 threads per SM.  Measured with 1 / 2 / 4 groups:
 // 2048-point lines of five components 85.2 / 73.1 / 87.8 us; 1024 points, eleven
@@ -401,7 +401,8 @@ int push_units_of(int layout, int n_in) {
 // FP64: 2, 3 or 6 groups while the launch has under 256 threads per SM (a warp's FP64
 // instruction takes 64 cycles: a small launch's time is the instructions of a thread).
 int push_groups_default(int layout, int L, int ept, int tb, int n_in, int64_t nlines, bool tc, bool f32, int sm_bytes) {
-  if (tc || L < ept || sm_bytes <= 0) return 1;
+  if (tc) return push_groups_ok(L, ept, tb, 2, tc, f32) ? 2 : 1;
+  if (L < ept || sm_bytes <= 0) return 1;
   const int T = L / ept, thr = T * tb;
   if (!f32) {
     int G = 1;
@@ -703,7 +704,7 @@ psatd_status check_tc_shape(psatd_plan p, int maxsm) {
   struct { int L; int64_t nb; } rows[2] = {{Lx, p->ny}, {(int)p->ny, p->nz}};
   for (int i = 0; i < (p->ndim == 3 ? 2 : 1); ++i) {
     const int T = rows[i].L / row_ept(rows[i].L, true);
-    if ((T << pick_log_tb_tc(rows[i].L, rows[i].nb, true)) < 128)
+    if ((T << pick_log_tb_tc(rows[i].L, rows[i].nb, 1 << 20)) < 128)
       return fail(nullptr, PSATD_ERR_UNSUPPORTED,
                   "mixed precision: a line pass of length %d over %lld lines has fewer than 128 threads per CTA",
                   rows[i].L, (long long)rows[i].nb);

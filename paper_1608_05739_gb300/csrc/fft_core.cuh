@@ -594,13 +594,10 @@ __device__ __forceinline__ const typename Types<R>::W* stage_tw(const ExBuf<C>& 
 // keeps W_L^(r k L/(Ns R)) at [tw_off(s) + (r-1) Ns + k], k < Ns, 1 <= r < R,
 // so the threads of a warp read consecutive entries.
 
-// One forward stage.  act = false: the thread only takes part in the stage's
-// barriers (and tensor-core rounds), touching no exchange memory (a component
-// group with no component to transform while the other group has one).
+// One forward stage.
 template <typename R, int L, int EPT, int S, int TC>
 __device__ __forceinline__ void fwd_stage(typename Types<R>::C (&v)[EPT], ExBuf<typename Types<R>::C>& ex,
-                                          const typename Types<R>::W* __restrict__ tw, int t, TcCtx* tc,
-                                          bool act = true) {
+                                          const typename Types<R>::W* __restrict__ tw, int t, TcCtx* tc) {
   typedef typename Types<R>::C C;
   typedef FFTPlan<L, EPT> P;
   constexpr int RS = P::radix(S), NS = P::span(S), Q = EPT / RS, T = P::kT;
@@ -617,18 +614,16 @@ __device__ __forceinline__ void fwd_stage(typename Types<R>::C (&v)[EPT], ExBuf<
 #pragma unroll
     for (int r = 0; r < RS; ++r) a[r] = v[q + r * Q];
     if constexpr (NS > 1) {
-      if (act) {
-        const typename Types<R>::W* tws = stage_tw<R>(ex) + P::tw_off(S) + k;
+      const typename Types<R>::W* tws = stage_tw<R>(ex) + P::tw_off(S) + k;
 #pragma unroll
-        for (int r = 1; r < RS; ++r) a[r] = twmul(a[r], __ldg(&tws[(r - 1) * NS]));
-      }
+      for (int r = 1; r < RS; ++r) a[r] = twmul(a[r], __ldg(&tws[(r - 1) * NS]));
     }
-    if constexpr (TC && RS == 16) tc_dft<16, false, TC == 2>(a, *tc, act);
-    else if (act) butterfly<RS, false>(a);
+    if constexpr (TC && RS == 16) tc_dft<16, false, TC == 2>(a, *tc);
+    else butterfly<RS, false>(a);
     if constexpr (LAST) {
 #pragma unroll
       for (int r = 0; r < RS; ++r) v[q + r * Q] = a[r];
-    } else if (act) {
+    } else {
       const int base = (j - k) * RS + k;
 #pragma unroll
       for (int r = 0; r < RS; ++r) buf[sw<CX>(base + r * NS)] = a[r];
@@ -636,18 +631,15 @@ __device__ __forceinline__ void fwd_stage(typename Types<R>::C (&v)[EPT], ExBuf<
   }
   if constexpr (!LAST) {
     ex.sync();
-    if (act) {
 #pragma unroll
-      for (int m = 0; m < EPT; ++m) v[m] = buf[sw<CX>(t + T * m)];
-    }
+    for (int m = 0; m < EPT; ++m) v[m] = buf[sw<CX>(t + T * m)];
   }
 }
 
 // Adjoint of fwd_stage<S>.
 template <typename R, int L, int EPT, int S, int TC>
 __device__ __forceinline__ void inv_stage(typename Types<R>::C (&v)[EPT], ExBuf<typename Types<R>::C>& ex,
-                                          const typename Types<R>::W* __restrict__ tw, int t, TcCtx* tc,
-                                          bool act = true) {
+                                          const typename Types<R>::W* __restrict__ tw, int t, TcCtx* tc) {
   typedef typename Types<R>::C C;
   typedef FFTPlan<L, EPT> P;
   constexpr int RS = P::radix(S), NS = P::span(S), Q = EPT / RS, T = P::kT;
@@ -656,10 +648,8 @@ __device__ __forceinline__ void inv_stage(typename Types<R>::C (&v)[EPT], ExBuf<
   C* buf = nullptr;
   if constexpr (!FIRST) {
     buf = ex.next();
-    if (act) {
 #pragma unroll
-      for (int m = 0; m < EPT; ++m) buf[sw<CX>(t + T * m)] = v[m];
-    }
+    for (int m = 0; m < EPT; ++m) buf[sw<CX>(t + T * m)] = v[m];
     ex.sync();
   }
   asm volatile("" : "+r"(t)::"memory");  // stage boundary (see fwd_stage)
@@ -671,33 +661,24 @@ __device__ __forceinline__ void inv_stage(typename Types<R>::C (&v)[EPT], ExBuf<
     if constexpr (FIRST) {
 #pragma unroll
       for (int r = 0; r < RS; ++r) a[r] = v[q + r * Q];
-    } else if (act) {
+    } else {
       const int base = (j - k) * RS + k;
 #pragma unroll
       for (int r = 0; r < RS; ++r) a[r] = buf[sw<CX>(base + r * NS)];
-    } else {
-#pragma unroll
-      for (int r = 0; r < RS; ++r) a[r] = v[q + r * Q];
     }
-    if constexpr (TC && RS == 16) tc_dft<16, true, TC == 2>(a, *tc, act);
-    else if (act) butterfly<RS, true>(a);
+    if constexpr (TC && RS == 16) tc_dft<16, true, TC == 2>(a, *tc);
+    else butterfly<RS, true>(a);
     if constexpr (NS > 1) {
-      if (act) {
-        const typename Types<R>::W* tws = stage_tw<R>(ex) + P::tw_off(S) + k;
+      const typename Types<R>::W* tws = stage_tw<R>(ex) + P::tw_off(S) + k;
 #pragma unroll
-        for (int r = 1; r < RS; ++r) a[r] = twmul_conj(a[r], __ldg(&tws[(r - 1) * NS]));
-      }
+      for (int r = 1; r < RS; ++r) a[r] = twmul_conj(a[r], __ldg(&tws[(r - 1) * NS]));
     }
 #pragma unroll
     for (int r = 0; r < RS; ++r) v[q + r * Q] = a[r];
   }
 }
 
-// Forward transform with the twiddles of stage s + 1 loaded before stage s's
-// exchange barrier (the barrier and the exchange hide their latency; plain
-// fwd_stage issues them right before the multiply that needs them).  Holds one
-// stage's twiddles in registers (kPF per thread), for kernels with registers to
-// spare (the fused pass at 8 elements per thread).
+// Twiddles of one stage per thread (fft_line.cuh): the most over the stages.
 template <int L, int EPT>
 struct PFCount {
   typedef FFTPlan<L, EPT> P;
@@ -706,168 +687,36 @@ struct PFCount {
   static constexpr int value = max_from(1);
 };
 
-template <typename R, int L, int EPT, int S>
-__device__ __forceinline__ void load_stage_tw(typename Types<R>::W (&pf)[PFCount<L, EPT>::value],
-                                              const typename Types<R>::W* __restrict__ base, int t) {
-  typedef FFTPlan<L, EPT> P;
-  if constexpr (S >= 1 && S < P::kStages) {
-    constexpr int RS = P::radix(S), NS = P::span(S), Q = EPT / RS, T = P::kT;
-    if constexpr (NS > 1) {
-#pragma unroll
-      for (int q = 0; q < Q; ++q) {
-        const int j = t + q * T;
-        const int k = is_pow2(NS) ? (j & (NS - 1)) : (int)((unsigned)j % (unsigned)NS);
-        const typename Types<R>::W* tws = base + P::tw_off(S) + k;
-#pragma unroll
-        for (int r = 1; r < RS; ++r) pf[q * (RS - 1) + r - 1] = __ldg(&tws[(r - 1) * NS]);
-      }
-    }
-  }
-}
-
-template <typename R, int L, int EPT, int S>
-__device__ __forceinline__ void fwd_stage_pf(typename Types<R>::C (&v)[EPT], ExBuf<typename Types<R>::C>& ex,
-                                             typename Types<R>::W (&pf)[PFCount<L, EPT>::value], int t) {
-  typedef typename Types<R>::C C;
-  typedef FFTPlan<L, EPT> P;
-  constexpr int RS = P::radix(S), NS = P::span(S), Q = EPT / RS, T = P::kT;
-  constexpr bool LAST = (S == P::kStages - 1);
-  constexpr int CX = P::swz(S);
-  C* buf = nullptr;
-  if constexpr (!LAST) buf = ex.next();
-#pragma unroll
-  for (int q = 0; q < Q; ++q) {
-    const int j = t + q * T;
-    const int k = is_pow2(NS) ? (j & (NS - 1)) : (int)((unsigned)j % (unsigned)NS);
-    C a[RS];
-#pragma unroll
-    for (int r = 0; r < RS; ++r) a[r] = v[q + r * Q];
-    if constexpr (NS > 1) {
-#pragma unroll
-      for (int r = 1; r < RS; ++r) a[r] = twmul(a[r], pf[q * (RS - 1) + r - 1]);
-    }
-    butterfly<RS, false>(a);
-    if constexpr (LAST) {
-#pragma unroll
-      for (int r = 0; r < RS; ++r) v[q + r * Q] = a[r];
-    } else {
-      const int base = (j - k) * RS + k;
-#pragma unroll
-      for (int r = 0; r < RS; ++r) buf[sw<CX>(base + r * NS)] = a[r];
-    }
-  }
-  if constexpr (!LAST) {
-    load_stage_tw<R, L, EPT, S + 1>(pf, stage_tw<R>(ex), t);
-    ex.sync();
-#pragma unroll
-    for (int m = 0; m < EPT; ++m) v[m] = buf[sw<CX>(t + T * m)];
-  }
-}
-
-template <typename R, int L, int EPT, int... S>
-__device__ __forceinline__ void fft_fwd_pf_seq(typename Types<R>::C (&v)[EPT], ExBuf<typename Types<R>::C>& ex,
-                                               int t, std::integer_sequence<int, S...>) {
-  typename Types<R>::W pf[PFCount<L, EPT>::value];
-  load_stage_tw<R, L, EPT, 1>(pf, stage_tw<R>(ex), t);
-  (fwd_stage_pf<R, L, EPT, S>(v, ex, pf, t), ...);
-}
-
 template <typename R, int L, int EPT, int TC, int... S>
 __device__ __forceinline__ void fft_fwd_seq(typename Types<R>::C (&v)[EPT], ExBuf<typename Types<R>::C>& ex,
-                                            const typename Types<R>::W* tw, int t, TcCtx* tc, bool act,
+                                            const typename Types<R>::W* tw, int t, TcCtx* tc,
                                             std::integer_sequence<int, S...>) {
-  (fwd_stage<R, L, EPT, S, TC>(v, ex, tw, t, tc, act), ...);
+  (fwd_stage<R, L, EPT, S, TC>(v, ex, tw, t, tc), ...);
 }
 template <typename R, int L, int EPT, int TC, int... S>
 __device__ __forceinline__ void fft_inv_seq(typename Types<R>::C (&v)[EPT], ExBuf<typename Types<R>::C>& ex,
-                                            const typename Types<R>::W* tw, int t, TcCtx* tc, bool act,
+                                            const typename Types<R>::W* tw, int t, TcCtx* tc,
                                             std::integer_sequence<int, S...>) {
-  (inv_stage<R, L, EPT, FFTPlan<L, EPT>::kStages - 1 - S, TC>(v, ex, tw, t, tc, act), ...);
+  (inv_stage<R, L, EPT, FFTPlan<L, EPT>::kStages - 1 - S, TC>(v, ex, tw, t, tc), ...);
 }
 
 // Forward DFT of length L: v holds x[t + T m] on entry, X[t + T m] on exit
 // (T = L/EPT, m < EPT).  Every thread of the block must call it (block-wide
 // barriers inside); the exchanges alternate between the two buffers of `ex`.
 // TC: the radix-16 stages run on the tensor cores (tc_dft.cuh, context *tc):
-// 1 split-FP16, 2 split-BF16.  act = false: barriers and tensor-core rounds
-// only (see fwd_stage).
+// 1 split-FP16, 2 split-BF16.
 template <typename R, int L, int EPT, int TC = 0>
 __device__ __forceinline__ void block_fft_fwd(typename Types<R>::C (&v)[EPT], ExBuf<typename Types<R>::C>& ex,
-                                              const typename Types<R>::W* tw, int t, TcCtx* tc = nullptr,
-                                              bool act = true) {
+                                              const typename Types<R>::W* tw, int t, TcCtx* tc = nullptr) {
   static_assert(!TC || sizeof(R) == 4, "tensor-core stages take float data");
-  fft_fwd_seq<R, L, EPT, TC>(v, ex, tw, t, tc, act, std::make_integer_sequence<int, FFTPlan<L, EPT>::kStages>{});
+  fft_fwd_seq<R, L, EPT, TC>(v, ex, tw, t, tc, std::make_integer_sequence<int, FFTPlan<L, EPT>::kStages>{});
 }
-// Adjoint of fwd_stage_pf's stage S: the stage's twiddles are loaded before its
-// exchange barrier (they are applied after the butterfly).
-template <typename R, int L, int EPT, int S>
-__device__ __forceinline__ void inv_stage_pf(typename Types<R>::C (&v)[EPT], ExBuf<typename Types<R>::C>& ex,
-                                             typename Types<R>::W (&pf)[PFCount<L, EPT>::value], int t) {
-  typedef typename Types<R>::C C;
-  typedef FFTPlan<L, EPT> P;
-  constexpr int RS = P::radix(S), NS = P::span(S), Q = EPT / RS, T = P::kT;
-  constexpr bool FIRST = (S == P::kStages - 1);
-  constexpr int CX = P::swz(S);
-  C* buf = nullptr;
-  if constexpr (!FIRST) {
-    buf = ex.next();
-#pragma unroll
-    for (int m = 0; m < EPT; ++m) buf[sw<CX>(t + T * m)] = v[m];
-  }
-  load_stage_tw<R, L, EPT, S>(pf, stage_tw<R>(ex), t);
-  if constexpr (!FIRST) ex.sync();
-#pragma unroll
-  for (int q = 0; q < Q; ++q) {
-    const int j = t + q * T;
-    const int k = is_pow2(NS) ? (j & (NS - 1)) : (int)((unsigned)j % (unsigned)NS);
-    C a[RS];
-    if constexpr (FIRST) {
-#pragma unroll
-      for (int r = 0; r < RS; ++r) a[r] = v[q + r * Q];
-    } else {
-      const int base = (j - k) * RS + k;
-#pragma unroll
-      for (int r = 0; r < RS; ++r) a[r] = buf[sw<CX>(base + r * NS)];
-    }
-    butterfly<RS, true>(a);
-    if constexpr (NS > 1) {
-#pragma unroll
-      for (int r = 1; r < RS; ++r) a[r] = twmul_conj(a[r], pf[q * (RS - 1) + r - 1]);
-    }
-#pragma unroll
-    for (int r = 0; r < RS; ++r) v[q + r * Q] = a[r];
-  }
-}
-
-template <typename R, int L, int EPT, int... S>
-__device__ __forceinline__ void fft_inv_pf_seq(typename Types<R>::C (&v)[EPT], ExBuf<typename Types<R>::C>& ex,
-                                               int t, std::integer_sequence<int, S...>) {
-  typename Types<R>::W pf[PFCount<L, EPT>::value];
-  (inv_stage_pf<R, L, EPT, FFTPlan<L, EPT>::kStages - 1 - S>(v, ex, pf, t), ...);
-}
-
-// block_fft_inv with each stage's twiddles loaded before its exchange barrier.
-template <typename R, int L, int EPT>
-__device__ __forceinline__ void block_fft_inv_pf(typename Types<R>::C (&v)[EPT], ExBuf<typename Types<R>::C>& ex,
-                                                 int t) {
-  fft_inv_pf_seq<R, L, EPT>(v, ex, t, std::make_integer_sequence<int, FFTPlan<L, EPT>::kStages>{});
-}
-
-// block_fft_fwd with next-stage twiddle prefetch (no tensor-core stages); the
-// twiddle table is read through ex.twslot, which must be visible before the call.
-template <typename R, int L, int EPT>
-__device__ __forceinline__ void block_fft_fwd_pf(typename Types<R>::C (&v)[EPT], ExBuf<typename Types<R>::C>& ex,
-                                                 int t) {
-  fft_fwd_pf_seq<R, L, EPT>(v, ex, t, std::make_integer_sequence<int, FFTPlan<L, EPT>::kStages>{});
-}
-
 // Unnormalised inverse DFT (adjoint of block_fft_fwd).
 template <typename R, int L, int EPT, int TC = 0>
 __device__ __forceinline__ void block_fft_inv(typename Types<R>::C (&v)[EPT], ExBuf<typename Types<R>::C>& ex,
-                                              const typename Types<R>::W* tw, int t, TcCtx* tc = nullptr,
-                                              bool act = true) {
+                                              const typename Types<R>::W* tw, int t, TcCtx* tc = nullptr) {
   static_assert(!TC || sizeof(R) == 4, "tensor-core stages take float data");
-  fft_inv_seq<R, L, EPT, TC>(v, ex, tw, t, tc, act, std::make_integer_sequence<int, FFTPlan<L, EPT>::kStages>{});
+  fft_inv_seq<R, L, EPT, TC>(v, ex, tw, t, tc, std::make_integer_sequence<int, FFTPlan<L, EPT>::kStages>{});
 }
 
 }  // namespace psatd

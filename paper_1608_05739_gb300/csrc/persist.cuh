@@ -98,7 +98,7 @@ __global__ void __launch_bounds__(kPersistXThreads, (FAM || TC) ? 2 : 4) k_persi
   __shared__ int slot;
   __shared__ __align__(16) XClassArgs A;
   TcCtx tc;
-  if constexpr (TC) tc_setup(tc, smem_raw, cls[0].io.gmat, 0u, cls[0].io.err, TC == 2, 0u, cls[0].io.tc_ctl);
+  if constexpr (TC) tc_setup(tc, smem_raw, cls[0].io.gmat, 0u, cls[0].io.err, TC == 2, 0u, cls[0].io.tc_ctl, 128, TcGeom<16>::kAPiece);
   for (;;) {
     const int i0 = persist_take(q, &slot);
     if (i0 >= q.n_items) break;
@@ -144,7 +144,7 @@ __global__ void __launch_bounds__(kPersistThreads, TC ? 2 : 4) k_persist_push(co
   StageCtx sc;
   stage_init(sc, &stage_mbar, cls[0].err ? cls[0].err : cls[0].chk_err);
   TcCtx tc;
-  if constexpr (TC) tc_setup(tc, smem_raw, cls[0].gmat, 0u, cls[0].err, TC == 2, 0u, cls[0].tc_ctl);
+  if constexpr (TC) tc_setup(tc, smem_raw, cls[0].gmat, 0u, cls[0].err, TC == 2, 0u, cls[0].tc_ctl, 128, TcGeom<16>::kATile);
   // (the queue's first take has a block barrier before any use of the stage mbarrier)
   for (;;) {
     const int i0 = persist_take(q, &slot);

@@ -219,6 +219,10 @@ __device__ __forceinline__ void fwd_T_body(const LineIO& io, const typename Type
     tc.a_tile3 = smem_u32(smem + (R2C ? TB * L : L * (TB + 1)));
   }
   ExBuf<C> ex{{smem + g * L, smem + g * L}, 0, &twslot, true};  // one exchange buffer per line
+  if constexpr (TC) {  // tensor-core units exchange among themselves
+    ex.bar_id = 1 + tc_tid() / tc.rn;
+    ex.bar_n = tc.rn;
+  }
   if constexpr (!TC && T % 32 == 0)
     if (TB <= 8) {  // each line's warps synchronise among themselves between stages
       ex.bar_id = 1 + g;
@@ -316,7 +320,9 @@ __global__ void __launch_bounds__(RowThreads<R, L>::value, sizeof(R) == 8 ? 1 : 
                                                int64_t out_sk, int log_tb, const int64_t* __restrict__ in_off) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   TcCtx tc;
-  if constexpr (TC) tc_setup(tc, smem_raw, io.gmat, 0u, io.err, TC == 2, 0u, io.tc_ctl);
+  constexpr int kRn = tc_unit_threads(FFTPlan<L, RowEPT<L, R>::value>::kT);
+  if constexpr (TC)
+    tc_setup(tc, smem_raw, io.gmat, 0u, io.err, TC == 2, 0u, io.tc_ctl, kRn, kRn / 128 * TcGeom<16>::kAPiece);
   const RowCta cta{(int)blockIdx.x, (int)blockIdx.y, (int)blockIdx.z, (int)threadIdx.x, (int)threadIdx.y, log_tb,
                    (int64_t)gridDim.x << log_tb};
   fwd_T_body<R, L, R2C, TC, false, LOC>(io, tw, in_sa0, in_sb, out_sa0, out_sk, in_off, cta, smem_raw, tc);
@@ -442,6 +448,10 @@ __device__ __forceinline__ void inv_T_body(const LineIO& io, const typename Type
     __syncthreads();
   }
   ExBuf<C> ex{{smem + g * L, smem + g * L}, 0, &twslot, true};  // one exchange buffer per line
+  if constexpr (TC) {  // tensor-core units exchange among themselves
+    ex.bar_id = 1 + tc_tid() / tc.rn;
+    ex.bar_n = tc.rn;
+  }
   if constexpr (!TC && T % 32 == 0)
     if (TB <= 8) {  // line-private stages: the line's own warps synchronise
       ex.bar_id = 1 + g;
@@ -473,7 +483,9 @@ __global__ void __launch_bounds__(RowThreads<R, L>::value, sizeof(R) == 8 ? 1 : 
                                                int64_t out_sb, int log_tb, const int64_t* __restrict__ out_off) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   TcCtx tc;
-  if constexpr (TC) tc_setup(tc, smem_raw, io.gmat, 0u, io.err, TC == 2, 0u, io.tc_ctl);
+  constexpr int kRn = tc_unit_threads(FFTPlan<L, RowEPT<L, R>::value>::kT);
+  if constexpr (TC)
+    tc_setup(tc, smem_raw, io.gmat, 0u, io.err, TC == 2, 0u, io.tc_ctl, kRn, kRn / 128 * TcGeom<16>::kAPiece);
   const RowCta cta{(int)blockIdx.x, (int)blockIdx.y, (int)blockIdx.z, (int)threadIdx.x, (int)threadIdx.y, log_tb,
                    (int64_t)gridDim.x << log_tb};
   inv_T_body<R, L, C2R, TC, false, LOC>(io, tw, in_sa0, in_sk, out_sa0, out_sb, out_off, cta, smem_raw, tc);
@@ -914,11 +926,10 @@ __device__ __forceinline__ void line_push_body(const PushArgs<R>& a_in, const ty
   // a private copy: its scalars stay in registers through the shared-memory stores of the transforms
   const PushArgs<R> a = a_in;
   typedef typename Types<R>::C C;
-  static_assert(!TC || EPT == 16, "tensor-core stages are radix 16");
+  static_assert(TC != 0 && EPT == 16, "tensor-core stages are radix 16 (the other plans run pair_push.cuh)");
   typedef FFTPlan<L, EPT> P;
   constexpr int T = P::kT;
   constexpr int CXL = P::kLastCX;
-  static_assert(!GRP || TC || T % 32 == 0, "SIMT component groups need whole-warp lines");
   if constexpr (!GRP) {  // the plain pass
     grp = 0;
     G = 1;
@@ -939,15 +950,9 @@ __device__ __forceinline__ void line_push_body(const PushArgs<R>& a_in, const ty
   C* spec = static_cast<C*>(a.spec);
   __shared__ const void* twslot;
   if (t == 0 && g == 0 && grp == 0) twslot = tw;
-  // exchange barrier of this line's group: the block's (G = 1), else a named one.
-  // Only kernels whose lines have whole warps (T a multiple of 32) contain the
-  // named barrier at all: its thread count must be a multiple of the warp size.
-  int bar_id = 0, bar_n = 0;
-  if constexpr (GRP && !TC) {
-    bar_id = 1 + g * G + grp;
-    bar_n = T;
-  }
-  if constexpr (TC) tc.a_tile = smem_u32(base + a.n_in * ss);  // split-BF16's third A piece: per component below
+  // exchange barrier: the tensor-core unit's
+  const int bar_id = 1 + tc_tid() / tc.rn, bar_n = tc.rn;
+  tc.a_tile = smem_u32(base + a.n_in * ss);  // split-BF16's third A pieces: per component below
 
   int mxi, myi, rowi;
   line_modes(a, valid ? line : 0, mxi, myi, rowi);
@@ -1001,29 +1006,22 @@ __device__ __forceinline__ void line_push_body(const PushArgs<R>& a_in, const ty
   }
   C v[EPT];
   if constexpr (TC && GRP) {
-    // Tensor-core component pairs: the two groups (128 rows each) transform the
-    // components c0 and c0 + 1 in lockstep, so that every tensor-core round (block
-    // barriers, one issuing thread, one commit) serves both; a group with no
-    // component in the last pair only takes part in the barriers and rounds.  Each
-    // component exchanges in its own slot (one buffer), its A_h / A_m tiles sit in
-    // that slot at the round (group j's at tc.a_tile + j x tile size = slot c0 + j:
-    // the slot stride of 128 rows of 16 complex values equals the tile size) and
-    // both third pieces in the spare region; the shared memory is the one-group
+    // Component groups: group j (128 rows, a unit of its own) transforms the components
+    // c = j, j + 2, ...  A component exchanges in its own slot (one buffer); its A_h /
+    // A_m tiles sit in that slot at the round (unit j's at tc.a_tile + j x tile size =
+    // slot c: the slot stride of 128 rows of 16 complex values equals the tile size) and
+    // both units' third pieces in the spare region; the shared memory is the one-group
     // pass's, with twice its threads.
     tc.a_tile3 = smem_u32(base + a.n_in * ss);
-    for (int c0 = 0; c0 < a.n_in; c0 += 2) {
-      const int c = c0 + grp;
-      const bool act = c < a.n_in;
-      C* sl = st + (act ? c : c0) * ss;
+    for (int c = grp; c < a.n_in; c += 2) {
+      C* sl = st + c * ss;
 #pragma unroll
-      for (int m = 0; m < EPT; ++m) v[m] = act ? sl[t + T * m] : mkc(R(0), R(0));
-      ExBuf<C> ex{{sl, sl}, 0, &twslot, true};
-      tc.a_tile = smem_u32(base + c0 * ss);
-      block_fft_fwd<R, L, EPT, TC>(v, ex, tw, t, &tc, act);
-      if (act) {
+      for (int m = 0; m < EPT; ++m) v[m] = sl[t + T * m];
+      ExBuf<C> ex{{sl, sl}, 0, &twslot, true, bar_id, bar_n};
+      tc.a_tile = smem_u32(base + (c - grp) * ss);
+      block_fft_fwd<R, L, EPT, TC>(v, ex, tw, t, &tc);
 #pragma unroll
-        for (int m = 0; m < EPT; ++m) sl[sw<CXL>(t + T * m)] = v[m];
-      }
+      for (int m = 0; m < EPT; ++m) sl[sw<CXL>(t + T * m)] = v[m];
     }
   } else {
     for (int c = grp; c < a.n_in; c += G) {
@@ -1032,11 +1030,8 @@ __device__ __forceinline__ void line_push_body(const PushArgs<R>& a_in, const ty
       for (int m = 0; m < EPT; ++m) v[m] = sl[t + T * m];
       ExBuf<C> ex{{sl, bufB}, 0, &twslot, false, bar_id, bar_n};
       ex.sync();  // the slot becomes an exchange buffer
-      if constexpr (TC) tc.a_tile3 = smem_u32(base + c * ss);
-      if constexpr (TC == 0 && (EPT == 8 || EPT == 12))
-        block_fft_fwd_pf<R, L, EPT>(v, ex, t);
-      else
-        block_fft_fwd<R, L, EPT, TC>(v, ex, tw, t, &tc);
+      tc.a_tile3 = smem_u32(base + c * ss);
+      block_fft_fwd<R, L, EPT, TC>(v, ex, tw, t, &tc);
 #pragma unroll
       for (int m = 0; m < EPT; ++m) sl[sw<CXL>(t + T * m)] = v[m];
     }
@@ -1058,17 +1053,15 @@ __device__ __forceinline__ void line_push_body(const PushArgs<R>& a_in, const ty
   }
   if (G > 1) __syncthreads();  // every mode is pushed
 
-  if constexpr (TC && GRP) {  // output pairs in lockstep, as the input pairs above
-    for (int c0 = 0; c0 < a.n_out; c0 += 2) {
-      const int c = c0 + grp;
-      const bool act = c < a.n_out;
-      C* sl = st + (act ? c : c0) * ss;
+  if constexpr (GRP) {  // outputs, as the inputs above
+    for (int c = 1 - grp; c < a.n_out; c += 2) {
+      C* sl = st + c * ss;
 #pragma unroll
-      for (int m = 0; m < EPT; ++m) v[m] = act ? sl[sw<CXL>(t + T * m)] : mkc(R(0), R(0));
-      ExBuf<C> ex{{sl, sl}, 0, &twslot, true};
-      tc.a_tile = smem_u32(base + c0 * ss);
-      block_fft_inv<R, L, EPT, TC>(v, ex, tw, t, &tc, act);
-      if (act && valid) {
+      for (int m = 0; m < EPT; ++m) v[m] = sl[sw<CXL>(t + T * m)];
+      ExBuf<C> ex{{sl, sl}, 0, &twslot, true, bar_id, bar_n};
+      tc.a_tile = smem_u32(base + (c - grp) * ss);
+      block_fft_inv<R, L, EPT, TC>(v, ex, tw, t, &tc);
+      if (valid) {
         C* dst = spec + c * a.cs + (int64_t)line * L;
 #pragma unroll
         for (int m = 0; m < EPT; ++m) dst[t + T * m] = v[m];
@@ -1076,16 +1069,13 @@ __device__ __forceinline__ void line_push_body(const PushArgs<R>& a_in, const ty
     }
     return;
   }
-  for (int c = G - 1 - grp; c < a.n_out; c += G) {
+  for (int c = 0; c < a.n_out; ++c) {
     C* sl = st + c * ss;
 #pragma unroll
     for (int m = 0; m < EPT; ++m) v[m] = sl[sw<CXL>(t + T * m)];
     ExBuf<C> ex{{sl, bufB}, 0, &twslot, false, bar_id, bar_n};
-    if constexpr (TC) tc.a_tile3 = smem_u32(base + c * ss);
-    if constexpr (TC == 0 && (EPT == 8 || EPT == 12))
-      block_fft_inv_pf<R, L, EPT>(v, ex, t);
-    else
-      block_fft_inv<R, L, EPT, TC>(v, ex, tw, t, &tc);
+    tc.a_tile3 = smem_u32(base + c * ss);
+    block_fft_inv<R, L, EPT, TC>(v, ex, tw, t, &tc);
     if (valid) {
       C* dst = spec + c * a.cs + (int64_t)line * L;
 #pragma unroll
@@ -1097,18 +1087,19 @@ __device__ __forceinline__ void line_push_body(const PushArgs<R>& a_in, const ty
 // Block (T, lines per CTA, component groups); the group variant (GRP) takes up
 // to 512 threads (the tensor-core pairs 256), the plain pass 256 (or T).
 template <typename R, int L, int LAYOUT, int TC, int EPT, bool GRP>
-__global__ void __launch_bounds__(GRP ? 512 : (FFTPlan<L, EPT>::kT > 256 ? FFTPlan<L, EPT>::kT : 256))
+__global__ void __launch_bounds__(256, GRP ? 2 : 1)
 k_line_push(PushArgs<R> a, const typename Types<R>::W* __restrict__ tw) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ __align__(8) uint64_t stage_mbar;
   StageCtx sc;
   stage_init(sc, &stage_mbar, a.err ? a.err : a.chk_err);
   TcCtx tc;
-  if constexpr (TC) tc_setup(tc, smem_raw, a.gmat, 0u, a.err, TC == 2, 0u, a.tc_ctl);  // has a block barrier
-  else __syncthreads();  // the stage mbarrier is initialised
+  constexpr int kRn = tc_unit_threads(FFTPlan<L, EPT>::kT);
+  tc_setup(tc, smem_raw, a.gmat, 0u, a.err, TC == 2, 0u, a.tc_ctl, kRn,
+           GRP ? TcGeom<16>::kAPiece : kRn / 128 * TcGeom<16>::kATile);  // has a block barrier
   line_push_body<R, L, LAYOUT, TC, EPT, GRP>(a, tw, (int)blockIdx.x, (int)threadIdx.x, (int)threadIdx.y,
                                              (int)blockDim.y, (int)threadIdx.z, (int)blockDim.z, smem_raw, tc, sc);
-  if constexpr (TC) tc_teardown(tc);
+  tc_teardown(tc);
 }
 
 

@@ -50,13 +50,15 @@ constexpr int kErrMmaWait = 1;  // an MMA-completion wait ran out of iterations
 constexpr int kTcStallMma = 1;
 
 struct TcCtx {
-  uint32_t mbar;     // shared address of the MMA-completion mbarrier
+  uint32_t mbar;     // shared address of this thread's unit's MMA-completion mbarrier
   uint32_t tmem;     // TMEM address of the CTA's accumulators (lane 0, first column)
   uint32_t a_tile;   // shared address of this CTA's A tiles (group g at + g * tile bytes)
-  uint32_t a_tile3;  // split-BF16: third A piece (group g at + g * piece bytes)
+  uint32_t a_tile3;  // split-BF16: third A pieces (unit u's at + u * a3_unit, a piece per 128 rows)
+  uint32_t a3_unit;
+  int rn;            // threads of a unit (below): 128, or a line's where that is more
   uint32_t bmat;     // shared address of the split DFT matrices, forward then adjoint
   uint32_t phase;    // parity of the next mbarrier phase (identical in every thread)
-  volatile int* abort;  // CTA-shared word: nonzero once any thread's completion wait ran out
+  volatile int* abort;  // the unit's shared word: nonzero once any of its threads' completion waits ran out
   int* err;          // device error word (may be null)
   int bf16;          // 0 split-FP16, 1 split-BF16
   int wait_iters;    // poll limit of each completion wait
@@ -185,25 +187,37 @@ __host__ __device__ constexpr int tc_tmem_cols(int nthreads) {
   return nthreads <= 128 ? 64 : nthreads <= 256 ? 128 : nthreads <= 512 ? 256 : 512;
 }
 
+// Threads of a unit for lines of T threads: whole lines, at least one MMA's 128 rows.
+__host__ __device__ constexpr int tc_unit_threads(int T) { return T > 128 ? T : 128; }
+__device__ __forceinline__ int tc_tid() {
+  return (threadIdx.z * blockDim.y + threadIdx.y) * blockDim.x + threadIdx.x;
+}
+// Barrier of the calling thread's unit (named barrier 1 + unit).
+__device__ __forceinline__ void tc_unit_sync(int rn) {
+  asm volatile("bar.sync %0, %1;" ::"r"(1 + tc_tid() / rn), "r"(rn) : "memory");
+}
+
 // One radix-RS DFT (forward, or adjoint for ADJ) of the RS values a[] of every
-// thread's butterfly, on the tensor cores.  Every thread of the CTA calls it
-// (block barriers inside); the block's thread count is a multiple of 128.  The
-// A tiles alias exchange space that holds no live data at a stage boundary.
+// thread's butterfly, on the tensor cores.  Called by whole units of tc.rn threads
+// (128, or 256 for lines of 4096 points), each a round of its own (unit barriers, one
+// issuing thread, its own mbarrier): the units of a CTA never wait for each other, so
+// one splits its operands while another's MMAs run.  Bound: the latency of a round
+// (operand stores, barrier, MMAs, TMEM read) at 16 warps per SM, not the tensor pipe (1 %).
+// CTA-wide rounds and scalar splits -> units and packed splits: 256^3 J-form split FP16
+// 2573 -> 2079 us a step, 512-patch split BF16 22.3 -> 20.1 ms per four steps.  The
+// A tiles alias exchange space of the unit that holds no live data at a stage boundary.
 // BF16: split-BF16 operands (else split-FP16).
-// Failure path: a thread whose completion wait runs out sets the CTA's abort
+// Failure path: a thread whose completion wait runs out sets the unit's abort
 // word and the error word and leaves a[] as it is (its TMEM row may still be
 // written by the MMAs).  The abort word is read after the stage's first
-// barrier, so every thread sees the same value: once it is set, no thread
+// barrier, so every thread of the unit sees the same value: once it is set, none
 // splits, issues, waits or reads TMEM again, and tc_teardown makes one last
 // bounded wait for the outstanding commit before it frees the TMEM columns.
-// act = false: the thread writes no operand (its 128-row group has no data this
-// round; its rows of the MMAs read whatever the tile holds and are not used).
 template <int RS, bool ADJ, bool BF16>
-__device__ __forceinline__ void tc_dft(float2 (&a)[RS], TcCtx& tc, bool act = true) {
+__device__ __forceinline__ void tc_dft(float2 (&a)[RS], TcCtx& tc) {
   typedef TcGeom<RS> G;
-  const int tid = (threadIdx.z * blockDim.y + threadIdx.y) * blockDim.x + threadIdx.x;
-  const int grp = tid >> 7, row = tid & 127;
-  const int ngrp = (blockDim.x * blockDim.y * blockDim.z) >> 7;
+  const int tid = tc_tid();
+  const int grp = tid >> 7, row = tid & 127, unit = tid / tc.rn, u0 = unit * (tc.rn >> 7);
 
   // row scale 2^k with max |component| * 2^k in [2^14, 2^15)
   float mx = 0.f;
@@ -213,29 +227,31 @@ __device__ __forceinline__ void tc_dft(float2 (&a)[RS], TcCtx& tc, bool act = tr
   int k = be ? 141 - be : 0;
   k = k > 126 ? 126 : k;
   const float s = __int_as_float((127 + k) << 23), is = __int_as_float((127 - k) << 23);
-  constexpr float kRound16 = 201326592.0f;    // 1.5 * 2^27: (t + c) - c rounds t to a multiple of 16
-  constexpr float kRound128 = 1610612736.0f;  // 1.5 * 2^30: to a multiple of 128
+  // (t + c) - c rounds t to a multiple of 16 (c = 1.5 * 2^27) or 128 (1.5 * 2^30); both
+  // halves of a complex value in packed arithmetic, x - y as fma(y, -1, x) (one rounding)
+  constexpr float kRound = BF16 ? 1610612736.0f : 201326592.0f;
+  const float2 s2 = make_float2(s, s), round2 = make_float2(kRound, kRound), nround2 = make_float2(-kRound, -kRound),
+               minus = make_float2(-1.f, -1.f);
 
-  __syncthreads();  // every exchange read of the previous stage is done
+  tc_unit_sync(tc.rn);  // every exchange read of the previous stage is done
   const bool aborted = *tc.abort != 0;
-  if (!aborted && act) {
+  if (!aborted) {
     const uint32_t base = tc.a_tile + grp * G::kATile + (row >> 3) * G::kSBO + (row & 7) * 16;
-    const uint32_t base3 = tc.a_tile3 + grp * G::kAPiece + (row >> 3) * G::kSBO + (row & 7) * 16;
+    const uint32_t base3 = tc.a_tile3 + unit * tc.a3_unit + (grp - u0) * G::kAPiece + (row >> 3) * G::kSBO + (row & 7) * 16;
 #pragma unroll
     for (int kc = 0; kc < RS / 4; ++kc) {
       uint32_t hi[4], lo[4], l3[4];
       if constexpr (BF16) {
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
-          const float tx = a[4 * kc + e].x * s, ty = a[4 * kc + e].y * s;
-          const float hx = __fsub_rn(__fadd_rn(tx, kRound128), kRound128);
-          const float hy = __fsub_rn(__fadd_rn(ty, kRound128), kRound128);
-          const float rx = __fsub_rn(tx, hx), ry = __fsub_rn(ty, hy);
-          const __nv_bfloat162 m = __floats2bfloat162_rn(rx, ry);
-          const float2 mf = __bfloat1622float2(m);
-          hi[e] = b2u(__floats2bfloat162_rn(hx, hy));
+          const float2 t = __fmul2_rn(a[4 * kc + e], s2);
+          const float2 h = __fadd2_rn(__fadd2_rn(t, round2), nround2);
+          const float2 r = __ffma2_rn(h, minus, t);
+          const __nv_bfloat162 m = __floats2bfloat162_rn(r.x, r.y);
+          const float2 l = __ffma2_rn(__bfloat1622float2(m), minus, r);
+          hi[e] = b2u(__floats2bfloat162_rn(h.x, h.y));
           lo[e] = b2u(m);
-          l3[e] = b2u(__floats2bfloat162_rn(__fsub_rn(rx, mf.x), __fsub_rn(ry, mf.y)));
+          l3[e] = b2u(__floats2bfloat162_rn(l.x, l.y));
         }
         asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(base3 + kc * 128), "r"(l3[0]),
                      "r"(l3[1]), "r"(l3[2]), "r"(l3[3])
@@ -243,11 +259,11 @@ __device__ __forceinline__ void tc_dft(float2 (&a)[RS], TcCtx& tc, bool act = tr
       } else {
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
-          const float tx = a[4 * kc + e].x * s, ty = a[4 * kc + e].y * s;
-          const float hx = __fsub_rn(__fadd_rn(tx, kRound16), kRound16);
-          const float hy = __fsub_rn(__fadd_rn(ty, kRound16), kRound16);
-          hi[e] = h2u(__floats2half2_rn(hx, hy));
-          lo[e] = h2u(__floats2half2_rn(__fsub_rn(tx, hx), __fsub_rn(ty, hy)));
+          const float2 t = __fmul2_rn(a[4 * kc + e], s2);
+          const float2 h = __fadd2_rn(__fadd2_rn(t, round2), nround2);
+          const float2 r = __ffma2_rn(h, minus, t);
+          hi[e] = h2u(__floats2half2_rn(h.x, h.y));
+          lo[e] = h2u(__floats2half2_rn(r.x, r.y));
         }
       }
       asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(base + kc * 128), "r"(hi[0]), "r"(hi[1]),
@@ -259,9 +275,9 @@ __device__ __forceinline__ void tc_dft(float2 (&a)[RS], TcCtx& tc, bool act = tr
     }
   }
   fence_async_smem();
-  __syncthreads();
+  tc_unit_sync(tc.rn);
   if (aborted) return;
-  if (tid == 0 && !tc.stall) {
+  if (tid == unit * tc.rn && !tc.stall) {
     tc_fence_after();
     const uint32_t g0 = tc.bmat + (ADJ ? G::kGDir : 0);
     constexpr uint32_t idesc = BF16 ? G::kIdescBF16 : G::kIdesc;
@@ -270,10 +286,10 @@ __device__ __forceinline__ void tc_dft(float2 (&a)[RS], TcCtx& tc, bool act = tr
     //   BF16: A_h G_m, A_m G_h, A_h G_l, A_l G_h, A_m G_m (A pieces h, m, l; G pieces h, m, l)
     constexpr int np = BF16 ? 6 : 5;
 #pragma unroll 1
-    for (int gi = 0; gi < ngrp; ++gi) {
-      const uint32_t a0 = tc.a_tile + gi * G::kATile;
-      const uint32_t a3 = tc.a_tile3 + gi * G::kAPiece;
-      const uint32_t d = tc.tmem + gi * 64;
+    for (int gi = 0; gi < (tc.rn >> 7); ++gi) {
+      const uint32_t a0 = tc.a_tile + (u0 + gi) * G::kATile;
+      const uint32_t a3 = tc.a_tile3 + unit * tc.a3_unit + gi * G::kAPiece;
+      const uint32_t d = tc.tmem + (u0 + gi) * 64;
 #pragma unroll
       for (int p = 0; p < np; ++p) {
         int ai, gj;
@@ -304,50 +320,53 @@ __device__ __forceinline__ void tc_dft(float2 (&a)[RS], TcCtx& tc, bool act = tr
   }
   tc_fence_after();
   const uint32_t taddr = tc.tmem + ((uint32_t)((tid >> 5) & 3) << 21) + grp * 64;  // lane base 32 (warp % 4)
-  // 16 columns (8 complex outputs) at a time: head, then correction added
+  // 16 columns (8 complex outputs) at a time: head and correction, added and scaled back
+  const float2 is2 = make_float2(is, is);
 #pragma unroll
   for (int h = 0; h < RS / 8; ++h) {
-    uint32_t r[16];
+    uint32_t r[16], q[16];
     tmem_ld16(taddr + h * 16, r);
+    tmem_ld16(taddr + 32 + h * 16, q);
     tmem_ld_wait();
 #pragma unroll
-    for (int q = 0; q < 8; ++q) a[8 * h + q] = make_float2(__uint_as_float(r[2 * q]), __uint_as_float(r[2 * q + 1]));
-    tmem_ld16(taddr + 32 + h * 16, r);
-    tmem_ld_wait();
-#pragma unroll
-    for (int q = 0; q < 8; ++q)
-      a[8 * h + q] = make_float2(__fadd_rn(a[8 * h + q].x, __uint_as_float(r[2 * q])) * is,
-                                 __fadd_rn(a[8 * h + q].y, __uint_as_float(r[2 * q + 1])) * is);
+    for (int e = 0; e < 8; ++e)
+      a[8 * h + e] = __fmul2_rn(__fadd2_rn(make_float2(__uint_as_float(r[2 * e]), __uint_as_float(r[2 * e + 1])),
+                                           make_float2(__uint_as_float(q[2 * e]), __uint_as_float(q[2 * e + 1]))),
+                                is2);
   }
   tc_fence_before();
 }
 
 
 // Shared-memory tail of a tensor-core pass kernel (at the start of its dynamic
-// shared memory): the split radix-16 DFT matrices of both directions, the
-// mbarrier, the TMEM address word and the abort word.
+// shared memory): the split radix-16 DFT matrices of both directions, the TMEM
+// address word and per unit the mbarrier and the abort word.
 constexpr int kTcTail = 2 * TcGeom<16>::kGDir + 1024;
 
 // Set up a tensor-core pass: copy the split DFT matrices (kTcTail image made
 // by the plan, 16-byte aligned) into the tail, allocate the CTA's TMEM
-// columns (warp 0), initialise the mbarrier and clear the abort word.
-// ctl: the pass's control word (kTcStallMma).  Contains a block barrier.
+// columns (warp 0), initialise the units' mbarriers and clear their abort words.
+// ctl: the pass's control word (kTcStallMma); rn, a3_unit: see TcCtx.  Contains a block
+// barrier.
 __device__ __forceinline__ void tc_setup(TcCtx& tc, unsigned char* tail, const void* gmat, uint32_t a_tile,
-                                         int* err, int bf16, uint32_t a_tile3, int ctl) {
+                                         int* err, int bf16, uint32_t a_tile3, int ctl, int rn, uint32_t a3_unit) {
   const int nthr = blockDim.x * blockDim.y * blockDim.z;
   const int tid = (threadIdx.z * blockDim.y + threadIdx.y) * blockDim.x + threadIdx.x;
   constexpr int kG = 2 * TcGeom<16>::kGDir;
   for (int i = tid; i < kG / 16; i += nthr)
     reinterpret_cast<uint4*>(tail)[i] = __ldg(static_cast<const uint4*>(gmat) + i);
-  uint64_t* mb = reinterpret_cast<uint64_t*>(tail + kG);
+  // per unit (at most 8): the mbarrier and the abort word
+  uint64_t* mb = reinterpret_cast<uint64_t*>(tail + kG + 64) + tid / rn;
   uint32_t* slot = reinterpret_cast<uint32_t*>(tail + kG + 8);
-  int* abort_word = reinterpret_cast<int*>(tail + kG + 12);
-  if (tid == 0) *abort_word = 0;
+  int* abort_word = reinterpret_cast<int*>(tail + kG + 128) + tid / rn;
+  if (tid % rn == 0) {
+    *abort_word = 0;
+    mbar_init(smem_u32(mb), 1);
+  }
   if (tid < 32) {
     tmem_alloc(smem_u32(slot), (uint32_t)tc_tmem_cols(nthr));
     tc_fence_before();
   }
-  if (tid == 0) mbar_init(smem_u32(mb), 1);
   fence_async_smem();
   __syncthreads();
   tc_fence_after();
@@ -355,6 +374,8 @@ __device__ __forceinline__ void tc_setup(TcCtx& tc, unsigned char* tail, const v
   tc.tmem = *reinterpret_cast<volatile uint32_t*>(slot);
   tc.a_tile = a_tile;
   tc.a_tile3 = a_tile3;
+  tc.a3_unit = a3_unit;
+  tc.rn = rn;
   tc.bf16 = bf16;
   tc.bmat = smem_u32(tail);
   tc.phase = 0u;
@@ -364,17 +385,17 @@ __device__ __forceinline__ void tc_setup(TcCtx& tc, unsigned char* tail, const v
   tc.wait_iters = tc.stall ? kTestWaitIters : kWaitIters;
 }
 
-// Release the TMEM columns once every thread is done with them (block barrier).
+// Release the TMEM columns once every thread is done with them (block barriers).
 // After an expired wait (abort word set) the last commit may still be
-// outstanding: warp 0 first waits for it once more (bounded), then frees.
+// outstanding: its unit first waits for it once more (bounded), then warp 0 frees.
 __device__ __forceinline__ void tc_teardown(const TcCtx& tc) {
   const int nthr = blockDim.x * blockDim.y * blockDim.z;
   const int tid = (threadIdx.z * blockDim.y + threadIdx.y) * blockDim.x + threadIdx.x;
   tc_fence_before();
   __syncthreads();
+  if (*tc.abort) mbar_wait(tc.mbar, tc.phase ^ 1u, tc.wait_iters);  // the unit's last commit, if outstanding
+  __syncthreads();
   if (tid < 32) {
-    if (*tc.abort) mbar_wait(tc.mbar, tc.phase ^ 1u, tc.wait_iters);
-    __syncwarp();
     tc_fence_after();
     tmem_free(tc.tmem, (uint32_t)tc_tmem_cols(nthr));
   }
