@@ -85,6 +85,7 @@ struct psatd_plan_s {
   void* gmat = nullptr;       // their split DFT matrices (kTcTail image, device)
   int* d_err = nullptr;       // device error word of the tensor-core passes
   int64_t caller_elems = 0;   // elements of each caller array (checked mode's extents)
+  bool alone = true;          // no other class's passes run beside this plan's
   LocalMap loc = {};          // psatd_local_step: the caller's arrays are the global grid's (px = 0: off)
 };
 
@@ -500,6 +501,16 @@ cudaError_t inv_T_any(int L, bool c2r, const PassGeom& g, cudaStream_t st, const
   return cudaErrorInvalidValue;
 }
 
+// Whether the plan's passes are launched early (launch_pass): up to spectra of 1.5 L2
+// sizes (half an L2 with tensor cores), and not beside other classes, whose blocks the waiting
+// ones would displace.  Early against plain launches: 64^2 TE 12.8 / 19.5 us, 2048^2 139 /
+// 144, 128^3 eleven components 166 / 176; but 192^3 nine components 549 / 500, 2048^2 split
+// BF16 295 / 285, FP32 batch on two branches 9.6 / 9.0 ms.
+bool plan_early(psatd_plan p) {
+  const int64_t bytes = p->n_in * p->cs * (p->f32 ? 8 : 16);
+  return p->alone && bytes <= (p->tc ? (int64_t)64 << 20 : (int64_t)192 << 20);
+}
+
 // Arguments of the fused pass of plan p over the spectra at sp (lines of Lline
 // points, nlines of them).
 template <typename R>
@@ -530,6 +541,7 @@ PushArgs<R> make_push_args(psatd_plan p, void* sp, int Lline, int64_t nlines) {
   a.ic_l = (R)(ic - (double)a.ic_h);
   a.s_src = (R)(1.0 / (p->d.eps0 * c * p->g0));
   a.s_a6 = (R)(1.0 / (p->d.eps0 * c * c * p->g0));
+  a.early = plan_early(p) ? 1 : 0;
   a.gmat = p->gmat;
   a.err = p->d_err;
   a.tc_ctl = (p->d.flags & PSATD_FLAG_TEST_STALL_MMA) ? kTcStallMma : 0;
@@ -592,6 +604,7 @@ psatd_status run_step(psatd_plan p, const void* in[kMaxComp], void* out[kMaxComp
   // pass 1: x rows (R2C), b = y -> spec1 [c][kx][z][y] (3D) / [c][patch][kx][y] (2D)
   {
     PassGeom g;
+    g.early = plan_early(p);
     g.log_tb = rows_per_cta(p, 0);
     g.grid = dim3((unsigned)(ny >> g.log_tb), (unsigned)na0, (unsigned)p->n_in);
     g.smem = tail + tpass_smem(Lx, g.log_tb, 0, csz) + tc_a3_bytes(p, (Lx / row_ept(Lx, p->f32)) << g.log_tb);
@@ -613,6 +626,7 @@ psatd_status run_step(psatd_plan p, const void* in[kMaxComp], void* out[kMaxComp
   if (p->ndim == 3) {
     // pass 2: y lines (C2C), b = z, a0 = kx: spec1 [c][kx][z][y] -> spec2 [c][kx][ky][z]
     PassGeom g;
+    g.early = plan_early(p);
     g.log_tb = rows_per_cta(p, 1);
     g.grid = dim3((unsigned)(nz >> g.log_tb), (unsigned)nxh, (unsigned)p->n_in);
     g.smem = tail + tpass_smem((int)ny, g.log_tb, (size_t)ny, csz) +
@@ -647,6 +661,7 @@ psatd_status run_step(psatd_plan p, const void* in[kMaxComp], void* out[kMaxComp
   if (p->ndim == 3) {
     // pass 4: inverse y lines: spec2 [c][kx][ky][z] -> spec1 [c][kx][z][y]
     PassGeom g;
+    g.early = plan_early(p);
     g.log_tb = rows_per_cta(p, 2);
     g.grid = dim3((unsigned)(nz >> g.log_tb), (unsigned)nxh, (unsigned)p->n_out);
     g.smem = tail + tpass_smem((int)ny, g.log_tb, (size_t)ny, csz) +
@@ -664,6 +679,7 @@ psatd_status run_step(psatd_plan p, const void* in[kMaxComp], void* out[kMaxComp
   // last pass: inverse x rows (C2R): spec1 -> out [z][y][x] (3D) / packed patches (2D)
   {
     PassGeom g;
+    g.early = plan_early(p);
     g.log_tb = rows_per_cta(p, 3);
     g.grid = dim3((unsigned)(ny >> g.log_tb), (unsigned)na0, (unsigned)p->n_out);
     g.smem = tail + tpass_smem(Lx, g.log_tb, 0, csz) + tc_a3_bytes(p, (Lx / row_ept(Lx, p->f32)) << g.log_tb);
@@ -1984,6 +2000,7 @@ extern "C" psatd_status psatd_batch_create(const psatd_desc* base, int32_t npatc
       const int k = (int)(std::min_element(load.begin(), load.end()) - load.begin());
       load[k] += cells(i);
       b->cls[i]->st = b->br[k];
+      b->cls[i]->alone = false;
       b->branch_of[i] = k;
     }
   }
@@ -2090,8 +2107,10 @@ extern "C" psatd_status psatd_batch_set_branches(psatd_batch b, int32_t forked) 
   b->gexec = nullptr;
   b->graph = nullptr;
   b->fork_on = forked != 0;
-  for (size_t i = 0; i < b->cls.size(); ++i)
+  for (size_t i = 0; i < b->cls.size(); ++i) {
     b->cls[i]->st = (b->fork_on && !b->br.empty()) ? b->br[b->branch_of[i]] : b->st;
+    b->cls[i]->alone = !b->fork_on || b->br.empty();
+  }
   return PSATD_OK;
 }
 

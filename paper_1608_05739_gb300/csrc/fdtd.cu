@@ -17,8 +17,8 @@
 // of a call the second half step of B and the first of the next use the same E:
 // one pass subtracts the half step twice (the same two roundings), 2 N + 1 passes
 // for N steps instead of 3 N.  Against one cell per thread and 3 N passes: CKC TE 2048^2
-// with J, 8 steps 700 -> 188 us; Yee 256^3 with J, one step 549 -> 313 us (2.0 GB moved,
-// 6.4 TB/s).
+// with J, 8 steps 700 -> 156 us; Yee 256^3 with J, one step 549 -> 309 us (2.0 GB moved,
+// 6.5 TB/s).
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -101,6 +101,7 @@ __device__ __forceinline__ R half_step(R b, R h, R curl) {
 template <typename R, int V, bool CKC, bool TWICE>
 __global__ void __launch_bounds__(128) k_faraday2(FdtdGrid g, R* Bx, R* By, R* Bz, const R* Ex, const R* Ey,
                                                   const R* Ez, FdtdCoef<R> f) {
+  pass_begin();
   const int i0 = (blockIdx.x * blockDim.x + threadIdx.x) * V;
   const int j0 = (blockIdx.y * blockDim.y + threadIdx.y) * g.M;
   if (i0 >= g.nx || j0 >= g.ny) return;
@@ -162,6 +163,7 @@ __global__ void __launch_bounds__(128) k_faraday2(FdtdGrid g, R* Bx, R* By, R* B
 template <typename R, int V>
 __global__ void __launch_bounds__(128) k_ampere2(FdtdGrid g, R* Ex, R* Ey, R* Ez, const R* Bx, const R* By,
                                                  const R* Bz, const R* Jx, const R* Jy, const R* Jz, FdtdCoef<R> f) {
+  pass_begin();
   const int i0 = (blockIdx.x * blockDim.x + threadIdx.x) * V;
   const int j0 = (blockIdx.y * blockDim.y + threadIdx.y) * g.M;
   if (i0 >= g.nx || j0 >= g.ny) return;
@@ -212,6 +214,7 @@ __global__ void __launch_bounds__(128) k_ampere2(FdtdGrid g, R* Ex, R* Ey, R* Ez
 template <typename R, int V, bool TWICE>
 __global__ void __launch_bounds__(128) k_faraday3(FdtdGrid g, R* Bx, R* By, R* Bz, const R* Ex, const R* Ey,
                                                   const R* Ez, FdtdCoef<R> f) {
+  pass_begin();
   const int i0 = (blockIdx.x * blockDim.x + threadIdx.x) * V;
   const int j = blockIdx.y * blockDim.y + threadIdx.y;
   const int k0 = blockIdx.z * g.M;
@@ -246,6 +249,7 @@ __global__ void __launch_bounds__(128) k_faraday3(FdtdGrid g, R* Bx, R* By, R* B
 template <typename R, int V>
 __global__ void __launch_bounds__(128) k_ampere3(FdtdGrid g, R* Ex, R* Ey, R* Ez, const R* Bx, const R* By,
                                                  const R* Bz, const R* Jx, const R* Jy, const R* Jz, FdtdCoef<R> f) {
+  pass_begin();
   const int i0 = (blockIdx.x * blockDim.x + threadIdx.x) * V;
   const int j = blockIdx.y * blockDim.y + threadIdx.y;
   const int k0 = blockIdx.z * g.M;
@@ -286,33 +290,33 @@ static cudaError_t run_fdtd(int ndim, int scheme, int64_t nx, int64_t ny, int64_
   FdtdGrid g{(int)nx, (int)ny, (int)nz, nx * ny, 1};
   const int tx = (int)((nx + V - 1) / V);
   const unsigned bx = tx >= 128 ? 128u : tx >= 64 ? 64u : 32u, by = 128u / bx;
-  // rows / planes per thread: as many as leave each SM 512 threads, at most 8 (CKC), 4 (Yee);
-  // the marched rows' overlap is what is saved
+  // two rows / planes per thread where that leaves each SM 512 threads: the next row's
+  // values are loaded once; more rows make blocks too few for an even spread over the SMs
+  // (CKC TE 2048^2, eight steps with 2 / 4 / 8 rows 156 / 159 / 193 us; Yee 200^3 291 / 301 / 331)
   const int64_t march = ndim == 3 ? nz : ny, across = (int64_t)tx * (ndim == 3 ? ny : 1);
-  const int most = scheme == 1 ? 8 : 4;
-  while (g.M * 2 <= most && across * (march / (g.M * 2)) >= 152 * 512) g.M *= 2;
+  if (across * (march / 2) >= 152 * 512) g.M = 2;
   const unsigned gx = (unsigned)((tx + bx - 1) / bx);
   const dim3 block(bx, by);
   const int64_t span = (int64_t)by * (ndim == 3 ? 1 : g.M);
   const dim3 grid(gx, (unsigned)((ny + span - 1) / span), ndim == 3 ? (unsigned)((nz + g.M - 1) / g.M) : 1u);
   auto faraday = [&](bool twice) {
     if (ndim == 3) {
-      if (twice) k_faraday3<R, V, true><<<grid, block, 0, st>>>(g, b[0], b[1], b[2], e[0], e[1], e[2], f);
-      else k_faraday3<R, V, false><<<grid, block, 0, st>>>(g, b[0], b[1], b[2], e[0], e[1], e[2], f);
+      if (twice) launch_pass(true, k_faraday3<R, V, true>, grid, block, 0, st, g, b[0], b[1], b[2], e[0], e[1], e[2], f);
+      else launch_pass(true, k_faraday3<R, V, false>, grid, block, 0, st, g, b[0], b[1], b[2], e[0], e[1], e[2], f);
     } else if (scheme == 1) {
-      if (twice) k_faraday2<R, V, true, true><<<grid, block, 0, st>>>(g, b[0], b[1], b[2], e[0], e[1], e[2], f);
-      else k_faraday2<R, V, true, false><<<grid, block, 0, st>>>(g, b[0], b[1], b[2], e[0], e[1], e[2], f);
+      if (twice) launch_pass(true, k_faraday2<R, V, true, true>, grid, block, 0, st, g, b[0], b[1], b[2], e[0], e[1], e[2], f);
+      else launch_pass(true, k_faraday2<R, V, true, false>, grid, block, 0, st, g, b[0], b[1], b[2], e[0], e[1], e[2], f);
     } else {
-      if (twice) k_faraday2<R, V, false, true><<<grid, block, 0, st>>>(g, b[0], b[1], b[2], e[0], e[1], e[2], f);
-      else k_faraday2<R, V, false, false><<<grid, block, 0, st>>>(g, b[0], b[1], b[2], e[0], e[1], e[2], f);
+      if (twice) launch_pass(true, k_faraday2<R, V, false, true>, grid, block, 0, st, g, b[0], b[1], b[2], e[0], e[1], e[2], f);
+      else launch_pass(true, k_faraday2<R, V, false, false>, grid, block, 0, st, g, b[0], b[1], b[2], e[0], e[1], e[2], f);
     }
   };
   for (int s = 0; s < nsteps; ++s) {
     faraday(s > 0);
     if (ndim == 3)
-      k_ampere3<R, V><<<grid, block, 0, st>>>(g, e[0], e[1], e[2], b[0], b[1], b[2], j[0], j[1], j[2], f);
+      launch_pass(true, k_ampere3<R, V>, grid, block, 0, st, g, e[0], e[1], e[2], b[0], b[1], b[2], j[0], j[1], j[2], f);
     else
-      k_ampere2<R, V><<<grid, block, 0, st>>>(g, e[0], e[1], e[2], b[0], b[1], b[2], j[0], j[1], j[2], f);
+      launch_pass(true, k_ampere2<R, V>, grid, block, 0, st, g, e[0], e[1], e[2], b[0], b[1], b[2], j[0], j[1], j[2], f);
     cudaError_t err = cudaGetLastError();
     if (err != cudaSuccess) return err;
   }

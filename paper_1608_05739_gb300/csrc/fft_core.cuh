@@ -30,6 +30,14 @@
 
 namespace psatd {
 
+// First statement of a pass launched with launch_pass (launch.h): wait for the passes
+// before it (everything they wrote is visible then), and let the next one be scheduled.
+// Before any allocation of tensor memory, so that a waiting pass holds none.
+__device__ __forceinline__ void pass_begin() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 template <typename R> struct Types;
 template <> struct Types<float> {
   typedef float2 C;   // complex value

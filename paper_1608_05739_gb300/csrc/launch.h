@@ -11,10 +11,33 @@
 
 namespace psatd {
 
+// Launch of a pass that begins with pass_begin().  early: it may be scheduled while its
+// predecessor in the stream drains, and waits there for its completion (programmatic
+// dependent launch), which hides the launch latency and the drain of the last wave
+// between the passes of a step.  The blocks then fill the SMs as the predecessor frees
+// them, not evenly, so it pays for passes of many more blocks than fit at once, or short
+// ones (the plans' rule: plan_early in capi.cu).
+template <class... P, class... A>
+static inline cudaError_t launch_pass(bool early, void (*kern)(P...), dim3 grid, dim3 block, size_t smem,
+                                      cudaStream_t st, A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = early ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kern, P(args)...);
+}
+
 struct PassGeom {
   dim3 grid;
   int log_tb;      // lines per CTA = 1 << log_tb
   size_t smem;     // dynamic shared memory bytes
+  bool early = false;  // launch_pass
 };
 
 // a0_off: optional device table of per-patch element offsets into the caller's

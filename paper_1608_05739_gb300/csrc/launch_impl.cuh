@@ -31,11 +31,12 @@ static cudaError_t fwd_T_L_k(const PassGeom& g, cudaStream_t st, const LineIO& i
     const size_t smem = (size_t)pairs * L * sizeof(C2);
     auto kern = k_fwd_P<L, R2C, LOC>;
     if ((e = set_smem(kern, smem)) != cudaSuccess) return e;
-    kern<<<g.grid, dim3(T, pairs), smem, st>>>(io, static_cast<const W*>(tw), a, b, c, d, g.log_tb, off);
+    return launch_pass(g.early, kern, g.grid, dim3(T, pairs), smem, st, io, static_cast<const W*>(tw), a, b, c, d, g.log_tb, off);
   } else {
     auto kern = k_fwd_T<R, L, R2C, TC, LOC>;
     if ((e = set_smem(kern, g.smem)) != cudaSuccess) return e;
-    kern<<<g.grid, dim3(T, 1u << g.log_tb), g.smem, st>>>(io, static_cast<const W*>(tw), a, b, c, d, g.log_tb, off);
+    return launch_pass(g.early, kern, g.grid, dim3(T, 1u << g.log_tb), g.smem, st, io, static_cast<const W*>(tw), a, b, c, d,
+                       g.log_tb, off);
   }
   return cudaGetLastError();
 }
@@ -60,11 +61,12 @@ static cudaError_t inv_T_L_k(const PassGeom& g, cudaStream_t st, const LineIO& i
     const size_t smem = (size_t)pairs * L * sizeof(C2);
     auto kern = k_inv_P<L, C2R, LOC>;
     if ((e = set_smem(kern, smem)) != cudaSuccess) return e;
-    kern<<<g.grid, dim3(T, pairs), smem, st>>>(io, static_cast<const W*>(tw), a, b, c, d, g.log_tb, off);
+    return launch_pass(g.early, kern, g.grid, dim3(T, pairs), smem, st, io, static_cast<const W*>(tw), a, b, c, d, g.log_tb, off);
   } else {
     auto kern = k_inv_T<R, L, C2R, TC, LOC>;
     if ((e = set_smem(kern, g.smem)) != cudaSuccess) return e;
-    kern<<<g.grid, dim3(T, 1u << g.log_tb), g.smem, st>>>(io, static_cast<const W*>(tw), a, b, c, d, g.log_tb, off);
+    return launch_pass(g.early, kern, g.grid, dim3(T, 1u << g.log_tb), g.smem, st, io, static_cast<const W*>(tw), a, b, c, d,
+                       g.log_tb, off);
   }
   return cudaGetLastError();
 }
@@ -103,7 +105,7 @@ static cudaError_t push_L(int layout, dim3 grid, int tb, int groups, size_t smem
   {                                                                            \
     auto kern = push_kernel<R, TC, EPT, L, LAY, GRP>();                        \
     if ((e = set_smem(kern, smem)) != cudaSuccess) return e;                   \
-    kern<<<grid, block, smem, st>>>(a, static_cast<const W*>(tw));             \
+    return launch_pass(a.early != 0, kern, grid, block, smem, st, a, static_cast<const W*>(tw)); \
   }
 #define PSATD_PUSH_CASE(LAY)                                                   \
   case LAY: {                                                                  \

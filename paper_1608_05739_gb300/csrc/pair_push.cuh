@@ -360,6 +360,7 @@ __global__ void __launch_bounds__(GRP ? 512 : 256)
 k_line_pair(PushArgs<R> a, const typename Types<R>::W* __restrict__ tw) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ __align__(8) uint64_t stage_mbar;
+  pass_begin();
   const uint32_t mbar = smem_u32(&stage_mbar);
   if (threadIdx.x == 0 && threadIdx.y == 0 && threadIdx.z == 0) mbar_init(mbar, 1);
   line_pair_body<R, L, LAYOUT, EPT, GRP>(a, tw, (int)blockIdx.x, (int)threadIdx.x, (int)threadIdx.y, (int)blockDim.y,

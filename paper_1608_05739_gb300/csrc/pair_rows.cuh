@@ -55,6 +55,7 @@ __global__ void __launch_bounds__(RowPairThreads<L>::value, RowEPT<L>::value >= 
 k_fwd_P(LineIO io, const float4* __restrict__ tw, int64_t in_sa0, int64_t in_sb, int64_t out_sa0, int64_t out_sk,
         int log_tb, const int64_t* __restrict__ in_off) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  pass_begin();
   constexpr int EPT = RowEPT<L>::value;
   typedef FFTPlan<L, EPT> P;
   constexpr int T = P::kT;
@@ -159,6 +160,7 @@ __global__ void __launch_bounds__(RowPairThreads<L>::value, RowEPT<L>::value >= 
 k_inv_P(LineIO io, const float4* __restrict__ tw, int64_t in_sa0, int64_t in_sk, int64_t out_sa0, int64_t out_sb,
         int log_tb, const int64_t* __restrict__ out_off) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  pass_begin();
   constexpr int EPT = RowEPT<L>::value;
   typedef FFTPlan<L, EPT> P;
   constexpr int T = P::kT;

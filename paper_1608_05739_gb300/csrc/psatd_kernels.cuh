@@ -83,6 +83,8 @@ struct PushArgs {
   int stag;          // staggered order-p plan (PSATD-p): k_p and half-cell phases below
   const double* kp[3];  // per axis, k_p / g0 for |m| = 0..n/2
   const void* ph[3];    // per axis, exp(-i pi m/n) for m = 0..n/2 (twiddle type)
+  int early;            // host: launch_pass
+  int pad;
 };
 
 // Error-word bits of the checked mode (PSATD_FLAG_CHECKED): the non-finite scan
@@ -319,6 +321,7 @@ __global__ void __launch_bounds__(RowThreads<R, L>::value, sizeof(R) == 8 ? 1 : 
                                                int64_t in_sa0, int64_t in_sb, int64_t out_sa0,
                                                int64_t out_sk, int log_tb, const int64_t* __restrict__ in_off) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  pass_begin();
   TcCtx tc;
   constexpr int kRn = tc_unit_threads(FFTPlan<L, RowEPT<L, R>::value>::kT);
   if constexpr (TC)
@@ -482,6 +485,7 @@ __global__ void __launch_bounds__(RowThreads<R, L>::value, sizeof(R) == 8 ? 1 : 
                                                int64_t in_sa0, int64_t in_sk, int64_t out_sa0,
                                                int64_t out_sb, int log_tb, const int64_t* __restrict__ out_off) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  pass_begin();
   TcCtx tc;
   constexpr int kRn = tc_unit_threads(FFTPlan<L, RowEPT<L, R>::value>::kT);
   if constexpr (TC)
@@ -1090,6 +1094,7 @@ template <typename R, int L, int LAYOUT, int TC, int EPT, bool GRP>
 __global__ void __launch_bounds__(256, GRP ? 2 : 1)
 k_line_push(PushArgs<R> a, const typename Types<R>::W* __restrict__ tw) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  pass_begin();
   __shared__ __align__(8) uint64_t stage_mbar;
   StageCtx sc;
   stage_init(sc, &stage_mbar, a.err ? a.err : a.chk_err);
