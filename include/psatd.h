@@ -227,7 +227,8 @@ psatd_status psatd_plan_autotune(psatd_plan plan, int32_t reps, char* report, si
  *   cfg[0..3] log2(lines per CTA) of the x forward, y forward (3D), y inverse
  *             (3D) and x inverse passes (-1 / unused: 2D y passes);
  *   cfg[4]    lines per CTA of the fused pass;
- *   cfg[5]    its elements per thread: 8 (radix-8 stages), 16 (radix-16; the
+ *   cfg[5]    its elements per thread: 8 (radix-8 stages; FP64 lines of up to 128
+ *             points run it as radix-4 stages, 4 elements), 16 (radix-16; the
  *             built-in choice of FP32 lines of 1024 points and more and of the mixed
  *             precisions) or, for a last axis of 3 * 2^k points, 12 (radix 12, then
  *             2/4), of 5 * 2^k points 20 (radix 10 or 20, then 4).

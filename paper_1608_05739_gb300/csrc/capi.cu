@@ -365,13 +365,13 @@ int push_lines_per_cta(int L, int64_t nlines, bool tc, bool f32, int ept) {
   return tb;
 }
 
-// Component groups of the fused pass (psatd_kernels.cuh): 1, or 2 / 4 thread
-// groups per line taking the components in turn, for FP32 plans without
+// Component groups of the fused pass that a caller or the autotuner may choose: 1, or 2 / 4
+// thread groups per line taking the transform units in turn, for FP32 plans without
 // tensor-core stages whose lines have a multiple of 32 threads (named barriers
 // per group: at most 15 per CTA; at most 512 threads; an even number of modes
 // per thread in the push).
-// Tensor-core plans take G = 2 only: component pairs in lockstep, one 128-row
-// MMA group each (256 threads).
+// Tensor-core plans take G = 2 only: two units of 128 threads, one 128-row
+// MMA group each.
 bool push_groups_ok(int L, int ept, int tb, int G, bool tc, bool f32) {
   if (G == 1) return true;
   if (L < ept) return false;
@@ -380,10 +380,10 @@ bool push_groups_ok(int L, int ept, int tb, int G, bool tc, bool f32) {
   if (!f32 || (G != 2 && G != 4)) return false;
   return T % 32 == 0 && (ept / G) % 2 == 0 && T * tb * G <= 512 && tb * G <= 15;
 }
-// shared memory of the fused pass: per line the n_in slots and one second
-// exchange buffer per group (split-BF16's third A piece sits in a slot); the
-// tensor-core pairs exchange in their own slots and keep the one spare buffer
-// for the third A pieces
+// shared memory that the choice is checked against: per line the n_in slots and one second
+// exchange buffer per group (split-BF16's third A piece sits in a slot; two tensor-core units
+// exchange in their own slots and keep the one spare buffer for the third A pieces).
+// FP32 and FP64 kernels use the slots alone.
 size_t push_smem(int n_in, int L, int tb, int G, size_t csz, bool tc = false) {
   return (size_t)tb * ((size_t)n_in + (size_t)(tc ? 1 : G)) * (size_t)L * csz;
 }
@@ -404,6 +404,11 @@ int push_units_of(int layout, int n_in) {
 int push_groups_default(int layout, int L, int ept, int tb, int n_in, int64_t nlines, bool tc, bool f32, int sm_bytes) {
   if (tc) return push_groups_ok(L, ept, tb, 2, tc, f32) ? 2 : 1;
   if (L < ept || sm_bytes <= 0) return 1;
+  if (layout == PSATD_FIELDS_2D6 && push_sets(f32, (nlines + tb - 1) / tb)) {  // two sets, the larger of TE's components
+    layout = PSATD_FIELDS_2D_TE;
+    n_in = n_in == 6 ? 3 : n_in == 9 ? 5 : 7;
+    nlines *= 2;
+  }
   const int T = L / ept, thr = T * tb;
   if (!f32) {
     int G = 1;
@@ -431,14 +436,18 @@ size_t tc_a3_bytes(psatd_plan p, int threads) {
 // the plan's next step (the configured values, else the rules above)
 int64_t push_nlines(psatd_plan p) { return p->ndim == 3 ? p->nxh * p->ny : p->nxh * p->npatch; }
 int push_line_len(psatd_plan p) { return (int)(p->ndim == 3 ? p->nz : p->ny); }
+// elements per thread of the kernel (by the grid's lines: a batch gives the bits of its patches' own plans)
+int push_kept(psatd_plan p) {
+  return push_kernel_ept(push_line_len(p), p->push_ept, p->f32, p->ndim == 3 ? p->nxh * p->ny : p->nxh);
+}
 int push_tb(psatd_plan p) {
   return p->cfg_push_tb > 0 ? p->cfg_push_tb
-                            : push_lines_per_cta(push_line_len(p), push_nlines(p), p->tc, p->f32, p->push_ept);
+                            : push_lines_per_cta(push_line_len(p), push_nlines(p), p->tc, p->f32, push_kept(p));
 }
 int push_groups(psatd_plan p) {
   const int L = push_line_len(p), tb = push_tb(p);
   if (p->cfg_push_groups <= 0)
-    return push_groups_default(p->layout, L, p->push_ept, tb, p->n_in, push_nlines(p), p->tc, p->f32, p->sm_bytes);
+    return push_groups_default(p->layout, L, push_kept(p), tb, p->n_in, push_nlines(p), p->tc, p->f32, p->sm_bytes);
   return push_groups_ok(L, p->push_ept, tb, p->cfg_push_groups, p->tc, p->f32) ? p->cfg_push_groups : 1;
 }
 
@@ -502,13 +511,14 @@ cudaError_t inv_T_any(int L, bool c2r, const PassGeom& g, cudaStream_t st, const
 }
 
 // Whether the plan's passes are launched early (launch_pass): up to spectra of 1.5 L2
-// sizes (half an L2 with tensor cores), and not beside other classes, whose blocks the waiting
-// ones would displace.  Early against plain launches: 64^2 TE 12.8 / 19.5 us, 2048^2 139 /
-// 144, 128^3 eleven components 166 / 176; but 192^3 nine components 549 / 500, 2048^2 split
-// BF16 295 / 285, FP32 batch on two branches 9.6 / 9.0 ms.
+// sizes (half an L2 with tensor cores; FP64 1.5 MB), and not beside other classes, whose
+// blocks the waiting ones would displace.  Early against plain launches: 64^2 TE 12.8 / 19.5
+// us, 2048^2 139 / 144, 128^3 eleven components 166 / 176, FP64 128^2 26.7 / 30.7; but 192^3
+// nine components 549 / 500, 2048^2 split BF16 295 / 285, FP64 256^2 73 / 60 (blocks of the
+// FP64-bound passes spread unevenly), FP32 batch on two branches 9.6 / 9.0 ms.
 bool plan_early(psatd_plan p) {
   const int64_t bytes = p->n_in * p->cs * (p->f32 ? 8 : 16);
-  return p->alone && bytes <= (p->tc ? (int64_t)64 << 20 : (int64_t)192 << 20);
+  return p->alone && bytes <= (!p->f32 ? (int64_t)3 << 19 : p->tc ? (int64_t)64 << 20 : (int64_t)192 << 20);
 }
 
 // Arguments of the fused pass of plan p over the spectra at sp (lines of Lline
@@ -570,6 +580,8 @@ cudaError_t launch_push(psatd_plan p, int L, dim3 grid, int tb, int G, size_t sm
   }
   if (p->push_ept == 16) return launch_line_push<R, TC, 16, LS>(L, p->layout, grid, tb, G, smem, p->st, a, tw);
   if constexpr (TC == 0) {
+    if constexpr (std::is_same<R, double>::value)
+      if (push_kept(p) == 4) return launch_line_push<R, TC, 4, LS>(L, p->layout, grid, tb, G, smem, p->st, a, tw);
     if (p->push_ept == 8) return launch_line_push<R, TC, 8, LS>(L, p->layout, grid, tb, G, smem, p->st, a, tw);
   }
   return cudaErrorInvalidValue;
@@ -776,7 +788,7 @@ psatd_status regen_push_twiddles(psatd_plan p) {
   if (p->ndim < 2) return PSATD_OK;
   const int i = p->ndim - 1;
   const int L = (int)(i == 2 ? p->nz : p->ny);
-  cudaError_t e = launch_twiddles(p->tw[i], L, p->push_ept, false, p->f32, p->st);
+  cudaError_t e = launch_twiddles(p->tw[i], L, push_kept(p), false, p->f32, p->st);
   return e == cudaSuccess ? PSATD_OK : cuda_fail(p, e, "twiddle table launch");
 }
 
@@ -1096,7 +1108,7 @@ psatd_status psatd_coeffs_init(psatd_plan p) {
     for (int i = 0; i < p->ndim; ++i) {
       const int L = i == 0 ? (int)(ns[0] / 2) : (int)ns[i];
       const bool push_axis = (i == p->ndim - 1) && i > 0;
-      e = launch_twiddles(p->tw[i], L, push_axis ? p->push_ept : row_ept(L, p->f32), i == 0, p->f32, p->st);
+      e = launch_twiddles(p->tw[i], L, push_axis ? push_kept(p) : row_ept(L, p->f32), i == 0, p->f32, p->st);
       if (e != cudaSuccess) return cuda_fail(p, e, "twiddle table launch");
     }
     if (p->tc) {
@@ -1561,7 +1573,7 @@ extern "C" psatd_status psatd_step_noalloc(const psatd_desc* desc, const psatd_f
   for (int i = 0; i < p.ndim; ++i) {
     const int L = i == 0 ? (int)(ns[0] / 2) : (int)ns[i];
     const bool push_axis = (i == p.ndim - 1) && i > 0;
-    e = launch_twiddles(p.tw[i], L, push_axis ? p.push_ept : row_ept(L, p.f32), i == 0, p.f32, p.st);
+    e = launch_twiddles(p.tw[i], L, push_axis ? push_kept(&p) : row_ept(L, p.f32), i == 0, p.f32, p.st);
     if (e != cudaSuccess) return cuda_fail(nullptr, e, "twiddle table launch");
   }
   const double N = (double)p.nx * (double)p.ny * (double)p.nz;

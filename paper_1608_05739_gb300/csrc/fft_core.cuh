@@ -500,8 +500,20 @@ struct RowEPT { static constexpr int value = row_ept(L, sizeof(R) == 4); };
 __host__ __device__ constexpr int push_ept(int L, bool tc, bool f32) {
   return odd_factor(L) == 3 ? 12 : odd_factor(L) == 5 ? 20 : (tc || (f32 && L >= 1024)) ? 16 : 8;
 }
-template <int L, int TC, bool F32>
-struct PushEPT { static constexpr int value = push_ept(L, TC != 0, F32); };
+// Elements per thread that the fused pass's kernel runs for a plan's choice `ept` on grids of
+// nlines lines: in FP64 the radix-8 schedule runs as radix-4 stages of 4 elements up to 128
+// points (as many operations per level, half of them per thread: see row_ept; a step of 128^2
+// TE 59 -> 31 us, six components 47 -> 31), while a line stays one warp (256^2 TE 60 -> 69 us)
+// and, at 128 points, the grid leaves the schedulers idle (128^3 1902 -> 1918 us; 64 points,
+// 128 x 128 x 64: 956 -> 931 us).
+__host__ __device__ constexpr int push_kernel_ept(int L, int ept, bool f32, int64_t nlines) {
+  return !f32 && ept == 8 && (L <= 64 || (L == 128 && nlines * (L / 8) < 256 * 152)) ? 4 : ept;
+}
+
+// Whether the fused pass takes the six 2D components as two sets, each a block of its own
+// (pair_push.cuh): FP32 always; FP64, bound by its units, while every block has an SM to
+// itself (128^2 30.7 -> 26.7 us a step; 2048 x 256 479 -> 497).
+constexpr bool push_sets(bool f32, int64_t blocks) { return f32 || 2 * blocks <= 152; }
 
 // Power-of-two L: a radix-2/4/8 first stage when log2 L is not a multiple of
 // log2 EPT, then radix-EPT stages.  Mixed lengths take the odd factor and a power of

@@ -92,14 +92,18 @@ template <typename R, int TC, int EPT, int L, int LS>
 static cudaError_t push_L(int layout, dim3 grid, int tb, int groups, size_t smem, cudaStream_t st,
                           const PushArgs<R>& a, const void* tw) {
   typedef typename Types<R>::W W;
-  if constexpr (L < EPT) {
+  if constexpr (L < EPT || (EPT == 4 && L > 128)) {
     return cudaErrorInvalidValue;
   } else {
     const dim3 block(FFTPlan<L, EPT>::kT, tb, groups);
     // component groups: their own instantiation; FP32 groups are whole warps
     constexpr bool kGrpOk = TC ? EPT == 16 : true;
     if (groups > 1 && (!kGrpOk || (kPairs<R, TC> && (block.x * block.y) % 32 != 0))) return cudaErrorInvalidValue;
-    if constexpr (TC == 0) smem = (size_t)a.n_in * tb * L * 2 * sizeof(R);  // the units alone
+    if constexpr (TC == 0) {  // the units alone; the six 2D components: the larger set's
+      const bool sets = layout == 1 && push_sets(sizeof(R) == 4, grid.x);
+      smem = (size_t)(sets ? 3 + 2 * a.form : a.n_in) * tb * L * 2 * sizeof(R);
+      if (sets) grid.y = 2;
+    }
     cudaError_t e;
 #define PSATD_PUSH_LAUNCH(LAY, GRP)                                            \
   {                                                                            \

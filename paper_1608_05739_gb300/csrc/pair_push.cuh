@@ -19,7 +19,13 @@
 // wavefronts per SM, 46.9 M -> 35.0 M instructions), 256^3 with eleven components 439 ->
 // 371 us, 512 x 512 x 1024 9.47 -> 6.83 ms.  FP64 is bound by its units (half an operation
 // per cycle and scheduler): 128^2, six components, 97 us with two lines to a one-warp
-// CTA, 36 us with a line's components over six groups on an SM of its own.
+// CTA, 16 us with a line's two sets of components on SMs of their own, a group each
+// component.
+//
+// The six 2D components are two independent sets, (Ex, Ey, Bz) and (Ez, Bx, By) with
+// their sources: a CTA of that layout takes one of them (blockIdx.y) as the TE or TM
+// pass over its slots (MAP), with half the shared memory and twice the CTAs (push_sets;
+// FP32, 256^2 rho-form step 25.9 -> 19.3 us, 1024 x 512 47.4 -> 41.1).
 //
 // Component groups (GRP, G = blockDim.z): group j takes the units j, j + G, ...
 // (inverse: from G - 1 - j); the block meets before and after the push, whose
@@ -106,6 +112,7 @@ __device__ __forceinline__ void push_units(unsigned char* base, int us, int g1, 
   } else if constexpr (LAYOUT == 3) {
     push_tm<R>(s[0], s[1], s[2], s[3], mx, my, f, cS_h, cS_l, Sc_h, Sc_l, a, form);
   } else if constexpr (LAYOUT == 1) {
+    static_assert(sizeof(R) == 8, "FP32 runs the six 2D components as the TE and TM sets");
     push_te<R>(s[0], s[1], s[5], s[6], s[7], s[9], s[10], mx, my, f, cS_h, cS_l, Sc_h, Sc_l, a, form);
     push_tm<R>(s[2], s[3], s[4], s[8], mx, my, f, cS_h, cS_l, Sc_h, Sc_l, a, form);
   } else {
@@ -189,21 +196,30 @@ __device__ __forceinline__ void push_line_units(unsigned char* base, int us, int
   }
 }
 
+// Slot of component c of the TE (MAP 1) or TM (MAP 2) set of the six-component layout
+// (E0 E1 E2 B0 B1 B2 J0 J1 J2 rho rho'); MAP 0: the slot itself.
+template <int MAP>
+__device__ __forceinline__ int set_slot(int c) {
+  return MAP == 1 ? (c < 2 ? c : c == 2 ? 5 : c < 5 ? c + 3 : c + 4) : MAP == 2 ? (c < 3 ? c + 2 : 8) : c;
+}
+
 // Body of one CTA: line block bx (tb lines; line g of the block handled by the
 // threads (t, g, grp)); mbar / phase: the stage mbarrier and the parity of its
 // next phase.  Returns false when a failed index check left the phase unused.
-template <typename R, int L, int LAYOUT, int EPT, bool GRP>
+template <typename R, int L, int LAYOUT, int EPT, bool GRP, int MAP = 0>
 __device__ __forceinline__ bool line_pair_body(const PushArgs<R>& a_in, const typename Types<R>::W* __restrict__ tw, int bx,
                                                int t, int g, int tb, int grp, int G, unsigned char* smem_raw,
                                                uint32_t mbar, uint32_t phase) {
   const PushArgs<R> a = a_in;  // a private copy: its scalars stay in registers
+  const int n_in = MAP == 1 ? 3 + 2 * a.form : MAP == 2 ? 3 + (a.form >= 1 ? 1 : 0) : a.n_in;
+  const int n_out = MAP ? 3 : a.n_out;
   typedef typename Types<R>::C C;
   typedef typename Types<R>::W W;
   typedef FFTPlan<L, EPT> P;
   constexpr int CS = (int)sizeof(C);
   constexpr int T = P::kT;
   // twiddles one stage ahead where a stage's fit beside two transforms' elements
-  constexpr bool PF = EPT == 8 || EPT == 12;
+  constexpr bool PF = EPT <= 12;
   if constexpr (!GRP) {
     grp = 0;
     G = 1;
@@ -228,7 +244,7 @@ __device__ __forceinline__ bool line_pair_body(const PushArgs<R>& a_in, const ty
   // last are zero-filled
   const int nv = a.nlines - line0 < tb ? a.nlines - line0 : tb;  // valid lines of the block
   if (!valid)
-    for (int c = 0, w; c < a.n_in; c += w) {
+    for (int c = 0, w; c < n_in; c += w) {
       w = pair_width<R, LAYOUT>(c);
       float4* dst = reinterpret_cast<float4*>(smem_raw + c * us + w * g1);
       for (int i = t + grp * T; i < w * L * CS / 16; i += G * T) dst[i] = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -238,17 +254,17 @@ __device__ __forceinline__ bool line_pair_body(const PushArgs<R>& a_in, const ty
     constexpr uint32_t bytes = (uint32_t)(L * CS);
     if (tid == 0) {
       fence_async_smem();
-      mbar_arrive_expect_tx(mbar, (uint32_t)(nv * a.n_in) * bytes);
+      mbar_arrive_expect_tx(mbar, (uint32_t)(nv * n_in) * bytes);
     }
     __syncwarp();
     const int step = nthr < 32 ? nthr : 32;
-    for (int i = tid; i < nv * a.n_in; i += step) {
-      const int gl = i / a.n_in, c = i - gl * a.n_in;
+    for (int i = tid; i < nv * n_in; i += step) {
+      const int gl = i / n_in, c = i - gl * n_in;
       const bool second = c > 0 && pair_start<R, LAYOUT>(c - 1);
       const int c0 = second ? c - 1 : c;
       const int w = pair_width<R, LAYOUT>(c0);
       bulk_copy_g2s(smem_u32(smem_raw + c0 * us + (gl * w + (second ? 1 : 0)) * (L * CS)),
-                    spec + c * a.cs + (int64_t)(line0 + gl) * L, bytes, mbar);
+                    spec + set_slot<MAP>(c) * a.cs + (int64_t)(line0 + gl) * L, bytes, mbar);
     }
   }
   int mxi, myi, rowi;
@@ -275,7 +291,7 @@ __device__ __forceinline__ bool line_pair_body(const PushArgs<R>& a_in, const ty
   }
 
 #pragma unroll 1
-  for (int c = 0, u = 0, w; c < a.n_in; c += w, ++u) {
+  for (int c = 0, u = 0, w; c < n_in; c += w, ++u) {
     w = pair_width<R, LAYOUT>(c);
     if (GRP && u % G != grp) continue;
     if constexpr (sizeof(R) == 4) {
@@ -318,10 +334,11 @@ __device__ __forceinline__ bool line_pair_body(const PushArgs<R>& a_in, const ty
   if (G > 1) __syncthreads();  // every mode is pushed
 
 #pragma unroll 1
-  for (int c = 0, u = 0, w; c < a.n_out; c += w, ++u) {
+  for (int c = 0, u = 0, w; c < n_out; c += w, ++u) {
     w = pair_width<R, LAYOUT>(c);
     if (GRP && u % G != G - 1 - grp) continue;
-    C* dst = spec + c * a.cs + (int64_t)line * L;
+    C* dst = spec + set_slot<MAP>(c) * a.cs + (int64_t)line * L;
+    [[maybe_unused]] const int64_t next = (set_slot<MAP>(c + 1) - set_slot<MAP>(c)) * a.cs;  // a pair's second
     if constexpr (sizeof(R) == 4) {
       if (w == 2) {
         C2* buf = reinterpret_cast<C2*>(smem_raw + c * us + g2);
@@ -333,7 +350,7 @@ __device__ __forceinline__ bool line_pair_body(const PushArgs<R>& a_in, const ty
 #pragma unroll
           for (int m = 0; m < EPT; ++m) {
             dst[t + T * m] = make_float2(v[m].x.a, v[m].y.a);
-            dst[a.cs + t + T * m] = make_float2(v[m].x.b, v[m].y.b);
+            dst[next + t + T * m] = make_float2(v[m].x.b, v[m].y.b);
           }
         }
         continue;
@@ -352,19 +369,31 @@ __device__ __forceinline__ bool line_pair_body(const PushArgs<R>& a_in, const ty
   return true;
 }
 
-// Block (T, lines per CTA, component groups); up to 512 threads (128 registers), or 256
+// Grid (line blocks, sets: 2 for the six 2D components), block (T, lines per CTA,
+// component groups); up to 512 threads (128 registers), or 256
 // without groups (GRP false).  Groups are whole warps: with several, T times the lines
 // per CTA is a multiple of 32.
 template <typename R, int L, int LAYOUT, int EPT, bool GRP>
-__global__ void __launch_bounds__(GRP ? 512 : 256)
+__global__ void __launch_bounds__(GRP || EPT == 4 ? 512 : 256)
 k_line_pair(PushArgs<R> a, const typename Types<R>::W* __restrict__ tw) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ __align__(8) uint64_t stage_mbar;
   pass_begin();
   const uint32_t mbar = smem_u32(&stage_mbar);
   if (threadIdx.x == 0 && threadIdx.y == 0 && threadIdx.z == 0) mbar_init(mbar, 1);
-  line_pair_body<R, L, LAYOUT, EPT, GRP>(a, tw, (int)blockIdx.x, (int)threadIdx.x, (int)threadIdx.y, (int)blockDim.y,
-                                      (int)threadIdx.z, (int)blockDim.z, smem_raw, mbar, 0u);
+  auto body = [&](auto lay, auto map) {
+    line_pair_body<R, L, decltype(lay)::value, EPT, GRP, decltype(map)::value>(
+        a, tw, (int)blockIdx.x, (int)threadIdx.x, (int)threadIdx.y, (int)blockDim.y, (int)threadIdx.z, (int)blockDim.z,
+        smem_raw, mbar, 0u);
+  };
+  if constexpr (LAYOUT == 1) {
+    if (sizeof(R) == 4 || gridDim.y == 2) {
+      if (blockIdx.y == 0) body(std::integral_constant<int, 2>{}, std::integral_constant<int, 1>{});
+      else body(std::integral_constant<int, 3>{}, std::integral_constant<int, 2>{});
+      return;
+    }
+  }
+  if constexpr (LAYOUT != 1 || sizeof(R) == 8) body(std::integral_constant<int, LAYOUT>{}, std::integral_constant<int, 0>{});
 }
 
 }  // namespace psatd

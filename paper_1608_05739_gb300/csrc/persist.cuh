@@ -165,10 +165,18 @@ __global__ void __launch_bounds__(kPersistThreads, TC ? 2 : 4) k_persist_push(co
     if constexpr (TC) {                                                                                    \
       line_push_body<R, LL, LAYOUT, TC, EPT>(A, tw, it.blk, t, g, kPersistThreads / T, 0, 1, smem_raw, tc, sc); \
     } else {                                                                                               \
-      __syncthreads(); /* the previous item's shared memory is free */                                     \
-      if (line_pair_body<R, LL, LAYOUT, EPT, false>(A, tw, it.blk, t, g, kPersistThreads / T, 0, 1, smem_raw, sc.mbar, \
-                                                 sc.phase))                                                 \
-        sc.phase ^= 1u;                                                                                    \
+      auto part = [&](auto lay, auto map) {                                                                \
+        __syncthreads(); /* the previous part's shared memory is free */                                   \
+        if (line_pair_body<R, LL, decltype(lay)::value, EPT, false, decltype(map)::value>(                 \
+                A, tw, it.blk, t, g, kPersistThreads / T, 0, 1, smem_raw, sc.mbar, sc.phase))              \
+          sc.phase ^= 1u;                                                                                  \
+      };                                                                                                   \
+      if constexpr (LAYOUT == 1) {                                                                         \
+        part(std::integral_constant<int, 2>{}, std::integral_constant<int, 1>{});                          \
+        part(std::integral_constant<int, 3>{}, std::integral_constant<int, 2>{});                          \
+      } else {                                                                                             \
+        part(std::integral_constant<int, LAYOUT>{}, std::integral_constant<int, 0>{});                     \
+      }                                                                                                    \
     }                                                                                                      \
   }
       PSATD_PERSIST_Y_LENGTHS(FAM, PSATD_Y_CASE)

@@ -1,5 +1,8 @@
-// psatd_kernels.cuh -- the PSATD step's pass kernels (templates; instantiated
-// per precision and variant by the rows_* / push_* translation units).
+// psatd_kernels.cuh -- the PSATD step's pass kernels of one line per T threads (templates;
+// instantiated per precision and variant by the rows_* / push_* translation units): the x and
+// y passes of FP64 and of the tensor-core variants, the tensor-core variants' fused pass,
+// and the push arithmetic of all.  FP32 rows: pair_rows.cuh; the FP32 and FP64 fused
+// pass: pair_push.cuh (same data flow).
 //
 // Data flow of one step (2D: passes 1, 3, 5; 3D: passes 1-5):
 //   1  k_fwd_T<R2C>  x-rows of every input array -> R2C -> half spectrum,

@@ -4,4 +4,6 @@
 namespace psatd {
 template cudaError_t launch_line_push<double, false, 8, 1>(int, int, dim3, int, int, size_t, cudaStream_t,
                                               const PushArgs<double>&, const void*);
+template cudaError_t launch_line_push<double, false, 4, 1>(int, int, dim3, int, int, size_t, cudaStream_t,
+                                              const PushArgs<double>&, const void*);
 }  // namespace psatd

@@ -16,6 +16,8 @@ CASES = [
     ((8, 16), "te", "J"), ((16, 32), "2d6", "rho"), ((32, 64), "tm", "none"), ((128, 128), "2d6", "none"),
     ((64, 256), "te", "rho"), ((128, 1024), "te", "J"), ((8, 8, 16), "3d6", "J"), ((16, 64, 32), "3d6", "rho"),
     ((16, 4096), "tm", "J"), ((2048, 32), "te", "none"),
+    ((64, 256), "2d6", "rho"),  # 129 blocks: the six components whole
+    ((128, 64, 128), "3d6", "none"),  # radix-8 stages in the last axis
 ]
 
 
@@ -37,3 +39,23 @@ def test_fp64_split(shape, layout, src):
     E1, B1 = psatd_gpu(shape, d, dt, E, B, J, r0, r1, layout=layout, prec="fp64", src=src, plan=plan)
     assert np.array_equal(E1, Eg) and np.array_equal(B1, Bg)
     plan.destroy()
+
+
+def test_six_components_as_two_sets_equal_the_whole():
+    """65 lines of a 128 x 128 plan run as the TE and TM sets, three patches' 195 lines with the six
+    components in a block: the same operations, the same bits."""
+    import torch
+    ensure_lib()
+    shape, d, dt, n = (128, 128), (1.0, 0.9), 0.4, 3
+    E, B, J = (synth.random_fields(shape, 3, s) for s in (91, 92, 93))
+    r0, r1 = (synth.random_fields(shape, 1, s)[0] for s in (94, 95))
+    one = psatd_gpu(shape, d, dt, E, B, J, r0, r1, layout="2d6", prec="fp64", src="rho")
+    rep = lambda a: torch.from_numpy(np.concatenate([a.ravel()] * n)).cuda()
+    Et, Bt, Jt = ([rep(a) for a in f] for f in (E, B, J))
+    batch = capi.Batch([(128, 128)] * n, d, dt, layout="2d6", prec="fp64", src="rho")
+    batch.step(Et, Bt, Jt, rep(r0), rep(r1))
+    torch.cuda.synchronize()
+    for got, want in zip(Et + Bt, list(one[0]) + list(one[1])):
+        for p in got.cpu().numpy().reshape(n, *shape):
+            assert np.array_equal(p, want)
+    batch.destroy()
