@@ -319,7 +319,7 @@ psatd_status fdtd_step(const psatd_desc* desc, int32_t scheme, const psatd_field
  * sum_{j<i} n[2j] n[2j+1]).
  * Patches of equal size form a class (own spectra and tables).  A step runs
  * the persistent passes below where the sizes allow; else one launch per pass
- * and class, forked from the batch's stream into up to four (FP32: two) internal streams
+ * and class, forked from the batch's stream into up to eight internal streams
  * that run the classes side by side, and joined back.  A call with nsteps > 1 on a
  * non-default stream records one step of all classes into a CUDA graph
  * (re-recorded when the field/source pointers change) and replays it nsteps

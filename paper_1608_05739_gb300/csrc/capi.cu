@@ -1980,11 +1980,14 @@ extern "C" psatd_status psatd_batch_create(const psatd_desc* base, int32_t npatc
       return s;
     }
   }
-  // branch streams, classes assigned largest first to the least loaded branch: 4, or 2 in FP32, whose
-  // passes fill the SMs' registers by themselves and keep their class's spectra in L2 with fewer classes
-  // in flight (512 patches, four steps with 1 / 2 / 3 / 4 / 8 branches: FP32 10.6 / 9.0 / 9.3 / 9.4 / 10.6
-  // ms, split BF16 23.2 / 22.3 / - / 22.2 / 22.4 ms)
-  const int nbr = (int)std::min<size_t>(b->f32 && !b->cls[0]->tc ? 2 : 4, b->cls.size());
+  // Branch streams, classes assigned largest first to the least loaded branch.  Many classes in flight
+  // fill the SMs when the batch is small; few keep their spectra in L2 when it is large.  Measured, us a
+  // step with 1 / 2 / 3 / 4 / 6 / 8 branches: FP32 16 patches 239 / 159 / 139 / 140 / 137 / 131, 64 patches
+  // (8.9 M cells) 658 / 482 / 424 / 398 / 377 / 408, 128 (18 M) 1063 / 782 / 707 / 710 / 733 / 726, 512 2659 /
+  // 2266 / 2205 / 2331 / 2429 / 2431; split BF16 32 patches (6 M) 635 / 600 / 499 / 449 / 464 / 405, 64 (12 M)
+  // 1031 / 1006 / 777 / 722 / 739 / 763, 512 5305 / 5123 / 4992 / 5018 / 5057 / 5020.
+  const int branches = !b->f32 ? 4 : b->cls[0]->tc ? (acc < 8000000 ? 8 : 4) : (acc < 13000000 ? 6 : 3);
+  const int nbr = (int)std::min<size_t>(branches, b->cls.size());
   if (nbr > 1) {
     cudaError_t e = cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming);
     for (int k = 0; k < nbr && e == cudaSuccess; ++k) {
