@@ -436,6 +436,17 @@ size_t tc_a3_bytes(psatd_plan p, int threads) {
 // the plan's next step (the configured values, else the rules above)
 int64_t push_nlines(psatd_plan p) { return p->ndim == 3 ? p->nxh * p->ny : p->nxh * p->npatch; }
 int push_line_len(psatd_plan p) { return (int)(p->ndim == 3 ? p->nz : p->ny); }
+// Whether the rows of an axis (0 x, 1 y) of a 3D grid run 16 FP64 elements per thread: grids
+// with 512 such threads per SM (128 x 128 x 32, 99 thousand: y passes 86 us with 4 elements, 77 with 16).
+bool row_is_wide(psatd_plan p, int axis) {
+  const int L = (int)(axis == 0 ? p->nx / 2 : p->ny);
+  const int64_t rows = axis == 0 ? p->ny * p->nz : p->nxh * p->nz;
+  return p->ndim == 3 && row_wide(L, p->f32) && rows * p->n_out * (L / 16) >= 512 * kSMs;
+}
+int row_kept(psatd_plan p, int axis) {
+  const int L = (int)(axis == 0 ? p->nx / 2 : p->ny);
+  return row_is_wide(p, axis) ? 16 : row_ept(L, p->f32);
+}
 // elements per thread of the kernel (by the grid's lines: a batch gives the bits of its patches' own plans)
 int push_kept(psatd_plan p) {
   return push_kernel_ept(push_line_len(p), p->push_ept, p->f32, p->ndim == 3 ? p->nxh * p->ny : p->nxh);
@@ -618,6 +629,7 @@ psatd_status run_step(psatd_plan p, const void* in[kMaxComp], void* out[kMaxComp
     PassGeom g;
     g.early = plan_early(p);
     g.log_tb = rows_per_cta(p, 0);
+    g.wide = row_is_wide(p, 0);
     g.grid = dim3((unsigned)(ny >> g.log_tb), (unsigned)na0, (unsigned)p->n_in);
     g.smem = tail + tpass_smem(Lx, g.log_tb, 0, csz) + tc_a3_bytes(p, (Lx / row_ept(Lx, p->f32)) << g.log_tb);
     for (int c = 0; c < p->n_in; ++c) {
@@ -640,6 +652,7 @@ psatd_status run_step(psatd_plan p, const void* in[kMaxComp], void* out[kMaxComp
     PassGeom g;
     g.early = plan_early(p);
     g.log_tb = rows_per_cta(p, 1);
+    g.wide = row_is_wide(p, 1);
     g.grid = dim3((unsigned)(nz >> g.log_tb), (unsigned)nxh, (unsigned)p->n_in);
     g.smem = tail + tpass_smem((int)ny, g.log_tb, (size_t)ny, csz) +
              tc_a3_bytes(p, ((int)ny / row_ept((int)ny, p->f32)) << g.log_tb);
@@ -675,6 +688,7 @@ psatd_status run_step(psatd_plan p, const void* in[kMaxComp], void* out[kMaxComp
     PassGeom g;
     g.early = plan_early(p);
     g.log_tb = rows_per_cta(p, 2);
+    g.wide = row_is_wide(p, 1);
     g.grid = dim3((unsigned)(nz >> g.log_tb), (unsigned)nxh, (unsigned)p->n_out);
     g.smem = tail + tpass_smem((int)ny, g.log_tb, (size_t)ny, csz) +
              tc_a3_bytes(p, ((int)ny / row_ept((int)ny, p->f32)) << g.log_tb);
@@ -693,6 +707,7 @@ psatd_status run_step(psatd_plan p, const void* in[kMaxComp], void* out[kMaxComp
     PassGeom g;
     g.early = plan_early(p);
     g.log_tb = rows_per_cta(p, 3);
+    g.wide = row_is_wide(p, 0);
     g.grid = dim3((unsigned)(ny >> g.log_tb), (unsigned)na0, (unsigned)p->n_out);
     g.smem = tail + tpass_smem(Lx, g.log_tb, 0, csz) + tc_a3_bytes(p, (Lx / row_ept(Lx, p->f32)) << g.log_tb);
     for (int c = 0; c < p->n_out; ++c) {
@@ -1108,7 +1123,7 @@ psatd_status psatd_coeffs_init(psatd_plan p) {
     for (int i = 0; i < p->ndim; ++i) {
       const int L = i == 0 ? (int)(ns[0] / 2) : (int)ns[i];
       const bool push_axis = (i == p->ndim - 1) && i > 0;
-      e = launch_twiddles(p->tw[i], L, push_axis ? push_kept(p) : row_ept(L, p->f32), i == 0, p->f32, p->st);
+      e = launch_twiddles(p->tw[i], L, push_axis ? push_kept(p) : row_kept(p, i), i == 0, p->f32, p->st);
       if (e != cudaSuccess) return cuda_fail(p, e, "twiddle table launch");
     }
     if (p->tc) {
@@ -1573,7 +1588,7 @@ extern "C" psatd_status psatd_step_noalloc(const psatd_desc* desc, const psatd_f
   for (int i = 0; i < p.ndim; ++i) {
     const int L = i == 0 ? (int)(ns[0] / 2) : (int)ns[i];
     const bool push_axis = (i == p.ndim - 1) && i > 0;
-    e = launch_twiddles(p.tw[i], L, push_axis ? push_kept(&p) : row_ept(L, p.f32), i == 0, p.f32, p.st);
+    e = launch_twiddles(p.tw[i], L, push_axis ? push_kept(&p) : row_kept(&p, i), i == 0, p.f32, p.st);
     if (e != cudaSuccess) return cuda_fail(nullptr, e, "twiddle table launch");
   }
   const double N = (double)p.nx * (double)p.ny * (double)p.nz;

@@ -480,14 +480,19 @@ __host__ __device__ constexpr bool is_pow2(int v) { return v > 0 && (v & (v - 1)
 // batch of 512 patches 10.1 -> 9.4 ms per four steps), and 24 beyond (1536 points: 121
 // us, with 12 131; 768 points: 19.0, with 12 20.6).  The fused pass takes 12 for 3 * 2^k.
 __host__ __device__ constexpr int odd_factor(int v) { return is_pow2(v) ? 1 : (v % 3 == 0 ? 3 : 5); }
-// FP64 takes as few as fit its threads, 4 up to 1024 points: radix-4 stages need no more
-// operations per level than radix 16, and at 2 FP64 operations per cycle and SM (half an
+// FP64 takes as few as fit its threads, 4 up to 1024 points: radix-4 butterflies need no more
+// operations per level than radix 16 (their twiddle products come on top), and at 2 FP64 operations per cycle and SM (half an
 // operation per scheduler, so 64 cycles per warp instruction) a small grid's time is
 // the instructions of one thread (x forward of 128^2, 6 components: 22.6 us with 16
-// elements per thread); the extra exchanges cost a tenth of that.
+// elements per thread); the extra exchanges cost a tenth of that.  Large 3D grids, whose
+// passes keep the FP64 units busy, run 128- and 256-point rows with 16 all the same (row_wide;
+// a third of the twiddle products: 256 x 128 x 128 J-form, x forward 1072 -> 980 us, y forward
+// 833 -> 737, y inverse 552 -> 487, x inverse 748 -> 639).
 __host__ __device__ constexpr int row_ept(int L, bool f32) {
   return !f32 ? (L <= 1024 ? 4 : L / 256) : odd_factor(L) == 3 ? (L <= 384 ? 12 : 24) : odd_factor(L) == 5 ? 20 : L >= 16 ? 16 : 8;
 }
+// lengths that also have a 16-element variant
+__host__ __device__ constexpr bool row_wide(int L, bool f32) { return !f32 && (L == 128 || L == 256); }
 template <int L, typename R = float>
 struct RowEPT { static constexpr int value = row_ept(L, sizeof(R) == 4); };
 // Elements per thread of the fused pass by default.  8 (radix-8 stages) up to 512

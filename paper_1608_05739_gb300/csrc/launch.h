@@ -38,6 +38,7 @@ struct PassGeom {
   int log_tb;      // lines per CTA = 1 << log_tb
   size_t smem;     // dynamic shared memory bytes
   bool early = false;  // launch_pass
+  bool wide = false;   // 16 elements per thread (row_wide lengths)
 };
 
 // a0_off: optional device table of per-patch element offsets into the caller's

@@ -33,6 +33,14 @@ static cudaError_t fwd_T_L_k(const PassGeom& g, cudaStream_t st, const LineIO& i
     if ((e = set_smem(kern, smem)) != cudaSuccess) return e;
     return launch_pass(g.early, kern, g.grid, dim3(T, pairs), smem, st, io, static_cast<const W*>(tw), a, b, c, d, g.log_tb, off);
   } else {
+    if constexpr (row_wide(L, sizeof(R) == 4) && !LOC) {
+      if (g.wide) {
+        auto kern = k_fwd_T<R, L, R2C, TC, LOC, 16>;
+        if ((e = set_smem(kern, g.smem)) != cudaSuccess) return e;
+        return launch_pass(g.early, kern, g.grid, dim3(L / 16, 1u << g.log_tb), g.smem, st, io, static_cast<const W*>(tw), a,
+                           b, c, d, g.log_tb, off);
+      }
+    }
     auto kern = k_fwd_T<R, L, R2C, TC, LOC>;
     if ((e = set_smem(kern, g.smem)) != cudaSuccess) return e;
     return launch_pass(g.early, kern, g.grid, dim3(T, 1u << g.log_tb), g.smem, st, io, static_cast<const W*>(tw), a, b, c, d,
@@ -63,6 +71,14 @@ static cudaError_t inv_T_L_k(const PassGeom& g, cudaStream_t st, const LineIO& i
     if ((e = set_smem(kern, smem)) != cudaSuccess) return e;
     return launch_pass(g.early, kern, g.grid, dim3(T, pairs), smem, st, io, static_cast<const W*>(tw), a, b, c, d, g.log_tb, off);
   } else {
+    if constexpr (row_wide(L, sizeof(R) == 4) && !LOC) {
+      if (g.wide) {
+        auto kern = k_inv_T<R, L, C2R, TC, LOC, 16>;
+        if ((e = set_smem(kern, g.smem)) != cudaSuccess) return e;
+        return launch_pass(g.early, kern, g.grid, dim3(L / 16, 1u << g.log_tb), g.smem, st, io, static_cast<const W*>(tw), a,
+                           b, c, d, g.log_tb, off);
+      }
+    }
     auto kern = k_inv_T<R, L, C2R, TC, LOC>;
     if ((e = set_smem(kern, g.smem)) != cudaSuccess) return e;
     return launch_pass(g.early, kern, g.grid, dim3(T, 1u << g.log_tb), g.smem, st, io, static_cast<const W*>(tw), a, b, c, d,

@@ -122,9 +122,9 @@ __global__ void k_nonfinite(NfPtrs ptrs, const int64_t* __restrict__ off, int64_
 
 // Threads per CTA a transposing pass of length L may use (the register budget
 // of 20 or 24 elements per thread halves it; FP64: 4096 elements).
-template <typename R, int L>
+template <typename R, int L, int EPT = RowEPT<L, R>::value>
 struct RowThreads {
-  static constexpr int value = sizeof(R) == 8 ? 4096 / RowEPT<L, R>::value : RowEPT<L, R>::value >= 20 ? 256 : 512;
+  static constexpr int value = sizeof(R) == 8 ? 4096 / EPT : EPT >= 20 ? 256 : 512;
 };
 
 // XOR mask of row r's buffer in the transposed stores and reads (TB = 1 << log_tb
@@ -190,13 +190,12 @@ struct RowCta {
   int64_t nb;
 };
 
-template <typename R, int L, bool R2C, int TC, bool PART, bool LOC = false>
+template <typename R, int L, bool R2C, int TC, bool PART, bool LOC = false, int EPT = RowEPT<L, R>::value>
 __device__ __forceinline__ void fwd_T_body(const LineIO& io, const typename Types<R>::W* __restrict__ tw,
                                            int64_t in_sa0, int64_t in_sb, int64_t out_sa0, int64_t out_sk,
                                            const int64_t* __restrict__ in_off, const RowCta& cta,
                                            unsigned char* smem_raw, TcCtx& tc) {
   typedef typename Types<R>::C C;
-  constexpr int EPT = RowEPT<L, R>::value;
   typedef FFTPlan<L, EPT> P;
   constexpr int T = P::kT;
   constexpr int NK = R2C ? L + 1 : L;
@@ -319,8 +318,8 @@ __device__ __forceinline__ void fwd_T_body(const LineIO& io, const typename Type
 // Launch bounds: two CTAs of the largest block per SM (at most 64 registers a
 // thread).  The tensor-core variants then keep part of each row on the stack,
 // but measured faster so than with 128 registers and half the resident warps.
-template <typename R, int L, bool R2C, int TC = 0, bool LOC = false>
-__global__ void __launch_bounds__(RowThreads<R, L>::value, sizeof(R) == 8 ? 1 : 2) k_fwd_T(LineIO io, const typename Types<R>::W* __restrict__ tw,
+template <typename R, int L, bool R2C, int TC = 0, bool LOC = false, int EPT = RowEPT<L, R>::value>
+__global__ void __launch_bounds__(RowThreads<R, L, EPT>::value, sizeof(R) == 8 ? 1 : 2) k_fwd_T(LineIO io, const typename Types<R>::W* __restrict__ tw,
                                                int64_t in_sa0, int64_t in_sb, int64_t out_sa0,
                                                int64_t out_sk, int log_tb, const int64_t* __restrict__ in_off) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -331,7 +330,7 @@ __global__ void __launch_bounds__(RowThreads<R, L>::value, sizeof(R) == 8 ? 1 : 
     tc_setup(tc, smem_raw, io.gmat, 0u, io.err, TC == 2, 0u, io.tc_ctl, kRn, kRn / 128 * TcGeom<16>::kAPiece);
   const RowCta cta{(int)blockIdx.x, (int)blockIdx.y, (int)blockIdx.z, (int)threadIdx.x, (int)threadIdx.y, log_tb,
                    (int64_t)gridDim.x << log_tb};
-  fwd_T_body<R, L, R2C, TC, false, LOC>(io, tw, in_sa0, in_sb, out_sa0, out_sk, in_off, cta, smem_raw, tc);
+  fwd_T_body<R, L, R2C, TC, false, LOC, EPT>(io, tw, in_sa0, in_sb, out_sa0, out_sk, in_off, cta, smem_raw, tc);
   if constexpr (TC) tc_teardown(tc);
 }
 
@@ -340,13 +339,12 @@ __global__ void __launch_bounds__(RowThreads<R, L>::value, sizeof(R) == 8 ? 1 : 
 // in[a1] + a0*in_sa0 + k*in_sk + b, inverse FFT along k, write the lines
 // contiguously to out[a1] + a0*out_sa0 + b*out_sb.  C2R: L+1 Hermitian bins
 // in, real rows of length 2L out (unnormalised).
-template <typename R, int L, bool C2R, int TC, bool PART, bool LOC = false>
+template <typename R, int L, bool C2R, int TC, bool PART, bool LOC = false, int EPT = RowEPT<L, R>::value>
 __device__ __forceinline__ void inv_T_body(const LineIO& io, const typename Types<R>::W* __restrict__ tw,
                                            int64_t in_sa0, int64_t in_sk, int64_t out_sa0, int64_t out_sb,
                                            const int64_t* __restrict__ out_off, const RowCta& cta,
                                            unsigned char* smem_raw, TcCtx& tc) {
   typedef typename Types<R>::C C;
-  constexpr int EPT = RowEPT<L, R>::value;
   typedef FFTPlan<L, EPT> P;
   constexpr int T = P::kT;
   constexpr int NK = C2R ? L + 1 : L;
@@ -483,8 +481,8 @@ __device__ __forceinline__ void inv_T_body(const LineIO& io, const typename Type
   for (int m = 0; m < EPT; ++m) row[t + T * m] = v[m];
 }
 
-template <typename R, int L, bool C2R, int TC = 0, bool LOC = false>
-__global__ void __launch_bounds__(RowThreads<R, L>::value, sizeof(R) == 8 ? 1 : 2) k_inv_T(LineIO io, const typename Types<R>::W* __restrict__ tw,
+template <typename R, int L, bool C2R, int TC = 0, bool LOC = false, int EPT = RowEPT<L, R>::value>
+__global__ void __launch_bounds__(RowThreads<R, L, EPT>::value, sizeof(R) == 8 ? 1 : 2) k_inv_T(LineIO io, const typename Types<R>::W* __restrict__ tw,
                                                int64_t in_sa0, int64_t in_sk, int64_t out_sa0,
                                                int64_t out_sb, int log_tb, const int64_t* __restrict__ out_off) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -495,7 +493,7 @@ __global__ void __launch_bounds__(RowThreads<R, L>::value, sizeof(R) == 8 ? 1 : 
     tc_setup(tc, smem_raw, io.gmat, 0u, io.err, TC == 2, 0u, io.tc_ctl, kRn, kRn / 128 * TcGeom<16>::kAPiece);
   const RowCta cta{(int)blockIdx.x, (int)blockIdx.y, (int)blockIdx.z, (int)threadIdx.x, (int)threadIdx.y, log_tb,
                    (int64_t)gridDim.x << log_tb};
-  inv_T_body<R, L, C2R, TC, false, LOC>(io, tw, in_sa0, in_sk, out_sa0, out_sb, out_off, cta, smem_raw, tc);
+  inv_T_body<R, L, C2R, TC, false, LOC, EPT>(io, tw, in_sa0, in_sk, out_sa0, out_sb, out_off, cta, smem_raw, tc);
   if constexpr (TC) tc_teardown(tc);
 }
 

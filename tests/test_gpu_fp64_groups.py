@@ -18,6 +18,7 @@ CASES = [
     ((16, 4096), "tm", "J"), ((2048, 32), "te", "none"),
     ((64, 256), "2d6", "rho"),  # 129 blocks: the six components whole
     ((128, 64, 128), "3d6", "none"),  # radix-8 stages in the last axis
+    ((64, 128, 256), "3d6", "none"), ((16, 256, 512), "3d6", "none"),  # rows of 128 and 256 points by 16 elements
 ]
 
 
