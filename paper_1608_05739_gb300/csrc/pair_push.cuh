@@ -34,6 +34,7 @@
 
 #include "fft_line.cuh"
 #include "psatd_kernels.cuh"
+#include "push_modes.h"
 
 namespace psatd {
 
@@ -133,7 +134,7 @@ __device__ __forceinline__ void push_units(unsigned char* base, int us, int g1, 
   }
 }
 
-// The push of this thread's modes l = t + T (grp + G i) (as push_line_modes).
+// The push of this thread's modes l = t + T (grp + G i), by push_mode_pairs.
 template <typename R, int L, int LAYOUT, int EPT, bool STAG, bool PSTD>
 __device__ __forceinline__ void push_line_units(unsigned char* base, int us, int g1, int g2, int gx,
                                                 const PushArgs<R>& a, const Coef<R>* trow, int t, int grp,
@@ -141,59 +142,45 @@ __device__ __forceinline__ void push_line_units(unsigned char* base, int us, int
                                                 typename Types<R>::W phy) {
   typedef FFTPlan<L, EPT> P;
   constexpr int T = P::kT;
-  auto coef = [&](int l) -> Coef<R> {
-    if constexpr (!PSTD) return trow[(l <= L / 2) ? l : L - l];  // |m| along the line axis
+  auto coef = [&](int m) -> Coef<R> {
+    if constexpr (!PSTD) return trow[coef_entry(t + T * m, L)];
     else return Coef<R>{};
   };
-  // two modes per iteration: both loads issued together, the next two before this update
-  Coef<R> qn[2] = {coef(t + T * grp), coef(t + T * (grp + G < EPT ? grp + G : grp))};
-#pragma unroll 1
-  for (int m0 = grp; m0 < EPT; m0 += 2 * G) {
-    const Coef<R> q[2] = {qn[0], qn[1]};
-    const int mn = m0 + 2 * G;
-    if (mn < EPT) {
-      qn[0] = coef(t + T * mn);
-      qn[1] = coef(t + T * (mn + G < EPT ? mn + G : mn));
-    }
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const int m = m0 + G * h;
-      if (m >= EPT) break;
-      const int l = t + T * m;
-      CoefReg<R> f;
-      f.C_h = q[h].C_h; f.C_l = q[h].C_l; f.S_h = q[h].S_h; f.S_l = q[h].S_l;
-      f.A1 = q[h].A1; f.A4 = q[h].A4; f.B1 = q[h].B1; f.B2 = q[h].B2;
-      const int p1 = own_pos<L, EPT, 2 * (int)sizeof(R)>(t, m, sizeof(R) == 8 ? gx : 0);
-      const int p2 = sizeof(R) == 8 ? 0 : own_pos<L, EPT, 16>(t, m, gx);
-      R mx, my, mz;
-      if constexpr (STAG) {
-        const int ml = l < L / 2 ? l : l - L;
-        R kl;
-        typename Types<R>::W pl;
-        stag_axis(a, a.ndim == 2 ? 1 : 2, ml, kl, pl);
-        typename Types<R>::W Ph[3];
-        Ph[0] = phx;
-        if (a.ndim == 2) {
-          mx = kpx; my = kl; mz = R(0);
-          Ph[1] = pl;
-          Ph[2] = phy;
-        } else {
-          mx = kpx; my = kpy; mz = kl;
-          Ph[1] = phy;
-          Ph[2] = pl;
-        }
-        push_units<R, LAYOUT, PSTD>(base, us, g1, g2, p1, p2, f, mx, my, mz, a, Ph);
+  push_mode_pairs<EPT>(grp, G, coef, [&](int m, const Coef<R>& q) {
+    const int l = t + T * m;
+    CoefReg<R> f;
+    f.C_h = q.C_h; f.C_l = q.C_l; f.S_h = q.S_h; f.S_l = q.S_l;
+    f.A1 = q.A1; f.A4 = q.A4; f.B1 = q.B1; f.B2 = q.B2;
+    const int p1 = own_pos<L, EPT, 2 * (int)sizeof(R)>(t, m, sizeof(R) == 8 ? gx : 0);
+    const int p2 = sizeof(R) == 8 ? 0 : own_pos<L, EPT, 16>(t, m, gx);
+    R mx, my, mz;
+    if constexpr (STAG) {
+      const int ml = l < L / 2 ? l : l - L;
+      R kl;
+      typename Types<R>::W pl;
+      stag_axis(a, a.ndim == 2 ? 1 : 2, ml, kl, pl);
+      typename Types<R>::W Ph[3];
+      Ph[0] = phx;
+      if (a.ndim == 2) {
+        mx = kpx; my = kl; mz = R(0);
+        Ph[1] = pl;
+        Ph[2] = phy;
       } else {
-        const int ml = (l == L / 2) ? 0 : (l < L / 2 ? l : l - L);
-        if (a.ndim == 2) {
-          mx = a.rx * R(mxi); my = a.ry * R(ml); mz = R(0);
-        } else {
-          mx = a.rx * R(mxi); my = a.ry * R(myi); mz = a.rz * R(ml);
-        }
-        push_units<R, LAYOUT, PSTD>(base, us, g1, g2, p1, p2, f, mx, my, mz, a, nullptr);
+        mx = kpx; my = kpy; mz = kl;
+        Ph[1] = phy;
+        Ph[2] = pl;
       }
+      push_units<R, LAYOUT, PSTD>(base, us, g1, g2, p1, p2, f, mx, my, mz, a, Ph);
+    } else {
+      const int ml = (l == L / 2) ? 0 : (l < L / 2 ? l : l - L);
+      if (a.ndim == 2) {
+        mx = a.rx * R(mxi); my = a.ry * R(ml); mz = R(0);
+      } else {
+        mx = a.rx * R(mxi); my = a.ry * R(myi); mz = a.rz * R(ml);
+      }
+      push_units<R, LAYOUT, PSTD>(base, us, g1, g2, p1, p2, f, mx, my, mz, a, nullptr);
     }
-  }
+  });
 }
 
 // Slot of component c of the TE (MAP 1) or TM (MAP 2) set of the six-component layout
@@ -280,7 +267,7 @@ __device__ __forceinline__ bool line_pair_body(const PushArgs<R>& a_in, const ty
 #pragma unroll
   for (int m = grp; m < EPT; m += G) {
     const int l = t + T * m;
-    asm volatile("prefetch.global.L2 [%0];" ::"l"(trow + ((l <= L / 2) ? l : L - l)));
+    asm volatile("prefetch.global.L2 [%0];" ::"l"(trow + coef_entry(l, L)));
   }
   // bounded wait; on expiry the error word is set and one more bounded wait lets
   // copies still in flight land before the buffers are used
