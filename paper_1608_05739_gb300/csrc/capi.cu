@@ -1638,6 +1638,7 @@ struct psatd_batch_s {
   void* d_xi = nullptr;
   void* d_push = nullptr;    // PushArgs<float> per class
   void* d_tws = nullptr;     // fused-axis twiddle table per class
+  std::vector<void*> own_tw; // tables of classes whose plan runs another radix schedule
   BatchItem* d_items = nullptr;
   unsigned* d_ctr = nullptr;  // two counters per queue
   struct Queue {
@@ -1658,6 +1659,8 @@ void batch_release(psatd_batch b) {
   void* bufs[] = {b->d_xf, b->d_xi, b->d_push, b->d_tws, b->d_items, b->d_ctr};
   for (void* q : bufs)
     if (q) cudaFree(q);
+  for (void* q : b->own_tw) cudaFree(q);
+  b->own_tw.clear();
   b->d_xf = b->d_xi = b->d_push = b->d_tws = nullptr;
   b->d_items = nullptr;
   b->d_ctr = nullptr;
@@ -1741,10 +1744,32 @@ psatd_status persist_setup(psatd_batch b) {
   const bool tc = b->cls[0]->tc;
   std::vector<PushArgs<float>> pa(ncls);
   std::vector<const void*> tws(ncls);
+  cudaError_t e;
+  auto dalloc = [&](void** ptr, size_t bytes) -> bool {
+    e = cudaMalloc(ptr, bytes);
+    if (e != cudaSuccess) {
+      *ptr = nullptr;
+      cudaGetLastError();
+      return false;
+    }
+    return true;
+  };
   for (int i = 0; i < ncls; ++i) {
     psatd_plan p = b->cls[i];
     pa[i] = make_push_args<float>(p, p->spec1, (int)p->ny, p->nxh * p->npatch);
     tws[i] = p->tw[1];
+    // the persistent kernel's radix schedule goes by the length alone; an autotuned plan may run
+    // another one, whose table has other entries
+    const int ept = push_ept((int)p->ny, p->tc, true);
+    if (p->push_ept != ept) {
+      void* t = nullptr;
+      if (!dalloc(&t, (size_t)p->ny * sizeof(Types<float>::W)))
+        return fail(nullptr, PSATD_ERR_OOM, "batch persistent tables: %s", cudaGetErrorString(e));
+      b->own_tw.push_back(t);
+      e = launch_twiddles(t, (int)p->ny, ept, false, true, b->st);
+      if (e != cudaSuccess) return cuda_fail(nullptr, e, "twiddle table launch");
+      tws[i] = t;
+    }
   }
   // work items, one queue per (pass, family), classes largest first
   std::vector<int> order(ncls);
@@ -1779,16 +1804,6 @@ psatd_status persist_setup(psatd_batch b) {
       q.n = (int)(items.size() - q.first);
       if (q.n) b->queues.push_back(q);
     }
-  cudaError_t e;
-  auto dalloc = [&](void** ptr, size_t bytes) -> bool {
-    e = cudaMalloc(ptr, bytes);
-    if (e != cudaSuccess) {
-      *ptr = nullptr;
-      cudaGetLastError();
-      return false;
-    }
-    return true;
-  };
   if (!dalloc(&b->d_xf, ncls * sizeof(XClassArgs)) || !dalloc(&b->d_xi, ncls * sizeof(XClassArgs)) ||
       !dalloc(&b->d_push, ncls * sizeof(PushArgs<float>)) || !dalloc(&b->d_tws, ncls * sizeof(void*)) ||
       !dalloc(reinterpret_cast<void**>(&b->d_items), items.size() * sizeof(BatchItem)) ||

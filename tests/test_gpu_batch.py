@@ -206,3 +206,32 @@ def test_serialised_classes_give_the_forked_bits():
         out.append(F[:3])
     for x, y in zip(*out):
         assert torch.equal(x, y)
+
+
+def test_persistent_passes_of_autotuned_classes():
+    """Classes for which the autotuner picked another radix schedule of the fused pass than the
+    built-in one (the persistent kernel's, by length alone): the persistent passes give the bits
+    of the batch with the built-in shapes."""
+    import torch
+    ensure_lib()
+    sizes = []
+    for n in [(nx, ny) for ny in (1024, 512, 256, 128, 64) for nx in (64, 128, 256, 512, 1024)]:
+        p = capi.Plan(n, (1.0, 1.0), 0.5, layout="te", prec="fp32", src="J", autotune=True)  # the batch recalls it
+        if p.get_launch()[5] != (16 if n[1] >= 1024 else 8):
+            sizes.append(n)
+        p.destroy()
+    assert sizes, "the autotuner picks the other schedule for some of the sizes"
+    tot = sum(a * b for a, b in sizes)
+    g = torch.Generator(device="cuda").manual_seed(41)
+    init = [torch.randn(tot, device="cuda", generator=g) for _ in range(5)]
+    out = []
+    for autotune, persistent in ((False, False), (True, True)):
+        F = [t.clone() for t in init]
+        b = capi.Batch(sizes, (1.0, 1.0), 0.5, layout="te", prec="fp32", src="J", autotune=autotune)
+        b.set_persistent(persistent)
+        b.step([F[0], F[1], None], [None, None, F[2]], [F[3], F[4], None], nsteps=2)
+        b.sync()
+        b.destroy()
+        out.append(F[:3])
+    for x, y in zip(*out):
+        assert torch.equal(x, y)
