@@ -357,11 +357,11 @@ __device__ __forceinline__ bool line_pair_body(const PushArgs<R>& a_in, const ty
 }
 
 // Grid (line blocks, sets: 2 for the six 2D components), block (T, lines per CTA,
-// component groups); up to 512 threads (128 registers), or 256
-// without groups (GRP false).  Groups are whole warps: with several, T times the lines
-// per CTA is a multiple of 32.
+// component groups); up to 512 threads (128 registers), or without groups (GRP false) 256,
+// or one line's threads where these are more (4096 points by 8 elements).  FP32 groups are
+// whole warps: with several, T times the lines per CTA is a multiple of 32.
 template <typename R, int L, int LAYOUT, int EPT, bool GRP>
-__global__ void __launch_bounds__(GRP || EPT == 4 ? 512 : 256)
+__global__ void __launch_bounds__(GRP || EPT == 4 || FFTPlan<L, EPT>::kT > 256 ? 512 : 256)
 k_line_pair(PushArgs<R> a, const typename Types<R>::W* __restrict__ tw) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ __align__(8) uint64_t stage_mbar;

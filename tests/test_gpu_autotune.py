@@ -149,3 +149,33 @@ def test_autotuned_batch_matches_oracle():
         assert rel_l2_fields(Eg, Bg, mask_layout(Eo, "te", "E"), mask_layout(Bo, "te", "B")) < TOL["fp32"]
         off += n
     b.destroy()
+
+
+def test_lines_of_4096_points():
+    """The longest lines: 512 threads with radix-8 stages, 256 with radix-16, both accepted by
+    set_launch and timed by the autotuner, also through the flag and for a batch class."""
+    import torch
+    ensure_lib()
+    n, shape, d, dt = (16, 4096), (4096, 16), (1.0, 1.0), 0.5
+    E, B, J = _inputs(shape, "te", 91, "fp32")
+    Eo, Bo = orc.psatd_step(E, B, J, d=d, dt=dt, form="J")
+    Eo, Bo = mask_layout(Eo, "te", "E"), mask_layout(Bo, "te", "B")
+    plan = capi.Plan(n, d, dt, layout="te", prec="fp32", src="J")
+    step = lambda: psatd_gpu(shape, d, dt, E, B, J, layout="te", prec="fp32", src="J", plan=plan)
+    for ept in (8, 16):
+        plan.set_launch([-1, -1, -1, -1, 1, ept])
+        Eg, Bg = step()
+        assert rel_l2_fields(Eg, Bg, Eo, Bo) < TOL["fp32"], ept
+    rep = plan.autotune(2)
+    assert "radix8 tb=1" in rep and "radix16 tb=1" in rep
+    Eg, Bg = step()
+    assert rel_l2_fields(Eg, Bg, Eo, Bo) < TOL["fp32"]
+    plan.destroy()
+    capi.Plan(n, d, dt, layout="tm", prec="fp32", src="none", autotune=True).destroy()
+    b = capi.Batch([n, n], d, dt, layout="te", prec="fp32", src="J", autotune=True)
+    F = [torch.from_numpy(np.stack([a, a])).float().cuda().ravel() for a in (E[0], E[1], B[2], J[0], J[1])]
+    b.step([F[0], F[1], None], [None, None, F[2]], [F[3], F[4], None])
+    b.sync()
+    b.destroy()
+    for q in F[0].double().cpu().numpy().reshape(2, *shape):
+        assert np.linalg.norm(q - Eo[0]) < TOL["fp32"] * np.linalg.norm(Eo[0])
