@@ -258,7 +258,9 @@ psatd_status psatd_plan_get_launch(psatd_plan plan, int32_t cfg[6]);
  * runs the same arithmetic).  set: INVALID_ARG when the shape is not valid
  * for the plan's current lines per CTA and elements per thread (a later
  * psatd_plan_set_launch that makes it invalid falls back to 1).  get: the G
- * the next step uses.                                                     */
+ * the next step uses, as far as set takes it: where the built-in choice runs
+ * groups that set does not (3 or 6 in FP64, several short lines in groups), the
+ * largest count below that it does.                                       */
 psatd_status psatd_plan_set_push_groups(psatd_plan plan, int32_t groups);
 psatd_status psatd_plan_get_push_groups(psatd_plan plan, int32_t* groups);
 

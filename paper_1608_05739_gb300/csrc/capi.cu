@@ -462,6 +462,13 @@ int push_groups(psatd_plan p) {
   return push_groups_ok(L, p->push_ept, tb, p->cfg_push_groups, p->tc, p->f32) ? p->cfg_push_groups : 1;
 }
 
+// Whether a caller may choose G groups for the plan's current lines per CTA and elements per thread.
+bool push_groups_settable(psatd_plan p, int G) {
+  const int L = push_line_len(p), tb = push_tb(p);
+  const size_t smem = (p->tc ? (size_t)kTcTail : 0) + push_smem(p->n_in, L, tb, G, p->f32 ? 8 : 16, p->tc);
+  return push_groups_ok(L, p->push_ept, tb, G, p->tc, p->f32) && (p->maxsm <= 0 || smem <= (size_t)p->maxsm);
+}
+
 // Event pair around one launch on the plan's stream.  While the stream is being
 // captured into a graph (multi-step batch calls) the events are captured as
 // external event-record nodes, so that every replay records them again (a plain
@@ -1213,24 +1220,21 @@ psatd_status psatd_plan_set_push_groups(psatd_plan p, int32_t groups) {
     p->cfg_push_groups = -1;
     return PSATD_OK;
   }
-  const int Ll = push_line_len(p);
   const int tb = push_tb(p);
-  int maxsm = 0;
-  cudaDeviceGetAttribute(&maxsm, cudaDevAttrMaxSharedMemoryPerBlockOptin, p->device);
-  const size_t csz = p->f32 ? 8 : 16;
-  const size_t smem = (p->tc ? (size_t)kTcTail : 0) + push_smem(p->n_in, Ll, tb, groups, csz, p->tc);
-  if (!push_groups_ok(Ll, p->push_ept, tb, groups, p->tc, p->f32) || (maxsm > 0 && smem > (size_t)maxsm))
+  if (!push_groups_settable(p, groups))
     return fail(p, PSATD_ERR_INVALID_ARG,
                 "fused pass: %d component groups not valid with %d-point lines, %d elements per thread, "
                 "%d lines per CTA and this precision",
-                groups, Ll, p->push_ept, tb);
+                groups, push_line_len(p), p->push_ept, tb);
   p->cfg_push_groups = groups;
   return PSATD_OK;
 }
 
 psatd_status psatd_plan_get_push_groups(psatd_plan p, int32_t* groups) {
   if (!p || !groups) return fail(p, PSATD_ERR_INVALID_ARG, "plan or groups is NULL");
-  *groups = push_groups(p);
+  int G = push_groups(p);
+  while (G > 1 && !push_groups_settable(p, G)) --G;
+  *groups = G;
   return PSATD_OK;
 }
 

@@ -215,3 +215,27 @@ def test_tensor_core_pairs_in_a_batch():
         b.destroy()
     for a, c in zip(res[0], res[1]):
         assert np.array_equal(a, c)
+
+
+@pytest.mark.parametrize("prec,n,layout,src", [
+    ("fp64", (64, 256), "te", "J"),      # built in: three groups
+    ("fp64", (32, 32, 32), "3d6", "J"),  # six
+    ("fp32", (64, 128), "te", "J"),      # two lines of 16 threads in groups
+    ("fp32", (64, 384), "te", "J"),      # four groups of 12 elements per thread
+    ("fp32", (128, 2048), "te", "J"), ("mixed_bf16", (128, 512), "te", "J"),
+])
+def test_a_read_shape_can_be_set_again(prec, n, layout, src):
+    """What get_push_groups and get_launch return, set_push_groups and set_launch accept, and
+    the step's bits stay."""
+    ensure_lib()
+    shape, d, dt = tuple(reversed(n)), (1.0,) * len(n), 0.4
+    E, B, J, _, _ = _inputs(shape, layout, 23)
+    plan = capi.Plan(n, d, dt, layout=layout, prec=prec, src=src)
+    ref = psatd_gpu(shape, d, dt, E, B, J, layout=layout, prec=prec, src=src, plan=plan)
+    G = plan.get_push_groups()
+    plan.set_push_groups(G)
+    plan.set_launch(plan.get_launch())
+    assert plan.get_push_groups() == G
+    got = psatd_gpu(shape, d, dt, E, B, J, layout=layout, prec=prec, src=src, plan=plan)
+    assert np.array_equal(got[0], ref[0]) and np.array_equal(got[1], ref[1])
+    plan.destroy()
