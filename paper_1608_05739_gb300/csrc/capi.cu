@@ -816,9 +816,10 @@ psatd_status regen_push_twiddles(psatd_plan p) {
 
 // Valid launch shapes of every knob: rows[k] = log2(lines per CTA) of
 // transposing pass k (empty if the pass does not exist), push = (elements per
-// thread, lines per CTA, component groups) of the fused pass.
+// thread, lines per CTA, component groups) of the fused pass; groups -1: the built-in
+// choice, where callers may not set its count; run: the count the launch runs.
 struct PushShape {
-  int ept, tb, groups;
+  int ept, tb, groups, run;
 };
 struct TuneSpace {
   std::vector<int> rows[4];
@@ -860,11 +861,17 @@ TuneSpace tune_space(psatd_plan p) {
     for (int tb = 1; tb * T <= (T > 256 ? T : 256); tb *= 2) {
       if (p->tc && (tb * T) % 128 != 0) continue;
       if (tb > 1 && tb / 2 >= nlines) break;
+      const int kept = push_kernel_ept(ts.Ll, ept, p->f32, p->ndim == 3 ? p->nxh * p->ny : p->nxh);
+      const int builtin = push_groups_default(p->layout, ts.Ll, kept, tb, p->n_in, nlines, p->tc, p->f32, p->sm_bytes);
+      bool any = false, found = false;
       for (int G : {1, 2, 4}) {
         if (!push_groups_ok(ts.Ll, ept, tb, G, p->tc, p->f32)) continue;
         if (maxsm > 0 && tail + push_smem(p->n_in, ts.Ll, tb, G, csz, p->tc) > (size_t)maxsm) continue;
-        ts.push.push_back({ept, tb, G});
+        ts.push.push_back({ept, tb, G, G});
+        any = true;
+        found = found || G == builtin;
       }
+      if (any && !found) ts.push.push_back({ept, tb, -1, builtin});
     }
   }
   return ts;
@@ -996,7 +1003,7 @@ psatd_status autotune(psatd_plan p, int reps, std::string* report) {
     std::snprintf(buf, sizeof buf, "push L=%d:", Ll);
     *report += buf;
     for (size_t i = 0; i < push.size(); ++i) {
-      std::snprintf(buf, sizeof buf, " radix%d tb=%d g=%d %.4fms%s", push[i].ept, push[i].tb, push[i].groups,
+      std::snprintf(buf, sizeof buf, " radix%d tb=%d g=%d %.4fms%s", push[i].ept, push[i].tb, push[i].run,
                     tpush[i], i == b ? "*" : "");
       *report += buf;
     }

@@ -137,6 +137,21 @@ def test_autotuner_considers_groups():
     plan.destroy()
 
 
+@pytest.mark.parametrize("prec,n,g", [("fp32", (64, 384), 4), ("fp32", (64, 128), 4), ("fp64", (64, 256), 3)])
+def test_autotuner_times_the_built_in_groups(prec, n, g):
+    """The built-in count of a small launch is a candidate where a caller may not set it."""
+    ensure_lib()
+    shape, d, dt = tuple(reversed(n)), (1.0, 1.0), 0.5
+    E, B, J, _, _ = _inputs(shape, "te", 29)
+    plan = capi.Plan(n, d, dt, layout="te", prec=prec, src="J")
+    assert " g=%d " % g in plan.autotune(2)
+    Eg, Bg = psatd_gpu(shape, d, dt, E, B, J, layout="te", prec=prec, src="J", plan=plan)
+    Eo, Bo = _oracle(shape, d, dt, E, B, J, None, None, "te", "J", {})
+    assert rel_l2_fields(Eg, Bg, Eo, Bo) < (1e-12 if prec == "fp64" else 2e-6)
+    plan.set_push_groups(plan.get_push_groups())
+    plan.destroy()
+
+
 def test_batch_groups_give_the_same_bits():
     """A batch of power-of-two, 3 * 2^k and 5 * 2^k patches: each class takes the
     groups where its shape admits them; every class's fields are unchanged."""
