@@ -1703,7 +1703,9 @@ bool persist_y_len(int L, bool tc) {
 int fam_of(int L) { return pow2(L) ? 0 : 1; }
 // rows per item of a transposing pass and lines per item of the fused pass
 int persist_x_tb(int L) { return kPersistXThreads / (L / row_ept(L, true)); }
-int persist_y_tb(int L, bool tc) { return kPersistThreads / (L / push_ept(L, tc, true)); }
+int persist_y_tb(int L, bool tc) {
+  return kPersistThreads / (L / push_ept(L, tc, true) * (tc ? 1 : persist_y_groups(L)));
+}
 
 // X-pass arguments of class plan p for the step's field / source pointers (as
 // run_step's first and last passes in 2D).

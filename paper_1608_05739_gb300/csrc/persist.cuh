@@ -78,6 +78,10 @@ __device__ __forceinline__ void copy_to_shared(T* dst, const T* src) {
   if constexpr (FAM == 0) { CASE(64) CASE(128) CASE(256) CASE(512) CASE(1024) } \
   else { CASE(48) CASE(96) CASE(192) CASE(384) CASE(768) }
 
+// Component groups of the FP32 fused pass's lines: two for 1024 points (16 elements per
+// thread), so that an item is as many values as the other lengths' (8 per thread).
+__host__ __device__ constexpr int persist_y_groups(int L) { return push_ept(L, false, true) == 16 ? 2 : 1; }
+
 template <int L>
 struct PersistRows {
   static constexpr int T = L / RowEPT<L>::value;
@@ -165,10 +169,11 @@ __global__ void __launch_bounds__(kPersistThreads, TC ? 2 : 4) k_persist_push(co
     if constexpr (TC) {                                                                                    \
       line_push_body<R, LL, LAYOUT, TC, EPT>(A, tw, it.blk, t, g, kPersistThreads / T, 0, 1, smem_raw, tc, sc); \
     } else {                                                                                               \
+      constexpr int G = persist_y_groups(LL), TB = kPersistThreads / (T * G);                              \
       auto part = [&](auto lay, auto map) {                                                                \
         __syncthreads(); /* the previous part's shared memory is free */                                   \
-        if (line_pair_body<R, LL, decltype(lay)::value, EPT, false, decltype(map)::value>(                 \
-                A, tw, it.blk, t, g, kPersistThreads / T, 0, 1, smem_raw, sc.mbar, sc.phase))              \
+        if (line_pair_body<R, LL, decltype(lay)::value, EPT, (G > 1), decltype(map)::value>(               \
+                A, tw, it.blk, t, g % TB, TB, g / TB, G, smem_raw, sc.mbar, sc.phase))                     \
           sc.phase ^= 1u;                                                                                  \
       };                                                                                                   \
       if constexpr (LAYOUT == 1) {                                                                         \
@@ -196,9 +201,14 @@ constexpr size_t persist_x_smem() {
   return (TC ? kTcTail : 0) + (size_t)kPersistXThreads * (FAM ? 24 : 16) * sizeof(typename Types<R>::C) +
          (TC == 2 ? (kPersistXThreads / 128) * TcGeom<16>::kAPiece : 0);
 }
+// FP32 items hold the transform units alone (the six 2D components: the larger set's), 8 or
+// 12 values per thread.  With an exchange buffer beside them and 16 values per thread for
+// every length, two CTAs were resident per SM instead of four: 512 patches of 2^k sides, TE
+// 1.52 -> 1.23 ms a step, six components 4.73 -> 2.70 (2^k and 3 * 2^k: 1.25 -> 1.07, 4.29 -> 2.47).
 template <typename R, int TC, int FAM>
-constexpr size_t persist_push_smem(int n_in) {
-  return (TC ? kTcTail : 0) + (size_t)(n_in + 1) * kPersistThreads * (FAM ? 12 : 16) * sizeof(typename Types<R>::C);
+constexpr size_t persist_push_smem(int layout, int n_in) {
+  const int slots = TC ? n_in + 1 : layout == 1 ? (n_in == 6 ? 3 : n_in == 9 ? 5 : 7) : n_in;
+  return (TC ? kTcTail : 0) + (size_t)slots * kPersistThreads * (TC ? 16 : FAM ? 12 : 8) * sizeof(typename Types<R>::C);
 }
 
 }  // namespace psatd

@@ -33,7 +33,7 @@ cudaError_t launch_persist_x(bool fwd, int grid, cudaStream_t st, const XClassAr
 template <typename R, int TC, int FAM>
 cudaError_t launch_persist_push(int layout, int n_in, int grid, cudaStream_t st, const PushArgs<R>* cls,
                                 const void* const* tws, const PersistQueue& q, int* occ) {
-  const size_t smem = persist_push_smem<R, TC, FAM>(n_in);
+  const size_t smem = persist_push_smem<R, TC, FAM>(layout, n_in);
   void (*kern)(const PushArgs<R>*, const void* const*, PersistQueue) = nullptr;
   switch (layout) {
     case 1: kern = k_persist_push<R, TC, FAM, 1>; break;

@@ -208,6 +208,33 @@ def test_serialised_classes_give_the_forked_bits():
         assert torch.equal(x, y)
 
 
+@pytest.mark.parametrize("layout,src", [("2d6", "none"), ("2d6", "rho"), ("te", "none"), ("te", "rho"), ("tm", "none")])
+def test_persistent_fused_pass_of_every_slot_count(layout, src):
+    """The persistent fused pass's shared memory is the transform units of its item alone: every
+    source form, lines of 1024 points (two component groups), 768 and a part-filled item."""
+    import torch
+    ensure_lib()
+    sizes = [(64, 1024), (96, 768), (128, 64), (64, 512)]
+    tot = sum(a * b for a, b in sizes)
+    g = torch.Generator(device="cuda").manual_seed(51)
+    pe, pb, pj = capi.PRESENT[layout]
+    mk = lambda p: [torch.randn(tot, device="cuda", generator=g) if p[i] else None for i in range(3)]
+    E0, B0, J = mk(pe), mk(pb), mk(pj)
+    rho = [torch.randn(tot, device="cuda", generator=g) for _ in range(2)] if src == "rho" else [None, None]
+    out = []
+    for persistent in (True, False):
+        E, B = ([t.clone() if t is not None else None for t in F] for F in (E0, B0))
+        b = capi.Batch(sizes, (1.0, 1.0), 0.5, layout=layout, prec="fp32", src=src)
+        b.set_persistent(persistent)
+        b.step(E, B, J if src != "none" else None, *rho, nsteps=2)
+        b.sync()
+        b.destroy()
+        out.append(E + B)
+    for x, y in zip(*out):
+        if x is not None:
+            assert torch.equal(x, y)
+
+
 def test_persistent_passes_of_autotuned_classes():
     """Classes for which the autotuner picked another radix schedule of the fused pass than the
     built-in one (the persistent kernel's, by length alone): the persistent passes give the bits
