@@ -78,6 +78,18 @@ __device__ __forceinline__ void copy_to_shared(T* dst, const T* src) {
   if constexpr (FAM == 0) { CASE(64) CASE(128) CASE(256) CASE(512) CASE(1024) } \
   else { CASE(48) CASE(96) CASE(192) CASE(384) CASE(768) }
 
+// Elements per thread of the transposing passes' lengths, the most of a family.
+template <int FAM> constexpr int kPersistXEpt = FAM ? 12 : 16;
+template <int FAM>
+constexpr bool persist_x_fits() {
+  bool ok = true;
+#define PSATD_X_EPT(LL) ok = ok && row_ept(LL, true) <= kPersistXEpt<FAM>;
+  PSATD_PERSIST_X_LENGTHS(FAM, PSATD_X_EPT)
+#undef PSATD_X_EPT
+  return ok;
+}
+static_assert(persist_x_fits<0>() && persist_x_fits<1>(), "shared memory of the persistent rows");
+
 // Component groups of the FP32 fused pass's lines: two for 1024 points (16 elements per
 // thread), so that an item is as many values as the other lengths' (8 per thread).
 __host__ __device__ constexpr int persist_y_groups(int L) { return push_ept(L, false, true) == 16 ? 2 : 1; }
@@ -91,13 +103,15 @@ struct PersistRows {
 
 // Transposing x pass (forward R2C or inverse C2R) over every class of the queue.
 // Register caps of the persistent passes (CTAs that must stay resident together),
-// as their standalone kernels: the SIMT transposing passes 64 registers (128 for
-// the 3 * 2^k lengths, 24 elements per thread), the tensor-core ones 128 (at 64
-// their 16-element rows and split pieces went to the stack); the SIMT fused pass
-// 128, the tensor-core one up to 255 (two CTAs per SM, as its shared memory allows
-// anyway; with every line length in one kernel it spilled at 128).
+// as their standalone kernels: the SIMT transposing passes 64 registers (12 or 16
+// elements per thread; 512 patches, rows of both families, forward 0.80 -> 0.71 ms and
+// inverse 0.59 -> 0.49 against 128 registers and 24 values per thread reserved for the
+// 3 * 2^k lengths), the tensor-core ones 128 (at 64 their 16-element rows and split
+// pieces went to the stack); the SIMT fused pass 128, the tensor-core one up to 255 (two
+// CTAs per SM, as its shared memory allows anyway; with every line length in one kernel
+// it spilled at 128).
 template <typename R, int TC, int FAM, bool FWD>
-__global__ void __launch_bounds__(kPersistXThreads, (FAM || TC) ? 2 : 4) k_persist_x(const XClassArgs* __restrict__ cls, PersistQueue q) {
+__global__ void __launch_bounds__(kPersistXThreads, TC ? 2 : 4) k_persist_x(const XClassArgs* __restrict__ cls, PersistQueue q) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ int slot;
   __shared__ __align__(16) XClassArgs A;
@@ -198,7 +212,7 @@ __global__ void __launch_bounds__(kPersistThreads, TC ? 2 : 4) k_persist_push(co
 template <typename R, int TC, int FAM>
 constexpr size_t persist_x_smem() {
   // TB lines of L values, plus split-BF16's third A piece (one per 128 threads)
-  return (TC ? kTcTail : 0) + (size_t)kPersistXThreads * (FAM ? 24 : 16) * sizeof(typename Types<R>::C) +
+  return (TC ? kTcTail : 0) + (size_t)kPersistXThreads * kPersistXEpt<FAM> * sizeof(typename Types<R>::C) +
          (TC == 2 ? (kPersistXThreads / 128) * TcGeom<16>::kAPiece : 0);
 }
 // FP32 items hold the transform units alone (the six 2D components: the larger set's), 8 or
