@@ -407,8 +407,9 @@ psatd_status psatd_batch_destroy(psatd_batch batch);
  * global: layout 2D6, TE or TM; precision, source form, cell sizes, dt, c and
  * eps0 as in psatd_plan_create; n[0], n[1] need not be powers of two, but the
  * extended sizes ix + 2 guard and iy + 2 guard must satisfy psatd_plan_create's
- * limits.  Owns a plan of the extended size (px*py patches); the patches' cells
- * are read from and written to the global arrays, never stored.
+ * limits.  Owns a plan of the extended size (px*py patches) and an array of the
+ * global size per source; the patches' cells are read from and written to the
+ * global arrays, never stored.
  * Errors: INVALID_ARG (NULL, px/py not dividing the grid, guard < 0),
  * UNSUPPORTED (3D, extended sizes out of range), OOM, CUDA.                 */
 typedef struct psatd_local_s* psatd_local;

@@ -49,3 +49,27 @@ def test_global_rows(prec, inner, patches, guard, order):
     assert rel_l2_fields(Eg, Bg, mask_layout(Eo, layout, "E"), mask_layout(Bo, layout, "B")) < tol
     a, b = run(3, 1), run(1, 3)
     assert np.array_equal(a[0], b[0]) and np.array_equal(a[1], b[1])
+
+
+@pytest.mark.parametrize("pinned", [False, True])
+def test_sources_are_held_over_the_call(pinned):
+    """Three steps of one call with J in a field's own array, on the device or pinned on the host,
+    equal three steps with J in an array of its own: sources are those of the call's start."""
+    import torch
+    ensure_lib()
+    shape, d, dt = (96, 96), (1.0, 0.9), 0.4
+    F = [synth.random_fields(shape, 1, s)[0] for s in (95, 96, 97)]
+
+    def run(alias):
+        t = [torch.from_numpy(a).float() for a in F]
+        t = [a.pin_memory() if pinned else a.cuda() for a in t]
+        own = t[0].clone()
+        J0 = t[0] if alias else own.pin_memory() if pinned else own
+        loc = capi.Local((96, 96), d, dt, px=2, py=2, guard=8, layout="te", prec="fp32", src="J")
+        loc.step([t[0], t[1], None], [None, None, t[2]], [J0, torch.zeros_like(t[1], device="cuda"), None], nsteps=3)
+        loc.sync()
+        loc.destroy()
+        return [a.cpu().numpy() for a in t]
+
+    for a, b in zip(run(True), run(False)):
+        assert np.array_equal(a, b)
