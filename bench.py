@@ -591,7 +591,7 @@ def run_batch_line(args, world, rank, local):
 
 def te2048_side(capi, torch, args, dev, world, hbm, peak_kind):
     """Side key of the headline line: the single 2048^2 TE grid in FP32 (the
-    fused pass k_line_push at its largest), with its own roofline."""
+    fused pass at its largest), with its own roofline."""
     dx = 1.0 / LAM_CELLS
     dt = dx / math.sqrt(2.0)
     stream = torch.cuda.current_stream()

@@ -181,9 +181,9 @@ int32_t psatd_abi_version(void);
  * Supported sizes: every n[i] a power of two, 16 <= n[0] <= 4096,
  * 8 <= n[1], n[2] <= 4096; with PSATD_FP32 also the mixed-radix lengths
  * n[0] = 6 * 2^k in [96, 3072] (x rows of n[0]/2 = 3 * 2^(k-1) points) and
- * n[1], n[2] = 3 * 2^k in [48, 3072] (radix-3 first stage), and
- * n[0] = 10 * 2^k in [160, 2560], n[1], n[2] = 5 * 2^k in [80, 1280] (radix-5
- * first stage), on any axis and combined freely with powers of two;
+ * n[1], n[2] = 3 * 2^k in [48, 3072], and
+ * n[0] = 10 * 2^k in [160, 2560], n[1], n[2] = 5 * 2^k in [80, 1280], on any
+ * axis and combined freely with powers of two;
  * PSATD_FP64, PSATD_FP32,
  * PSATD_MIXED_FP16 or _BF16; flags from PSATD_FLAG_*.  A last axis of n
  * points needs (n_in + 1) * n * 8 (FP32) or 16 (FP64) bytes of shared memory
@@ -360,7 +360,8 @@ psatd_status psatd_batch_sync(psatd_batch batch);
  * returns to one launch per pass and size class on the branch streams described
  * above, which keeps a class's spectra in L2 between its passes and measured
  * faster; UNSUPPORTED when the sizes do not allow the persistent passes.  The
- * results are the same bits either way.  psatd_batch_launches_per_step: kernel launches of
+ * results are the same bits either way (for classes whose radix schedule is the
+ * built-in one; the autotuner may choose another).  psatd_batch_launches_per_step: kernel launches of
  * one step in the current mode (without PSATD_FLAG_CHECKED's scans).  The
  * first step after the field or source pointers change uploads the classes'
  * argument tables (a synchronising copy, outside any graph capture). */
@@ -376,7 +377,7 @@ psatd_status psatd_batch_set_branches(psatd_batch batch, int32_t forked);
 /* Component groups of every size class's fused pass (psatd_plan_set_push_groups):
  * each class takes `groups` (2 or 4) where its shape admits them and one group
  * otherwise; 1 everywhere; -1 the built-in choice.  The per-class launches use
- * it (the persistent passes keep one group).  Synchronises the batch's streams;
+ * it (the persistent passes do not).  Synchronises the batch's streams;
  * the same bits either way.  INVALID_ARG for other values. */
 psatd_status psatd_batch_set_push_groups(psatd_batch batch, int32_t groups);
 

@@ -107,7 +107,7 @@ psatd_status cuda_fail(psatd_plan p, cudaError_t e, const char* what) {
 }
 
 bool pow2(int64_t v) { return v > 0 && (v & (v - 1)) == 0; }
-// 3 * 2^k with k >= 4: the mixed-radix lengths of the FP32 passes (radix-3 first stage)
+// 3 * 2^k with k >= 4: the mixed-radix lengths of the FP32 passes (first stage radix 3, 6 or 12)
 bool three_pow2(int64_t v) { return v >= 48 && v % 3 == 0 && pow2(v / 3); }
 // 5 * 2^k with k >= 4: the radix-5 lengths of the FP32 passes
 bool five_pow2(int64_t v) { return v >= 80 && v % 5 == 0 && pow2(v / 5); }

@@ -17,8 +17,8 @@
 // of a call the second half step of B and the first of the next use the same E:
 // one pass subtracts the half step twice (the same two roundings), 2 N + 1 passes
 // for N steps instead of 3 N.  Against one cell per thread and 3 N passes: CKC TE 2048^2
-// with J, 8 steps 700 -> 156 us; Yee 256^3 with J, one step 549 -> 309 us (2.0 GB moved,
-// 6.5 TB/s).
+// with J, 8 steps 705 -> 161 us; Yee 256^3 with J, one step 549 -> 303 us (2.0 GB moved,
+// 6.6 TB/s).
 #include <cuda_runtime.h>
 #include <stdint.h>
 

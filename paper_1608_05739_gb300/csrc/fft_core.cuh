@@ -85,7 +85,6 @@ __device__ __forceinline__ C2 mkc(F2 a, F2 b) { return C2{a, b}; }
 
 template <class C> __device__ __forceinline__ C cadd(C a, C b) { return mkc(a.x + b.x, a.y + b.y); }
 template <class C> __device__ __forceinline__ C csub(C a, C b) { return mkc(a.x - b.x, a.y - b.y); }
-template <class C> __device__ __forceinline__ C cmul_mi(C a) { return mkc(a.y, -a.x); }  // * (-i)
 template <class C> __device__ __forceinline__ C cmul_pi(C a) { return mkc(-a.y, a.x); }  // * (+i)
 template <class C> __device__ __forceinline__ C cconj(C a) { return mkc(a.x, -a.y); }
 // a +- i b (the rotation costs no operation, also in the packed type)

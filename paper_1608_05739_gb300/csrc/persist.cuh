@@ -70,7 +70,8 @@ __device__ __forceinline__ void copy_to_shared(T* dst, const T* src) {
 
 // Lengths of the persistent passes: FAM 0 powers of two, FAM 1 the 3 * 2^k
 // lengths (FP32).  Transposing passes: x lines of L = nx/2 points; fused pass:
-// last-axis lines.  Lines of T = L/EPT threads, kPersistThreads / T of them per item.
+// last-axis lines.  Lines of T = L/EPT threads (times persist_y_groups), as many per item
+// as fill the CTA.
 #define PSATD_PERSIST_X_LENGTHS(FAM, CASE) \
   if constexpr (FAM == 0) { CASE(32) CASE(64) CASE(128) CASE(256) CASE(512) } \
   else { CASE(48) CASE(96) CASE(192) CASE(384) }

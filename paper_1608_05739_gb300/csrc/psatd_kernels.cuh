@@ -8,7 +8,7 @@
 //   1  k_fwd_T<R2C>  x-rows of every input array -> R2C -> half spectrum,
 //                    written with the row index b contiguous (tile transpose)
 //   2  k_fwd_T<C2C>  (3D) y-lines -> C2C, written z-contiguous
-//   3  k_line_push   the last axis: forward FFT of every input component,
+//   3  k_line_push   (k_line_pair) the last axis: forward FFT of every input component,
 //                    the analytic PSATD push per mode (Sec. III.B), inverse FFT
 //                    of the E and B components, in place
 //   4  k_inv_T<C2C>  (3D) inverse y-lines, read z-contiguous
@@ -315,9 +315,10 @@ __device__ __forceinline__ void fwd_T_body(const LineIO& io, const typename Type
   }
 }
 
-// Launch bounds: two CTAs of the largest block per SM (at most 64 registers a
-// thread).  The tensor-core variants then keep part of each row on the stack,
-// but measured faster so than with 128 registers and half the resident warps.
+// Launch bounds: FP64 one CTA of the largest block per SM (64 registers a thread with 4
+// elements, 255 with 16), else two (64 registers).  The tensor-core variants then keep
+// part of each row on the stack, but measured faster so than with 128 registers and half
+// the resident warps.
 template <typename R, int L, bool R2C, int TC = 0, bool LOC = false, int EPT = RowEPT<L, R>::value>
 __global__ void __launch_bounds__(RowThreads<R, L, EPT>::value, sizeof(R) == 8 ? 1 : 2) k_fwd_T(LineIO io, const typename Types<R>::W* __restrict__ tw,
                                                int64_t in_sa0, int64_t in_sb, int64_t out_sa0,
@@ -912,34 +913,24 @@ __device__ __forceinline__ void push_line_modes(typename Types<R>::C* st, int ss
   }
 }
 
-// Fused last-axis pass: for TB lines (kx in 2D, (kx, ky) in 3D), forward FFT
-// of every input slot, per-mode push, inverse FFT of the n_out field slots,
-// written back in place.  Shared memory, component-major: slot c of the TB
-// lines (TB x L values, line g at offset g L), c < n_in, then one extra
-// exchange buffer per line (contiguous, so that in the tensor-core variant TC
-// they hold the A tiles of the CTA's 128-row groups); a slot doubles as the
-// other exchange buffer of its own transforms, and in split-BF16 the TB lines'
-// slot c of the component being transformed holds the third A piece (no line
-// keeps live data there at a tensor-core stage boundary), so the pass needs no
-// further region.  After its forward FFT a slot holds the spectrum at positions
-// sw<kLastCX>(t + T m), so the push and the inverse FFT's first exchange only
-// touch each thread's own positions.
-// EPT: elements per thread, 8 (radix-8 stages) or 16 (radix-16 stages; the
-// only choice of the tensor-core variant).
-// Component groups (G > 1, T a multiple of 32, no tensor-core stages): each
-// line has G x T threads; group grp transforms the input components c = grp,
-// grp + G, ... and the output components c = G - 1 - grp, 2G - 1 - grp, ...
-// (the groups with an extra forward transform get one fewer inverse one), with
-// its own second exchange buffer per line and its own named barrier (id
-// 1 + g G + grp over its T threads), so that the groups run side by side; the
-// whole CTA meets at a block barrier before and after the push, in which the
-// groups split each thread position's modes.  G = 1 is the plain pass (block
-// barriers throughout, as the tensor-core stages need).
-// Body of one CTA of the fused pass: line block bx (lines bx tb .. bx tb + tb - 1,
-// line g of the block handled by the threads g T .. g T + T - 1 of each
-// component group, t their position).
-// GRP: the component-group variant (a kernel of its own, so that the plain pass
-// compiles with G = 1 as a constant).
+// Fused last-axis pass of the tensor-core variants (pair_push.cuh: the others): for TB
+// lines (kx in 2D, (kx, ky) in 3D), forward FFT of every input slot, per-mode push,
+// inverse FFT of the n_out field slots, written back in place.  Shared memory,
+// component-major: slot c of the TB lines (TB x L values, line g at offset g L), c < n_in,
+// then one extra exchange buffer per line (contiguous, so that they hold the A tiles of
+// the CTA's 128-row groups); a slot doubles as the other exchange buffer of its own
+// transforms, and in split-BF16 the TB lines' slot c of the component being transformed
+// holds the third A piece (no line keeps live data there at a tensor-core stage
+// boundary), so the pass needs no further region.  After its forward FFT a slot holds the
+// spectrum at positions sw<kLastCX>(t + T m), so the push and the inverse FFT's first
+// exchange only touch each thread's own positions.  16 elements per thread (radix-16
+// stages).
+// Component groups (GRP, a kernel of its own; G = 2): the CTA's lines are 128 threads, one
+// unit, per group; group grp transforms the input components c = grp, grp + 2, ... and the
+// output components c = 1 - grp, 3 - grp, ..., each exchanging in its own slot; the CTA
+// meets at a block barrier before and after the push, whose modes the groups split.
+// Body of one CTA: line block bx (lines bx tb .. bx tb + tb - 1, line g of the block
+// handled by the threads g T .. g T + T - 1 of each component group, t their position).
 template <typename R, int L, int LAYOUT, int TC, int EPT, bool GRP = false>
 __device__ __forceinline__ void line_push_body(const PushArgs<R>& a_in, const typename Types<R>::W* __restrict__ tw,
                                                int bx, int t, int g, int tb, int grp, int G, unsigned char* smem_raw,
@@ -1105,8 +1096,8 @@ __device__ __forceinline__ void line_push_body(const PushArgs<R>& a_in, const ty
   }
 }
 
-// Block (T, lines per CTA, component groups); the group variant (GRP) takes up
-// to 512 threads (the tensor-core pairs 256), the plain pass 256 (or T).
+// Block (T, lines per CTA, component groups), up to 256 threads: two units of 128 with
+// component groups (GRP), else one or two.
 template <typename R, int L, int LAYOUT, int TC, int EPT, bool GRP>
 __global__ void __launch_bounds__(256, GRP ? 2 : 1)
 k_line_push(PushArgs<R> a, const typename Types<R>::W* __restrict__ tw) {

@@ -1,5 +1,5 @@
 // push3_f32_tetm.cu -- float instantiation of the fused last-axis FFT + PSATD push
-// pass for the mixed lengths 3 * 2^k (radix-3 first stage, 24 elements per thread).
+// pass for the mixed lengths 3 * 2^k (radix-12 first stage, 12 elements per thread).
 #include "launch_impl.cuh"
 
 namespace psatd {

@@ -1,5 +1,5 @@
 // push5_f32_six.cu -- float instantiation of the fused last-axis FFT + PSATD push
-// pass for the mixed lengths 5 * 2^k (radix-5 first stage, 20 elements per thread).
+// pass for the mixed lengths 5 * 2^k (radix-10 or -20 first stage, 20 elements per thread).
 #include "launch_impl.cuh"
 
 namespace psatd {

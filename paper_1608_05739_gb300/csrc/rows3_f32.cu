@@ -1,5 +1,5 @@
 // rows3_f32.cu -- float instantiation of the transposing line-FFT passes for the
-// mixed lengths 3 * 2^k (radix-3 first stage, 24 elements per thread).
+// mixed lengths 3 * 2^k (radix-3, -6 or -12 first stage, 12 or 24 elements per thread).
 #include "launch_impl.cuh"
 
 namespace psatd {

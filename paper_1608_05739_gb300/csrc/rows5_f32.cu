@@ -1,5 +1,5 @@
 // rows5_f32.cu -- float instantiation of the transposing line-FFT passes for the
-// mixed lengths 5 * 2^k (radix-5 first stage, 20 elements per thread).
+// mixed lengths 5 * 2^k (radix-10 or -20 first stage, 20 elements per thread).
 #include "launch_impl.cuh"
 
 namespace psatd {

@@ -133,8 +133,8 @@ PERSIST_SIZES = {
 @pytest.mark.parametrize("prec,layout", [("fp32", "te"), ("fp32", "tm"), ("fp32", "2d6"), ("mixed_fp16", "te"),
                                          ("mixed_bf16", "te"), ("mixed_bf16", "2d6")])
 def test_persistent_passes_equal_per_class_launches(prec, layout):
-    """One persistent launch per pass type and length family over every patch (the
-    default where the sizes allow) gives the bits of the per-class launches, in a
+    """One persistent launch per pass type and length family over every patch (on
+    request, where the sizes allow) gives the bits of the per-class launches, in a
     graph replay of several steps, and matches the oracle on a patch of each family."""
     import torch
     ensure_lib()

@@ -1,8 +1,8 @@
 """GPU parity of the mixed-radix line lengths L = 3 * 2^k and 5 * 2^k (FP32):
 every pass (R2C x rows of nx/2 points, C2C y lines in 3D, the fused last-axis
-pass, the inverses) transforms such lines with a radix-3 first stage, then
-radix-2/4 and radix-8 stages, or a radix-5 first stage, then radix-2 and
-radix-4 stages.  The method does not restrict the grid to powers of two; these
+pass, the inverses) transforms such lines with a radix-3, -6 or -12 first stage,
+then radix-8 or radix-2 and radix-4 stages, or a radix-10 or -20 first stage,
+then radix-4 stages.  The method does not restrict the grid to powers of two; these
 lengths matter for the local FFTs of Sec. II.A.3, whose extended patches are
 an interior plus two guard regions (e.g. 16 + 2 * 16 = 48 cells).
 

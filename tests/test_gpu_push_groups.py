@@ -2,9 +2,9 @@
 
 With G > 1 each line's input components are forward-transformed, and its
 output components inverse-transformed, by G thread groups in turn, which meet
-only for the per-mode push (tensor-core plans: two groups in lockstep, one
-128-row MMA group each, sharing every tensor-core round).  Every transform and every mode's update runs the
-same arithmetic in the same order as with one group, so the fields must be
+only for the per-mode push (tensor-core plans: two groups, a 128-row MMA group with
+tensor-core rounds of its own each).  Every transform and every mode's update runs the same
+arithmetic in the same order as with one group, so the fields must be
 bitwise identical for every valid G; one G > 1 case per shape is also checked
 against the FP64 oracle.  Shapes: 2D TE (lines of 256 and 2048 points), 2D
 six-component, 3D rho-form (eleven input components), TM vacuum, 3 * 2^k and
@@ -178,9 +178,9 @@ def test_batch_groups_give_the_same_bits():
         capi.Batch(sizes, (1.0, 1.0), 0.5, layout="te", prec="fp32", src="J").set_push_groups(3)
 
 
-# tensor-core pairs: (array shape, layout, source form); odd and even component counts
+# two tensor-core groups: (array shape, layout, source form); odd and even component counts
 TC_CASES = [
-    ((512, 128), "te", "J"),       # 5 inputs, 3 outputs: the last pair of each has one component
+    ((512, 128), "te", "J"),       # 5 inputs, 3 outputs: one group has a component more
     ((64, 128), "2d6", "rho"),     # 11 inputs, 6 outputs
     ((1024, 128), "tm", "none"),   # 3 inputs, 3 outputs
     ((128, 256), "te", "J"),       # 128-point lines: 8 threads a line, 16 lines per group
