@@ -202,7 +202,7 @@ __device__ __forceinline__ void tc_unit_sync(int rn) {
 // (128, or 256 for lines of 4096 points), each a round of its own (unit barriers, one
 // issuing thread, its own mbarrier): the units of a CTA never wait for each other, so
 // one splits its operands while another's MMAs run.  Bound: the latency of a round
-// (operand stores, barrier, MMAs, TMEM read) at 16 warps per SM, not the tensor pipe (1 %).
+// (operand stores, barrier, MMAs, TMEM read) at 16 warps per SM, not the tensor pipe (7 %).
 // CTA-wide rounds and scalar splits -> units and packed splits: 256^3 J-form split FP16
 // 2573 -> 2079 us a step, 512-patch split BF16 22.3 -> 20.1 ms per four steps.  The
 // A tiles alias exchange space of the unit that holds no live data at a stage boundary.
