@@ -1022,13 +1022,17 @@ def run_te2048_line(args, world, rank, local):
         dist.destroy_process_group()
 
 
-def timed_steps(step, steps, warmup, flush, stream):
+def timed_steps(step, steps, warmup, flush, stream, plan=None):
     """Run ``warmup`` untimed steps, then ``steps`` steps each preceded by an L2
-    flush and bracketed by CUDA events on ``stream``; returns total ms and clocks."""
+    flush and bracketed by CUDA events on ``stream``; returns total ms and clocks.
+    ``plan``: its per-launch timing is switched on after the warm-up (whose first
+    launches load the kernels)."""
     import torch
     for n in range(warmup):
         step(n)
     torch.cuda.synchronize()
+    if plan is not None:
+        plan.set_timing(True)
     starts = [torch.cuda.Event(enable_timing=True) for _ in range(steps)]
     ends = [torch.cuda.Event(enable_timing=True) for _ in range(steps)]
     clocks = ClockSampler(torch.cuda.current_device())
@@ -1068,8 +1072,7 @@ def run_side_workload(args):
         B = [torch.zeros(n, n, n, device=dev) for _ in range(3)]
         J = [J[i].contiguous() for i in range(3)]
         plan = capi.Plan((n, n, n), (d, d, d), dt, layout="3d6", prec="fp32", src="rho", stream=stream)
-        plan.set_timing(True)
-        ms, clk = timed_steps(lambda i: plan.step(E, B, J, r0, r1), args.steps, args.warmup, flush, stream)
+        ms, clk = timed_steps(lambda i: plan.step(E, B, J, r0, r1), args.steps, args.warmup, flush, stream, plan)
         kt = plan.kernel_times()
         alg = algorithmic_bytes(n, n, n, 11, 6)
         cells = n ** 3
@@ -1102,8 +1105,7 @@ def run_side_workload(args):
             E = [E0[i].clone() for i in range(3)]
             B = [B0[i].clone() for i in range(3)]
             plan = capi.Plan((512, 512, 1024), d, dt, layout="3d6", prec=prec, src="rho", stream=stream)
-            plan.set_timing(True)
-            ms, c_ = timed_steps(lambda i: plan.step(E, B, J, r0, r1), args.steps, args.warmup, flush, stream)
+            ms, c_ = timed_steps(lambda i: plan.step(E, B, J, r0, r1), args.steps, args.warmup, flush, stream, plan)
             kt = plan.kernel_times()
             plan.sync()
             plan.destroy()
